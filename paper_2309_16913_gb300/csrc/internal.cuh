@@ -325,7 +325,7 @@ struct SelIO {
     const int64_t *off_leaf;  // DESC: offsets of the leaf hits
     const int64_t *off_rng;   // DESC: offsets of the whole-subtree ranges
     int32_t *leaf_out;        // DESC: leaf hits
-    int2 *rng_out;            // DESC: (lo, hi) ranges of the tree's id array
+    int2 *rng_out;            // DESC: {first entry of the tree's id array, place among the query's run ids}
     // Work-queue mapping only: per-query write cursors (zeroed before the
     // pass), because several warps may emit results for one query.
     int32_t *cur_ids;         // SCATTER
@@ -369,9 +369,11 @@ struct SelectBuffers {
 rtree_status select_enqueue(const rtree *t, const float4 *queries, int64_t q, int mapping,
                             const SelectBuffers &b, cudaStream_t s);
 
-// Where the ids of segment i come from: leaf[off_leaf[i] .. off_leaf[i+1])
-// followed by tree_ids[lo .. hi) for every (lo, hi) in
-// rng[off_rng[i] .. off_rng[i+1]).  rng may be null (no ranges).
+// Where the ids of segment i come from: leaf[off_leaf[i] .. off_leaf[i+1]),
+// and runs of tree_ids: range r of rng[off_rng[i] .. off_rng[i+1]) starts at
+// tree_ids[rng[r].x] and fills places rng[r].y .. rng[r+1].y among the
+// segment's run ids (the last one: up to the segment's length less its leaf
+// hits).  rng may be null (no ranges).
 struct SortSources {
     const int32_t *leaf;
     const int64_t *off_leaf;  // segment i's leaf hits start at off_leaf[i] and end at

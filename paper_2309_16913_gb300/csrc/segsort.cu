@@ -7,16 +7,15 @@
 //   2..256 ids    one warp: gather into shared memory, then a bitonic network
 //                 on 1-8 keys per lane in registers (shuffles across lanes,
 //                 swaps inside a lane);
-//   257..16384    one CTA of 64-512 threads (32 keys each), entirely in
-//                 shared memory:
-//                 bucket the keys by value within their range (at most 8192
-//                 buckets: a few keys each for spread-out ids) with shared
-//                 atomics, then each thread sorts whole buckets in registers
-//                 with a bitonic network; a crowded bucket sends the segment
-//                 to a stable LSD radix sort (8-bit digits);
-//   16385..40960  the same with one CTA of 1024 threads, 40 keys each (160 KB
-//                 of shared memory; a crowded one goes on to the next path);
-//   > 40960       gathered into place, partitioned by its top differing bits
+//   257..32768  one CTA of 64-1024 threads (32 ids each), entirely in shared
+//                 memory: asynchronous copies in, buckets by value (one id
+//                 each on average) counted with byte counters, and every id's
+//                 rank among its bucket's neighbours gives its place in the
+//                 output (cta_bucket_sort); ids in bands are bucketed again
+//                 through equalized buckets, and what overflows those too
+//                 (heavily repeated ids) goes to a stable LSD radix sort
+//                 (8-bit digits), or above 16384 ids to the next path;
+//   > 32768       gathered into place, partitioned by its top differing bits
 //                 into buckets of about 8K ids (MSD step through a scratch
 //                 area), each bucket then sorted like a mid-size segment.
 // Each class runs as a persistent grid whose CTAs claim segments from an
@@ -36,19 +35,17 @@ namespace {
 constexpr int kBins = 256;
 constexpr int kItems = 16;              // keys per thread of the LSD fallback (1024 threads)
 constexpr int kCtaMax = 1024 * kItems;  // 16384: longest segment the LSD fallback takes
-constexpr int kItemsMid = 32;           // keys per thread of the CTA sorts up to kCtaMax
-constexpr int kItemsBig = 40;           // keys per thread of the CTA sort above kCtaMax
-constexpr int kCtaBigMax = 1024 * kItemsBig;
 constexpr uint32_t kSign = 0x80000000u;
-constexpr int kBucketBitsMax = 13;      // at most 8192 buckets
-constexpr int kBucketDensity = 1;       // 2^(ceil(log2 n) - 1) buckets of the key range
-constexpr int kBucketCrowded = 32;      // a longer bucket sends the segment to LSD
+
+// The ids a CTA sort takes: 252 per warp and eight ids a lane (see the
+// transposition in cta_bucket_sort).
+constexpr int cta_ids(int threads, int items) { return threads / 32 * (items / 8) * 252; }
+constexpr int kMidMax = cta_ids(512, 32);  // longest segment below the largest class: 16128
 
 // Segment classes (index into the class lists).
 enum {
     C_W1 = 0, C_W2, C_W4, C_W8,       // warp sorts, 32*K ids
-    C_CTA2K, C_CTA4K, C_CTA8K, C_CTA16K,  // CTA sorts of 64..512 threads, kItemsMid ids each
-    C_CTA40K,                             // CTA sort of 1024 threads, kItemsBig ids each
+    C_CTA1K, C_CTA2K, C_CTA4K, C_CTA8K, C_CTA16K, C_CTA32K,  // CTA sorts
     C_LARGE,                          // MSD partition first
     C_COUNT
 };
@@ -68,11 +65,12 @@ __device__ __forceinline__ int class_of(int64_t n)
     if (n <= 64) return C_W2;
     if (n <= 128) return C_W4;
     if (n <= 256) return C_W8;
-    if (n <= 2048) return C_CTA2K;
-    if (n <= 4096) return C_CTA4K;
-    if (n <= 8192) return C_CTA8K;
-    if (n <= kCtaMax) return C_CTA16K;
-    if (n <= kCtaBigMax) return C_CTA40K;
+    if (n <= cta_ids(64, 16)) return C_CTA1K;
+    if (n <= cta_ids(128, 16)) return C_CTA2K;
+    if (n <= cta_ids(256, 16)) return C_CTA4K;
+    if (n <= cta_ids(512, 16)) return C_CTA8K;
+    if (n <= kMidMax) return C_CTA16K;
+    if (n <= cta_ids(1024, 32)) return C_CTA32K;
     return C_LARGE;
 }
 
@@ -130,41 +128,34 @@ __global__ void k_classify(const int64_t *__restrict__ off, int64_t nseg, int32_
 }
 
 // ------------------------------------------------------------- gathering
-// One warp copies segment i's ids into sm[0 .. n) (in source order).
+// One warp copies segment i's n ids into sm[0 .. n) (in source order).
 __device__ __forceinline__ void warp_gather(int32_t *__restrict__ sm, const SortSources &S,
-                                            int64_t i, int lane)
+                                            int64_t i, int n, int lane)
 {
     const int64_t l0 = S.off_leaf[i], l1 = leaf_end(S, i);
     for (int64_t e = l0 + lane; e < l1; e += 32)
         sm[e - l0] = S.leaf[e];
-    int pos = (int)(l1 - l0);
     if (S.rng) {
         const int64_t r0 = S.off_rng[i], r1 = S.off_rng[i + 1];
+        const int nl = (int)(l1 - l0);
         for (int64_t rb = r0; rb < r1; rb += 32) {
-            // lanes hold up to 32 ranges; an inclusive scan of their lengths
-            // gives each range's place, then the warp copies them in turn
+            // lanes hold up to 32 ranges, which the warp copies in turn; a
+            // range ends where the next one starts
             const int64_t r = rb + lane;
-            int2 rg = make_int2(0, 0);
+            int2 rg = make_int2(0, n - nl);
             if (r < r1)
                 rg = S.rng[r];
-            const int len = rg.y - rg.x;
-            int inc = len;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int u = __shfl_up_sync(RT_FULL, inc, o);
-                if (lane >= o)
-                    inc += u;
-            }
-            const int start = pos + inc - len;
+            int after = n - nl;  // the start of the range behind this chunk
+            if (rb + 32 < r1)
+                after = S.rng[rb + 32].y;
             const int cnt = (int)(r1 - rb < 32 ? r1 - rb : 32);
             for (int k = 0; k < cnt; ++k) {
                 const int lo = __shfl_sync(RT_FULL, rg.x, k);
-                const int ln = __shfl_sync(RT_FULL, len, k);
-                const int st = __shfl_sync(RT_FULL, start, k);
-                for (int e = lane; e < ln; e += 32)
-                    sm[st + e] = __ldg(S.tree_ids + lo + e);
+                const int st = __shfl_sync(RT_FULL, rg.y, k);
+                const int en = k + 1 < 32 ? __shfl_sync(RT_FULL, rg.y, k + 1) : after;
+                for (int e = lane; e < en - st; e += 32)
+                    sm[nl + st + e] = __ldg(S.tree_ids + lo + e);
             }
-            pos += __shfl_sync(RT_FULL, inc, 31);
         }
     }
     __syncwarp();
@@ -197,7 +188,7 @@ __global__ void __launch_bounds__(256) k_sort_warp(const int32_t *__restrict__ l
         const int32_t seg = list[wi];
         const int64_t o = off[seg];
         const int n = (int)(off[seg + 1] - o);
-        warp_gather(sm, S, seg, lane);
+        warp_gather(sm, S, seg, n, lane);
         int v[K];
 #pragma unroll
         for (int k = 0; k < K; ++k) {
@@ -243,41 +234,45 @@ __global__ void __launch_bounds__(256) k_sort_warp(const int32_t *__restrict__ l
 }
 
 // ------------------------------------------------------------ CTA sort
-constexpr int log2_floor(int v) { return v > 1 ? 1 + log2_floor(v / 2) : 0; }
+constexpr int kHalo = 32;          // slots kept before and after the keys (a window is at most 31)
+constexpr int kNet = 5;            // ids a bucket may hold for the register network
+constexpr int kCoarse = 4;         // coarse bins per thread of the equalized buckets
+constexpr int kRetry = 12;         // a bucket this full asks for equalized buckets
+constexpr int kLongRange = 512;    // longer id runs are copied by the whole CTA
 
-template <int THREADS, int ITEMS = kItems>
-struct CtaSmem {
-    static constexpr int W = THREADS / 32;
-    // at most 2^(ceil(log2 n) - 1) <= n/2 buckets are used (and at most 2^13)
-    static constexpr int kCntBits = log2_floor(THREADS * ITEMS / 2) < kBucketBitsMax
-                                        ? log2_floor(THREADS * ITEMS / 2) : kBucketBitsMax;
-    uint32_t buf[THREADS * ITEMS];
-    union {
-        uint32_t cnt[1 << kCntBits];  // bucket sort: per-bucket counts, then ends
-        struct {                            // LSD ranks
-            uint32_t wcnt[W][kBins];
-            uint32_t dcount[kBins];
-            uint32_t dstart[kBins];
-        };
-        struct {                            // gathering: one chunk of ranges
-            int32_t rlo[THREADS];
-            int32_t rstart[THREADS];
-            int32_t rlen[THREADS];
-        };
-    };
-    uint32_t wsum[W];
-    uint32_t red0[W], red1[W];  // per-warp partial reductions
-    uint32_t crowded;
-    long long claim;  // the list entry this CTA takes next
+// A segment to sort: n ids of which nl are leaf hits, nr whole subtrees.
+struct Piece {
+    int64_t dst;  // where its ids go in the output
+    int64_t src;  // its leaf hits in S.leaf (or its ids in the scratch area)
+    int64_t rng;  // its ranges in S.rng
+    int32_t n;    // < 0: nothing left
+    int32_t nl;
+    int32_t nr;
+    int32_t seg;  // list entry: the segment
 };
 
-// Exclusive block scan of one int per thread (uses sm.wsum); returns the
-// prefix and writes the block total to *total.
+// Shared memory of one CTA sort: 4 bytes of key and 1 byte of bucket counter
+// per id.
 template <int THREADS, int ITEMS>
-__device__ __forceinline__ int block_scan_int(CtaSmem<THREADS, ITEMS> &sm, int v, int *total)
+struct CtaSmem {
+    static constexpr int N = cta_ids(THREADS, ITEMS);
+    static_assert(ITEMS % 16 == 0 && THREADS % 32 == 0, "a thread's counter words are read 16 bytes at a time");
+    uint32_t slots[THREADS * ITEMS + 192];  // kHalo smallest ids, then the ids and their upper halo
+    uint32_t cnt[THREADS * ITEMS / 4];       // four byte counters a word; then the packed bucket starts
+    uint32_t win[THREADS * ITEMS / 32 + 4];       // per 32 positions: largest bucket of more than kNet there, less one
+    uint32_t coarse[kCoarse * THREADS + 2];  // equalized buckets: first bucket of each coarse bin
+    uint32_t red0[32], red1[32];       // per-warp partial results
+    Piece next;                        // the segment this CTA takes next
+    __device__ __forceinline__ uint32_t *buf() { return slots + kHalo; }
+};
+
+// Exclusive block scan of one int per thread (w: one word per warp); returns
+// the prefix and writes the block total to *total.  One barrier: the caller
+// has another before w is written again.
+template <int THREADS>
+__device__ __forceinline__ int block_scan_int(uint32_t *w, int v, int *total)
 {
-    constexpr int W = THREADS / 32;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
     int inc = v;
 #pragma unroll
     for (int o = 1; o < 32; o <<= 1) {
@@ -286,274 +281,422 @@ __device__ __forceinline__ int block_scan_int(CtaSmem<THREADS, ITEMS> &sm, int v
             inc += u;
     }
     if (lane == 31)
-        sm.wsum[w] = (uint32_t)inc;
+        w[wid] = (uint32_t)inc;
     __syncthreads();
-    int before = 0, all = 0;
-    for (int x = 0; x < W; ++x) {
-        const int s = (int)sm.wsum[x];
-        if (x < w)
-            before += s;
-        all += s;
-    }
-    *total = all;
-    __syncthreads();
-    return before + inc - v;
+    const unsigned s = lane < THREADS / 32 ? w[lane] : 0u;
+    *total = (int)__reduce_add_sync(RT_FULL, s);
+    return (int)__reduce_add_sync(RT_FULL, lane < wid ? s : 0u) + inc - v;
 }
 
-// The CTA copies segment i's ids into sm.buf[0 .. n), flipped to keys.  The
-// first chunk of range descriptors is requested before the leaf hits are
-// copied, so both loads are in flight together.
-template <int THREADS, int ITEMS>
-__device__ __forceinline__ void cta_gather(CtaSmem<THREADS, ITEMS> &sm, const SortSources &S, int64_t i)
+// Block-wide minimum and maximum (w0, w1: one word per warp); every thread
+// gets both.  One barrier, as block_scan_int.
+template <int THREADS>
+__device__ __forceinline__ void block_minmax(uint32_t *w0, uint32_t *w1, int &kmin, int &kmax)
 {
-    constexpr int W = THREADS / 32;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    const int64_t l0 = S.off_leaf[i], l1 = leaf_end(S, i);
-    int64_t r0 = 0, r1 = 0;
-    if (S.rng) {
-        r0 = S.off_rng[i];
-        r1 = S.off_rng[i + 1];
-    }
-    int2 rg = make_int2(0, 0);
-    if (r0 + threadIdx.x < r1)
-        rg = S.rng[r0 + threadIdx.x];
-    const int nl = (int)(l1 - l0);
-#pragma unroll 4
-    for (int e = threadIdx.x; e < nl; e += THREADS)
-        sm.buf[e] = (uint32_t)S.leaf[l0 + e] ^ kSign;
-    int pos = nl;
-    for (int64_t rb = r0; rb < r1; rb += THREADS) {
-        if (rb != r0) {
-            rg = make_int2(0, 0);
-            if (rb + threadIdx.x < r1)
-                rg = S.rng[rb + threadIdx.x];
-        }
-        const int len = rg.y - rg.x;
-        int total;
-        const int start = block_scan_int<THREADS>(sm, len, &total);
-        sm.rlo[threadIdx.x] = rg.x;
-        sm.rlen[threadIdx.x] = len;
-        sm.rstart[threadIdx.x] = pos + start;
-        __syncthreads();
-        const int cnt = (int)(r1 - rb < THREADS ? r1 - rb : THREADS);
-        for (int k = w; k < cnt; k += W) {  // warp w copies ranges w, w+W, ...
-            const int lo = sm.rlo[k], ln = sm.rlen[k], st = sm.rstart[k];
-            for (int e = lane; e < ln; e += 32)
-                sm.buf[st + e] = (uint32_t)__ldg(S.tree_ids + lo + e) ^ kSign;
-        }
-        pos += total;
-        __syncthreads();
-    }
-    __syncthreads();
-}
-
-// The CTA copies keys src[0 .. n) (xor flip) into sm.buf.
-template <int THREADS, int ITEMS>
-__device__ __forceinline__ void cta_load(CtaSmem<THREADS, ITEMS> &sm, const uint32_t *__restrict__ src,
-                                         int n, uint32_t flip)
-{
-    for (int p = threadIdx.x; p < n; p += THREADS)
-        sm.buf[p] = src[p] ^ flip;
-    __syncthreads();
-}
-
-// Block-wide AND and OR of the keys' bits; every thread gets AND ^ OR.
-template <int THREADS, int ITEMS>
-__device__ __forceinline__ uint32_t block_diff(CtaSmem<THREADS, ITEMS> &sm, uint32_t a_and, uint32_t a_or)
-{
-    constexpr int W = THREADS / 32;
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
-#pragma unroll
-    for (int d = 16; d > 0; d >>= 1) {
-        a_and &= __shfl_xor_sync(RT_FULL, a_and, d);
-        a_or |= __shfl_xor_sync(RT_FULL, a_or, d);
-    }
-    if (lane == 0) {
-        sm.red0[w] = a_and;
-        sm.red1[w] = a_or;
-    }
-    __syncthreads();
-    a_and = 0xffffffffu;
-    a_or = 0;
-    for (int x = 0; x < W; ++x) {
-        a_and &= sm.red0[x];
-        a_or |= sm.red1[x];
-    }
-    __syncthreads();
-    return a_and ^ a_or;
-}
-
-// Block-wide minimum and maximum of the keys; every thread gets both.
-template <int THREADS, int ITEMS>
-__device__ __forceinline__ void block_minmax(CtaSmem<THREADS, ITEMS> &sm, uint32_t &kmin, uint32_t &kmax)
-{
-    constexpr int W = THREADS / 32;
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const int wid = threadIdx.x >> 5, lane = threadIdx.x & 31;
     kmin = __reduce_min_sync(RT_FULL, kmin);
     kmax = __reduce_max_sync(RT_FULL, kmax);
     if (lane == 0) {
-        sm.red0[w] = kmin;
-        sm.red1[w] = kmax;
+        w0[wid] = (uint32_t)kmin;
+        w1[wid] = (uint32_t)kmax;
     }
     __syncthreads();
-    kmin = 0xffffffffu;
-    kmax = 0;
-    for (int x = 0; x < W; ++x) {
-        kmin = min(kmin, sm.red0[x]);
-        kmax = max(kmax, sm.red1[x]);
-    }
-    __syncthreads();
+    kmin = __reduce_min_sync(RT_FULL, lane < THREADS / 32 ? (int)w0[lane] : INT_MAX);
+    kmax = __reduce_max_sync(RT_FULL, lane < THREADS / 32 ? (int)w1[lane] : INT_MIN);
 }
 
-// Sorts buf[s0 .. s0+c), c <= N, in registers: a bitonic network over N
-// values padded with the largest key (the first c outputs are then exactly
-// the sorted bucket, whatever equal keys it holds).
-template <int N>
-__device__ __forceinline__ void bucket_network(uint32_t *buf, int s0, int c)
+__device__ __forceinline__ void cp_async4(uint32_t *dst, const void *src)
 {
-    uint32_t v[N];
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async16(uint32_t *dst, const void *src)
+{
+    asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src)
+                 : "memory");
+}
+__device__ __forceinline__ void cp_async_wait()
+{
+    asm volatile("cp.async.wait_all;" ::: "memory");
+}
+
+// `lanes` threads (this one is number t) start the copy of src[0 .. n) into
+// shared memory: 16 bytes at a time where both sides are aligned.
+__device__ __forceinline__ void copy_async(uint32_t *dst, const int32_t *src, int n, int t, int lanes)
+{
+    const unsigned both = (unsigned)(uintptr_t)src | (unsigned)__cvta_generic_to_shared(dst);
+    int done = 0;
+    if ((both & 15u) == 0) {
+        done = n & ~3;
+        for (int e = 4 * t; e < done; e += 4 * lanes)
+            cp_async16(dst + e, src + e);
+    }
+    for (int e = done + t; e < n; e += lanes)
+        cp_async4(dst + e, src + e);
+}
+
+// The CTA starts copying piece m's ids into shared memory: the ids of its
+// whole subtrees first, then its leaf hits.  The copies are asynchronous
+// (cp.async), so every range's loads are in flight together: with a register
+// copy each warp waited for one range at a time, which was a third of the
+// sort's time.  Subtree runs of full leaves keep 16-byte alignment on both
+// sides, and so do leaf hits in slots reserved F at a time.
+template <int THREADS, int ITEMS>
+__device__ __forceinline__ void cta_gather(CtaSmem<THREADS, ITEMS> &sm, const SortSources &S, const Piece &m)
+{
+    uint32_t *buf = sm.buf();
+    const int nrl = m.n - m.nl;
+    copy_async(buf + nrl, S.leaf + m.src, m.nl, threadIdx.x, THREADS);
+    // 4 to 32 lanes a range: 16 bytes a lane copy the average one
+    const int lg = nrl > 64 * m.nr ? 5 : nrl > 32 * m.nr ? 4 : nrl > 16 * m.nr ? 3 : 2;
+    const int sub = threadIdx.x & ((1 << lg) - 1);
+    const int2 *rng = S.rng + m.rng;
+    bool some_long = false;
+    for (int k = threadIdx.x >> lg; k < m.nr; k += THREADS >> lg) {
+        const int2 g = rng[k];
+        const int e = k + 1 < m.nr ? rng[k + 1].y : nrl;
+        if (e - g.y > kLongRange)
+            some_long = true;
+        else if (g.y >= 0 && e <= nrl)
+            copy_async(buf + g.y, S.tree_ids + g.x, e - g.y, sub, 1 << lg);
+    }
+    if (__syncthreads_or(some_long)) {  // longer ranges: the whole CTA, one after another
+        for (int b = 0; b < m.nr; b += 32) {
+            const int k = b + (int)(threadIdx.x & 31);
+            int2 g = make_int2(0, 0);
+            int e = 0;
+            if (k < m.nr) {
+                g = rng[k];
+                e = k + 1 < m.nr ? rng[k + 1].y : nrl;
+            }
+            unsigned todo = __ballot_sync(RT_FULL, e - g.y > kLongRange && g.y >= 0 && e <= nrl);
+            while (todo) {
+                const int l = __ffs(todo) - 1;
+                todo &= todo - 1;
+                const int lo = __shfl_sync(RT_FULL, g.x, l), st = __shfl_sync(RT_FULL, g.y, l);
+                const int en = __shfl_sync(RT_FULL, e, l);
+                copy_async(buf + st, S.tree_ids + lo, en - st, threadIdx.x, THREADS);
+            }
+        }
+    }
+}
+
+// Value buckets: id * mult + add as a 64-bit product is (id - smallest id) *
+// mult; its high word is the bucket (one multiply-add an id).
+// Plain: n equal parts of the id range.  Equalized: kCoarse * THREADS equal coarse
+// bins of the range, each cut into as many equal parts as it holds ids (the
+// product's low word is the place within the bin).  Both are monotone.
+struct BucketMap {
+    int mult;
+    int64_t add;
+    const uint32_t *coarse;
+};
+__device__ __forceinline__ uint32_t coarse_of(const BucketMap &m, int id)
+{
+    return (uint32_t)(((int64_t)id * m.mult + m.add) >> 32);
+}
+template <bool EQ>
+__device__ __forceinline__ uint32_t bucket_of(const BucketMap &m, int id)
+{
+    if (!EQ)
+        return coarse_of(m, id);
+    const uint64_t p = (uint64_t)((int64_t)id * m.mult + m.add);
+    const uint32_t c = (uint32_t)(p >> 32);
+    const uint32_t h0 = m.coarse[c];
+    return h0 + __umulhi((uint32_t)p, m.coarse[c + 1] - h0);
+}
+// mult = parts * 2^32 / (range + 1), rounded down past float's rounding error
+// so that the largest id maps below `parts` (and below 2^31: a range shorter
+// than 2 * parts then leaves the upper parts empty).
+__device__ __forceinline__ BucketMap bucket_map(int parts, int kmin, int kmax, const uint32_t *coarse)
+{
+    const float span = (float)((uint32_t)kmax - (uint32_t)kmin);
+    const float m = (float)parts * 4294967296.f / (span + 1.f) * (1.f - 4.76837158e-7f);
+    BucketMap b;
+    b.mult = m < 2147483520.f ? (int)m : 2147483520;
+    b.add = -(int64_t)kmin * b.mult;
+    b.coarse = coarse;
+    return b;
+}
+
+// Calls f(k, p) for each of the thread's keys: key k of the thread is element
+// p = 4*THREADS*(k/4) + 4*threadIdx.x + k%4 of the n.  Whole rounds of
+// 4*THREADS elements need no test per key; only the last one tests (a branch
+// per key was a fifth of the instructions).
+template <int THREADS, int ITEMS, typename F>
+__device__ __forceinline__ void each_key(int n, F f)
+{
+    const int p0 = (int)threadIdx.x * 4;
 #pragma unroll
-    for (int k = 0; k < N; ++k)
-        v[k] = k < c ? buf[s0 + k] : 0xffffffffu;
+    for (int i = 0; i < ITEMS / 4; ++i) {
+        if ((i + 1) * 4 * THREADS <= n) {
 #pragma unroll
-    for (int size = 2; size <= N; size <<= 1) {
+            for (int j = 0; j < 4; ++j)
+                f(4 * i + j, i * 4 * THREADS + p0 + j);
+        } else if (i * 4 * THREADS < n) {
 #pragma unroll
-        for (int stride = size >> 1; stride > 0; stride >>= 1) {
+            for (int j = 0; j < 4; ++j)
+                if (i * 4 * THREADS + p0 + j < n)
+                    f(4 * i + j, i * 4 * THREADS + p0 + j);
+        }
+    }
+}
+
+// Counts the keys into byte counters (each key's arrival number within its
+// bucket stays in `arr`), and turns the counters into bucket starts, packed
+// {start of the word's first bucket: 17 bits; keys before its fourth, third
+// and second bucket: 5 bits each}.  Needs cnt and win zeroed.  False if a
+// field overflowed (the starts are unusable) or, for plain buckets, if one
+// holds kRetry keys or more.
+template <int THREADS, int ITEMS, bool EQ>
+__device__ __forceinline__ bool count_buckets(CtaSmem<THREADS, ITEMS> &sm, const BucketMap &bm,
+                                              const int (&key)[ITEMS], uint32_t (&arr)[ITEMS / 4], int n)
+{
+    constexpr int WORDS = ITEMS / 4;  // counter words of a thread
+    each_key<THREADS, ITEMS>(n, [&](int k, int) {
+        const uint32_t b = bucket_of<EQ>(bm, key[k]);
+        const uint32_t sh = (b << 3) & 31u;
+        const uint32_t old = atomicAdd(&sm.cnt[b >> 2], 1u << sh);
+        const uint32_t a = old >> sh;  // its low byte goes to byte k%4
+        const int j = k & 3;
+        arr[k >> 2] = j == 0 ? a : __byte_perm(arr[k >> 2], a, j == 1 ? 0x3240 : j == 2 ? 0x3410 : 0x4210);
+    });
+    __syncthreads();
+    const int w0 = (int)threadIdx.x * WORDS;
+    const bool mine = w0 < ((n + 3) >> 2);
+    uint32_t w[WORDS], over = 0, top = 0, sum = 0;
+    if (mine) {
 #pragma unroll
-            for (int k = 0; k < N; ++k) {
-                const int m = k ^ stride;
-                if (m > k) {
-                    const bool up = (k & size) == 0;
-                    const uint32_t a = v[k], b = v[m];
-                    v[k] = up ? min(a, b) : max(a, b);
-                    v[m] = up ? max(a, b) : min(a, b);
+        for (int k = 0; k < WORDS; k += 4) {
+            const uint4 a = *reinterpret_cast<const uint4 *>(sm.cnt + w0 + k);
+            w[k] = a.x, w[k + 1] = a.y, w[k + 2] = a.z, w[k + 3] = a.w;
+        }
+#pragma unroll
+        for (int k = 0; k < WORDS; ++k) {
+            over |= w[k] & 0xe0e0e0e0u;
+            top = __vmaxu2(top, __vmaxu2(w[k] & 0x00ff00ffu, (w[k] >> 8) & 0x00ff00ffu));
+            sum = __dp4a(w[k], 0x01010101u, sum);
+        }
+    }
+    // a counter past 255 carries into the next one or out of the word, which
+    // only ever makes the total smaller than n
+    int total;
+    uint32_t run = (uint32_t)block_scan_int<THREADS>(sm.red0, (int)sum, &total);
+    const uint32_t biggest = max(top & 0xffffu, top >> 16);
+    if (mine) {
+        if (biggest > (uint32_t)kNet && total == n)
+            for (uint32_t c = run >> 5; c <= (run + sum - 1) >> 5; ++c)
+                atomicMax(&sm.win[c], biggest - 1);
+#pragma unroll
+        for (int k = 0; k < WORDS; ++k) {
+            const uint32_t pre = w[k] * 0x01010100u;  // byte q: keys before the word's bucket q
+            const uint32_t next = run + (pre >> 24) + (w[k] >> 24);
+            over |= pre & 0xe0e0e000u;
+            w[k] = (run << 15) | ((pre >> 8) & 31u) | ((pre >> 11) & (31u << 5)) | ((pre >> 14) & (31u << 10));
+            run = next;
+        }
+#pragma unroll
+        for (int k = 0; k < WORDS; k += 4)
+            *reinterpret_cast<uint4 *>(sm.cnt + w0 + k) = make_uint4(w[k], w[k + 1], w[k + 2], w[k + 3]);
+    }
+    return __syncthreads_or(over != 0 || total != n || (!EQ && biggest >= (uint32_t)kRetry)) == 0;
+}
+
+// Moves the keys (all of them in registers) to their buckets in sm.buf().
+template <int THREADS, int ITEMS, bool EQ>
+__device__ __forceinline__ void scatter_buckets(CtaSmem<THREADS, ITEMS> &sm, const BucketMap &bm,
+                                                const int (&key)[ITEMS], const uint32_t (&arr)[ITEMS / 4], int n)
+{
+    uint32_t *buf = sm.buf();
+    each_key<THREADS, ITEMS>(n, [&](int k, int) {
+        const uint32_t b = bucket_of<EQ>(bm, key[k]);
+        const uint32_t v = sm.cnt[b >> 2];
+        buf[(v >> 15) + (((v << 5) >> (5 * (b & 3u))) & 31u) + __byte_perm(arr[k >> 2], 0, 0x4440 | (k & 3))] = (uint32_t)key[k];
+    });
+}
+
+template <int THREADS, int ITEMS>
+__device__ __forceinline__ void zero_counters(CtaSmem<THREADS, ITEMS> &sm, int n)
+{
+    uint4 *c = reinterpret_cast<uint4 *>(sm.cnt);
+    const int n4 = ((n + 31) >> 5) * 2;  // whole groups of 8 words (32 buckets)
+    for (int k = threadIdx.x; k < n4; k += THREADS)
+        c[k] = make_uint4(0, 0, 0, 0);
+    for (int k = threadIdx.x; k < (n >> 5) + 4; k += THREADS)
+        sm.win[k] = 0;
+}
+
+// Sorts the n ids in sm.buf() and writes them to dst.
+//
+// The ids are bucketed by value, one bucket per id on average.  After the
+// scatter into bucket order an id is at most (its bucket's size - 1) places
+// from where it belongs, so a few rounds of odd-even transposition finish the
+// sort: kNet rounds in registers sort every bucket of up to kNet ids, and
+// where a larger one lies (win) the write-out counts inversions instead: an
+// id at p belongs at p + (later ids smaller than it) - (earlier ids larger).
+//
+// Bound by shared memory and by instruction issue together (22 wavefronts and
+// 95-115 warp instructions per 32 ids, half of the peak of either; the random
+// atomics, loads and stores of the count and the scatter are ten of the 22).
+// All classes on 1.43G ids (10M rectangles, 1M queries): 7.65 ms, against
+// 10.4 ms with buckets of three to five ids sorted by per-thread bitonic
+// networks, a third of whose instructions were the networks' padding.
+//
+// Ids that fill some buckets with kRetry or more (ids in bands, e.g. rows
+// stored region by region) are bucketed again through equalized buckets.  If
+// those overflow too (heavily repeated ids) the function returns false with
+// the unsorted ids in dst, and the caller sorts them another way.
+// after_count and before_write are called on the way, by all threads (unless
+// the function returns early): the caller's loads for the next piece.
+template <int THREADS, int ITEMS, typename P1, typename P2>
+__device__ __forceinline__ bool cta_bucket_sort(CtaSmem<THREADS, ITEMS> &sm, int32_t *__restrict__ dst, int n,
+                                                P1 after_count, P2 before_write)
+{
+    uint32_t *buf = sm.buf();
+    const int lane = threadIdx.x & 31;
+    int key[ITEMS];
+    uint32_t arr[ITEMS / 4];
+    int kmin = INT_MAX, kmax = INT_MIN;
+#pragma unroll
+    for (int i = 0; i < ITEMS / 4; ++i) {
+        if (i * 4 * THREADS < n) {
+            const int4 v = *reinterpret_cast<const int4 *>(buf + (i * THREADS + threadIdx.x) * 4);
+            key[4 * i] = v.x, key[4 * i + 1] = v.y, key[4 * i + 2] = v.z, key[4 * i + 3] = v.w;
+            if ((i + 1) * 4 * THREADS <= n) {
+                kmin = __vimin3_s32(kmin, __vimin3_s32(v.x, v.y, v.z), v.w);
+                kmax = __vimax3_s32(kmax, __vimax3_s32(v.x, v.y, v.z), v.w);
+            } else {
+                const int p = (i * THREADS + (int)threadIdx.x) * 4;
+#pragma unroll
+                for (int j = 0; j < 4; ++j) {
+                    if (p + j < n) {
+                        kmin = min(kmin, key[4 * i + j]);
+                        kmax = max(kmax, key[4 * i + j]);
+                    }
                 }
             }
         }
     }
-#pragma unroll
-    for (int k = 0; k < N; ++k)
-        if (k < c)
-            buf[s0 + k] = v[k];
-}
-
-// Sorts the n <= THREADS*kItems keys in sm.buf and writes them to dst (xor
-// kSign back to ids).  Keys are bucketed by value, (key - min) >> shift with
-// B = ceil(log2 n) - 1 bits (at most 13) of the key range, using shared
-// atomics, so a bucket of spread-out keys holds one to a few keys (about
-// five on average for the 40960-id class); each
-// bucket is then sorted in registers.  Measuring from the minimum keeps a
-// range that straddles a power of two (e.g. ids around 2^k, or of both
-// signs) from crowding into a few buckets.
-// Returns false, having written the unsorted ids to dst, if a bucket holds
-// more than kBucketCrowded keys (the caller then sorts dst with LSD).
-template <int THREADS, int ITEMS>
-__device__ __forceinline__ bool cta_bucket_sort(CtaSmem<THREADS, ITEMS> &sm, int32_t *__restrict__ dst,
-                                                int n)
-{
-    uint32_t key[ITEMS];
-    uint32_t kmin = 0xffffffffu, kmax = 0;
-#pragma unroll
-    for (int i = 0; i < ITEMS; ++i) {
-        if (i * THREADS >= n)
-            break;
-        const int p = i * THREADS + threadIdx.x;
-        key[i] = 0;
-        if (p < n) {
-            key[i] = sm.buf[p];
-            kmin = min(kmin, key[i]);
-            kmax = max(kmax, key[i]);
-        }
-    }
-    block_minmax<THREADS>(sm, kmin, kmax);
-    if (kmin == kmax) {  // all keys equal
+    block_minmax<THREADS>(sm.red0, sm.red1, kmin, kmax);
+    if (kmin == kmax) {  // all ids equal
         for (int p = threadIdx.x; p < n; p += THREADS)
-            dst[p] = (int32_t)(sm.buf[p] ^ kSign);
-        __syncthreads();
+            dst[p] = kmin;
         return true;
     }
-    // bucket = (key - kmin) >> shift: B = ceil(log2 n) - 1 bits (at most 13)
-    // of the key range, so only buckets inside [kmin, kmax] exist
-    const uint32_t span = kmax - kmin;
-    const int width = 32 - __clz(span);
-    int bits = (32 - __clz((unsigned)(n - 1))) - kBucketDensity;
-    constexpr int kMaxBits = CtaSmem<THREADS, ITEMS>::kCntBits;
-    bits = bits < 1 ? 1 : (bits > kMaxBits ? kMaxBits : bits);
-    if (bits > width)
-        bits = width;
-    const int shift = width - bits;
-    const int nb = (int)(span >> shift) + 1;
-    for (int b = threadIdx.x; b < nb; b += THREADS)
-        sm.cnt[b] = 0;
-    if (threadIdx.x == 0)
-        sm.crowded = 0;
-    __syncthreads();
+    BucketMap bm = bucket_map(n, kmin, kmax, sm.coarse);
+    bool eq = false;
+    if (!count_buckets<THREADS, ITEMS, false>(sm, bm, key, arr, n)) {
+        eq = true;
+        constexpr int C = kCoarse * THREADS;  // coarse bins
+        bm = bucket_map(C, kmin, kmax, sm.coarse);
+        zero_counters(sm, n);
 #pragma unroll
-    for (int i = 0; i < ITEMS; ++i) {
-        if (i * THREADS >= n)
-            break;
-        if (i * THREADS + threadIdx.x < n)
-            atomicAdd(&sm.cnt[(key[i] - kmin) >> shift], 1u);
-    }
-    __syncthreads();
-    {  // exclusive scan of the nb counts: each thread owns a run of them
-        const int per = (nb + THREADS - 1) / THREADS;
-        const int lo = threadIdx.x * per;
-        int sum = 0;
-        for (int b = lo; b < lo + per && b < nb; ++b)
-            sum += (int)sm.cnt[b];
-        int total;
-        int run = block_scan_int<THREADS>(sm, sum, &total);
-        for (int b = lo; b < lo + per && b < nb; ++b) {
-            const int c = (int)sm.cnt[b];
-            if (c > kBucketCrowded)
-                sm.crowded = 1;
-            sm.cnt[b] = (uint32_t)run;
-            run += c;
-        }
-    }
-    __syncthreads();
-    if (sm.crowded) {
-        for (int p = threadIdx.x; p < n; p += THREADS)
-            dst[p] = (int32_t)(sm.buf[p] ^ kSign);
+        for (int k = 0; k < kCoarse; ++k)
+            sm.coarse[k * THREADS + threadIdx.x] = 0;
         __syncthreads();
-        return false;
-    }
+        each_key<THREADS, ITEMS>(n, [&](int k, int) { atomicAdd(&sm.coarse[coarse_of(bm, key[k])], 1u); });
+        __syncthreads();
+        uint32_t h[kCoarse], sum = 0;
 #pragma unroll
-    for (int i = 0; i < ITEMS; ++i) {
-        if (i * THREADS >= n)
-            break;
-        if (i * THREADS + threadIdx.x < n) {
-            const uint32_t pos = atomicAdd(&sm.cnt[(key[i] - kmin) >> shift], 1u);
-            sm.buf[pos] = key[i];
+        for (int k = 0; k < kCoarse; ++k) {
+            h[k] = sm.coarse[kCoarse * threadIdx.x + k];
+            sum += h[k];
+        }
+        int total;
+        uint32_t run = (uint32_t)block_scan_int<THREADS>(sm.red1, (int)sum, &total);
+#pragma unroll
+        for (int k = 0; k < kCoarse; ++k) {
+            sm.coarse[kCoarse * threadIdx.x + k] = run;
+            run += h[k];
+        }
+        if (threadIdx.x == 0)
+            sm.coarse[C] = (uint32_t)total;
+        __syncthreads();
+        if (!count_buckets<THREADS, ITEMS, true>(sm, bm, key, arr, n)) {
+            each_key<THREADS, ITEMS>(n, [&](int k, int p) { dst[p] = key[k]; });
+            return false;
+        }
+    }
+    after_count();
+    if (threadIdx.x < kHalo)
+        buf[n + threadIdx.x] = (uint32_t)INT_MAX;
+    if (eq)
+        scatter_buckets<THREADS, ITEMS, true>(sm, bm, key, arr, n);
+    else
+        scatter_buckets<THREADS, ITEMS, false>(sm, bm, key, arr, n);
+    __syncthreads();
+    // Eight consecutive positions a thread and round, with four neighbours on
+    // either side: five rounds of odd-even transposition over the whole array
+    // (each thread computes what its own eight depend on).  A warp's tile is
+    // 252 positions: the lanes with bit 2 set start 124 positions on, so that
+    // the eight lanes of one 128-byte access phase hit different banks (the
+    // four positions both halves compute are equal).
+    const int place = (lane & 4) * 31 + 8 * ((lane & 3) | (lane >> 3 << 2));
+#pragma unroll
+    for (int i = 0; i < ITEMS / 8; ++i) {
+        const int p = (i * (THREADS / 32) + (int)(threadIdx.x >> 5)) * 252 + place;
+        if (p < n) {
+            int v[16];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                const int4 x = *reinterpret_cast<const int4 *>(buf + p - 4 + 4 * q);
+                v[4 * q] = x.x, v[4 * q + 1] = x.y, v[4 * q + 2] = x.z, v[4 * q + 3] = x.w;
+            }
+#pragma unroll
+            for (int r = 0; r < kNet; ++r) {
+#pragma unroll
+                for (int j = r; j < 15 - r; j += 2) {
+                    const int lo = min(v[j], v[j + 1]), hi = max(v[j], v[j + 1]);
+                    v[j] = lo;
+                    v[j + 1] = hi;
+                }
+            }
+#pragma unroll
+            for (int j = 0; j < 8; ++j)
+                key[8 * i + j] = v[4 + j];
         }
     }
     __syncthreads();
-    // cnt[b] is now the end of bucket b.  Each thread sorts whole buckets in
-    // registers with a sorting network sized to the warp's largest bucket.
-    for (int b0 = threadIdx.x - (threadIdx.x & 31); b0 < nb; b0 += THREADS) {
-        const int b = b0 + (threadIdx.x & 31);
-        int s0 = 0, c = 0;
-        if (b < nb) {
-            s0 = b ? (int)sm.cnt[b - 1] : 0;
-            c = (int)sm.cnt[b] - s0;
+#pragma unroll
+    for (int i = 0; i < ITEMS / 8; ++i) {
+        const int p = (i * (THREADS / 32) + (int)(threadIdx.x >> 5)) * 252 + place;
+        if (p < n) {
+            *reinterpret_cast<int4 *>(buf + p) = make_int4(key[8 * i], key[8 * i + 1], key[8 * i + 2], key[8 * i + 3]);
+            *reinterpret_cast<int4 *>(buf + p + 4) =
+                make_int4(key[8 * i + 4], key[8 * i + 5], key[8 * i + 6], key[8 * i + 7]);
         }
-        const int cmax = __reduce_max_sync(RT_FULL, c);
-        if (cmax <= 1)
-            continue;
-        if (cmax <= 4)
-            bucket_network<4>(sm.buf, s0, c);
-        else if (cmax <= 8)
-            bucket_network<8>(sm.buf, s0, c);
-        else if (cmax <= 16)
-            bucket_network<16>(sm.buf, s0, c);
-        else
-            bucket_network<32>(sm.buf, s0, c);
     }
     __syncthreads();
-    for (int p = threadIdx.x; p < n; p += THREADS)
-        dst[p] = (int32_t)(sm.buf[p] ^ kSign);
-    __syncthreads();
+    before_write();
+    // write-out, a warp 128 positions at a time
+    for (int p0 = (threadIdx.x >> 5) * 128; p0 < n; p0 += 4 * THREADS) {
+        const int *at = reinterpret_cast<const int *>(buf) + p0 + lane;
+        int32_t *to = dst + p0 + lane;
+        const uint4 w = *reinterpret_cast<const uint4 *>(sm.win + (p0 >> 5));
+        int k[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+            k[u] = at[32 * u];
+        if (p0 + 128 <= n && (w.x | w.y | w.z | w.w) == 0) {
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                to[32 * u] = k[u];
+        } else {  // the end of the segment, or a bucket too large for the network: count inversions
+            const int widest = (int)max(max(w.x, w.y), max(w.z, w.w));
+            int move[4] = {0, 0, 0, 0};
+            for (int d = 1; d <= widest; ++d) {
+#pragma unroll
+                for (int u = 0; u < 4; ++u) {
+                    move[u] += at[32 * u + d] < k[u];
+                    move[u] -= at[32 * u - d] > k[u];
+                }
+            }
+#pragma unroll
+            for (int u = 0; u < 4; ++u)
+                if (p0 + 32 * u + lane < n)
+                    to[32 * u + move[u]] = k[u];
+        }
+    }
     return true;
 }
 
@@ -580,61 +723,152 @@ __device__ __forceinline__ void push_large(const LongList &lg, int32_t seg, int6
     lg.tmp[slot] = (int64_t)atomicAdd(lg.hdr + HDR_SCRATCH, (unsigned long long)n);
 }
 
+constexpr int cta_per_sm(int threads, int items) { return (items <= 16 ? 1536 : 1024) / threads; }
+
 // One CTA per listed segment.  BUCKETS: the list holds SegDesc entries whose
-// keys sit in `scratch`; otherwise segment ids whose ids are gathered from S.
-// ITEMS keys per thread; a segment of more than 16384 ids whose buckets are
-// crowded goes to the MSD path.  CTAs claim list entries from the counter
-// *next (zero at launch), so a CTA that drew short segments takes more.
-template <int THREADS, bool BUCKETS, int ITEMS = kItems>
-__global__ void __launch_bounds__(THREADS, 1024 / THREADS)
+// ids sit in `scratch`; otherwise segment ids whose ids are gathered from S.
+// A segment of more than 16384 ids whose buckets overflow goes to the MSD
+// path.  CTAs claim list entries from the counter *next (zero at launch), so
+// a CTA that drew short segments takes more.
+template <int THREADS, int ITEMS, bool BUCKETS>
+__global__ void __launch_bounds__(THREADS, cta_per_sm(THREADS, ITEMS))
     k_sort_cta(const void *__restrict__ list, const unsigned long long *__restrict__ count,
                int64_t list_cap, const int64_t *__restrict__ off, SortSources S,
-               const uint32_t *__restrict__ scratch, int32_t *__restrict__ out,
+               const int32_t *__restrict__ scratch, int32_t *__restrict__ out,
                SegDesc *__restrict__ crowded, unsigned long long *__restrict__ n_crowded,
                int64_t crowded_cap, LongList lg, unsigned long long *__restrict__ next)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    CtaSmem<THREADS, ITEMS> &sm = *reinterpret_cast<CtaSmem<THREADS, ITEMS> *>(smem_raw);
+    using Smem = CtaSmem<THREADS, ITEMS>;
+    Smem &sm = *reinterpret_cast<Smem *>(smem_raw);
     const int64_t cnt = list_len(count, list_cap);
-    for (;;) {
+    if (threadIdx.x < kHalo)
+        sm.slots[threadIdx.x] = (uint32_t)INT_MIN;
+    // The next piece is claimed and its description loaded by the first warp
+    // while the current one is sorted, one dependent load per phase (claim,
+    // list entry, offsets); the chain's latency was a tenth of the time of
+    // the largest class, of which an SM holds one CTA.
+    const bool first = threadIdx.x < 32;
+    unsigned long long claimed = 0;
+    int32_t seg = -1;
+    int64_t v = 0;
+    int32_t hits = 0;
+    auto claim = [&] {
         if (threadIdx.x == 0)
-            sm.claim = (long long)atomicAdd(next, 1ull);
-        __syncthreads();
-        const int64_t b = sm.claim;
-        __syncthreads();  // every thread has read the claim before the next one is written
-        if (b >= cnt)
-            break;
-        int64_t dof;
-        int n;
+            claimed = atomicAdd(next, 1ull);
+    };
+    auto load_entry_of_list = [&] {
+        if (!first)
+            return;
+        const long long c = (long long)__shfl_sync(RT_FULL, claimed, 0);
+        seg = c >= cnt ? -1 : BUCKETS ? (int32_t)c : static_cast<const int32_t *>(list)[c];
+    };
+    auto load_fields = [&] {  // lane j: field j
+        const int j = threadIdx.x;
+        v = 0;
+        if (!first || seg < 0)
+            return;
         if (BUCKETS) {
-            const SegDesc d = static_cast<const SegDesc *>(list)[b];
-            dof = d.dst;
-            n = d.n;
-            if (n > THREADS * ITEMS)
-                continue;
-            cta_load<THREADS>(sm, scratch + d.src, n, 0u);
+            const SegDesc *d = static_cast<const SegDesc *>(list) + seg;
+            v = j == 0 ? d->dst : j == 1 ? d->n : j == 2 ? d->src : 0;
         } else {
-            const int32_t seg = static_cast<const int32_t *>(list)[b];
-            dof = off[seg];
-            n = (int)(off[seg + 1] - dof);
-            if (n > THREADS * ITEMS)
-                continue;
-            cta_gather<THREADS>(sm, S, seg);
+            const int64_t *at = j < 2 ? off + seg + j : j < 4 ? S.off_leaf + seg + (j - 2) : S.off_rng + seg + (j - 4);
+            if (j < 4 || (j < 6 && S.rng))
+                v = *at;
+            hits = S.leaf_len ? S.leaf_len[seg] : 0;
         }
-        if (!cta_bucket_sort<THREADS>(sm, out + dof, n) && threadIdx.x == 0) {
-            if (!BUCKETS && n > kCtaMax)  // longer than the LSD fallback takes: MSD path
-                push_large(lg, static_cast<const int32_t *>(list)[b], n);
+    };
+    auto store_piece = [&] {
+        if (!first)
+            return;
+        const int64_t f0 = __shfl_sync(RT_FULL, v, 0), f1 = __shfl_sync(RT_FULL, v, 1), f2 = __shfl_sync(RT_FULL, v, 2),
+                      f3 = __shfl_sync(RT_FULL, v, 3), f4 = __shfl_sync(RT_FULL, v, 4), f5 = __shfl_sync(RT_FULL, v, 5);
+        if (threadIdx.x == 0) {
+            Piece m;
+            m.dst = f0;
+            m.src = f2;
+            m.rng = f4;
+            m.n = seg < 0 ? -1 : (int)(BUCKETS ? f1 : f1 - f0);
+            const int64_t nl = BUCKETS ? f1 : S.leaf_len ? hits : f3 - f2;
+            m.nl = (int)(nl < m.n ? nl : m.n);
+            m.nr = (int)(f5 - f4);
+            m.seg = seg;
+            sm.next = m;
+        }
+    };
+    claim();
+    load_entry_of_list();
+    load_fields();
+    store_piece();
+    for (;;) {
+        __syncthreads();  // also: the previous piece is done with the shared memory
+        const Piece m = sm.next;
+        if (m.n < 0)
+            break;
+        claim();
+        bool ok = true;
+        bool loaded = false;
+        if (m.n <= Smem::N) {
+            zero_counters(sm, m.n);
+            if (BUCKETS)
+                copy_async(sm.buf(), scratch + m.src, m.n, threadIdx.x, THREADS);
             else
-                push_crowded(crowded, n_crowded, crowded_cap, dof, n);
+                cta_gather(sm, S, m);
+            cp_async_wait();
+            __syncthreads();
+            ok = cta_bucket_sort(sm, out + m.dst, m.n, load_entry_of_list, [&] {
+                load_fields();
+                loaded = true;
+            });
+        } else {
+            __syncthreads();  // every thread has read sm.next
+        }
+        if (!loaded) {
+            load_entry_of_list();
+            load_fields();
+        }
+        store_piece();
+        if (!ok && threadIdx.x == 0) {
+            if (THREADS == 1024)  // the long path follows on this class's stream
+                push_large(lg, m.seg, m.n);
+            else
+                push_crowded(crowded, n_crowded, crowded_cap, m.dst, m.n);
         }
     }
+}
+
+// Shared memory of the LSD fallback.
+struct LsdSmem {
+    static constexpr int W = 32;
+    uint32_t buf[1024 * kItems];
+    uint32_t wcnt[W][kBins];
+    uint32_t dcount[kBins];
+    uint32_t dstart[kBins];
+    uint32_t red0[W], red1[W];
+};
+
+// Block-wide AND and OR of the keys' bits; every thread gets AND ^ OR.
+__device__ __forceinline__ uint32_t block_diff(LsdSmem &sm, uint32_t a_and, uint32_t a_or)
+{
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    a_and = __reduce_and_sync(RT_FULL, a_and);
+    a_or = __reduce_or_sync(RT_FULL, a_or);
+    if (lane == 0) {
+        sm.red0[w] = a_and;
+        sm.red1[w] = a_or;
+    }
+    __syncthreads();
+    a_and = __reduce_and_sync(RT_FULL, sm.red0[lane]);
+    a_or = __reduce_or_sync(RT_FULL, sm.red1[lane]);
+    __syncthreads();
+    return a_and ^ a_or;
 }
 
 // Ranks the keys held in registers for one LSD pass; on return pos[i] is the
 // position of key[i] in the pass's output order.  Warp w owns keys
 // [w*run, (w+1)*run), taken 32 at a time.
 template <int THREADS>
-__device__ __forceinline__ void rank_pass(CtaSmem<THREADS> &sm, const uint32_t (&key)[kItems],
+__device__ __forceinline__ void rank_pass(LsdSmem &sm, const uint32_t (&key)[kItems],
                                           int rounds, int run, int n, int shift,
                                           uint32_t (&pos)[kItems])
 {
@@ -699,7 +933,7 @@ __device__ __forceinline__ void rank_pass(CtaSmem<THREADS> &sm, const uint32_t (
 }
 
 // Stable LSD radix sort of n <= 16384 ids in place at ids[0 .. n).
-__device__ __forceinline__ void cta_lsd_sort(CtaSmem<1024> &sm, int32_t *__restrict__ ids, int n)
+__device__ __forceinline__ void cta_lsd_sort(LsdSmem &sm, int32_t *__restrict__ ids, int n)
 {
     constexpr int THREADS = 1024, W = 32;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -717,7 +951,7 @@ __device__ __forceinline__ void cta_lsd_sort(CtaSmem<1024> &sm, int32_t *__restr
             a_or |= key[i];
         }
     }
-    const uint32_t diff = block_diff<THREADS>(sm, a_and, a_or);
+    const uint32_t diff = block_diff(sm, a_and, a_or);
     int last = -1;
     for (int shift = 0; shift < 32; shift += 8)
         if ((diff >> shift) & 0xffu)
@@ -753,7 +987,7 @@ __global__ void __launch_bounds__(1024, 1)
                int64_t cap, int32_t *__restrict__ out)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    CtaSmem<1024> &sm = *reinterpret_cast<CtaSmem<1024> *>(smem_raw);
+    LsdSmem &sm = *reinterpret_cast<LsdSmem *>(smem_raw);
     int64_t cnt = (int64_t)*count;
     if (cnt > cap)
         cnt = cap;
@@ -774,8 +1008,6 @@ __global__ void __launch_bounds__(1024)
                    unsigned long long *__restrict__ next)
 {
     const int64_t cnt = list_len(count, list_cap);
-    __shared__ int32_t rstart[1024];
-    __shared__ int32_t wsum[32];
     __shared__ long long claim;
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     for (;;) {
@@ -794,48 +1026,21 @@ __global__ void __launch_bounds__(1024)
         if (S.leaf + l0 != dst)
             for (int64_t e = l0 + threadIdx.x; e < l1; e += 1024)
                 dst[e - l0] = S.leaf[e];
-        int64_t pos = l1 - l0;
         if (!S.rng)
             continue;
         const int64_t r0 = S.off_rng[i], r1 = S.off_rng[i + 1];
-        for (int64_t rb = r0; rb < r1; rb += 1024) {
-            const int64_t r = rb + threadIdx.x;
-            int2 rg = make_int2(0, 0);
-            if (r < r1)
-                rg = S.rng[r];
-            const int len = rg.y - rg.x;
-            int inc = len;
-#pragma unroll
-            for (int o = 1; o < 32; o <<= 1) {
-                const int u = __shfl_up_sync(RT_FULL, inc, o);
-                if (lane >= o)
-                    inc += u;
-            }
-            if (lane == 31)
-                wsum[w] = inc;
-            __syncthreads();
-            int before = 0, all = 0;
-            for (int x = 0; x < 32; ++x) {
-                if (x < w)
-                    before += wsum[x];
-                all += wsum[x];
-            }
-            rstart[threadIdx.x] = before + inc - len;
-            __syncthreads();
-            const int cntr = (int)(r1 - rb < 1024 ? r1 - rb : 1024);
-            for (int k = w; k < cntr; k += 32) {
-                const int2 g = S.rng[rb + k];
-                const int64_t st = pos + rstart[k];
-                for (int e = lane; e < g.y - g.x; e += 32)
-                    dst[st + e] = __ldg(S.tree_ids + g.x + e);
-            }
-            pos += all;
-            __syncthreads();
+        const int64_t nl = l1 - l0;
+        const int nrl = (int)(off[i + 1] - off[i] - nl);
+        for (int64_t r = r0 + w; r < r1; r += 32) {
+            const int2 g = S.rng[r];
+            const int e = r + 1 < r1 ? S.rng[r + 1].y : nrl;
+            for (int x = lane; x < e - g.y; x += 32)
+                dst[nl + g.y + x] = __ldg(S.tree_ids + g.x + x);
         }
     }
 }
 
-// One CTA per listed long segment (over 40960 ids, or over 16384 with crowded
+// One CTA per listed long segment (over 32768 ids, or over 16384 with crowded
 // buckets): partitions its keys by their top b differing bits (2^b buckets
 // of about kCtaMax/2) into the scratch area and lists every bucket for the
 // CTA sort (or, if a bucket is still too long, for the global LSD fallback).
@@ -843,7 +1048,7 @@ __global__ void __launch_bounds__(1024)
     k_msd_partition(const int32_t *__restrict__ list, const int64_t *__restrict__ tmp_off,
                     const unsigned long long *__restrict__ count, int64_t list_cap,
                     int64_t scratch_cap, const int64_t *__restrict__ off,
-                    const uint32_t *__restrict__ ids, uint32_t *__restrict__ scratch,
+                    const int32_t *__restrict__ ids, int32_t *__restrict__ scratch,
                     SegDesc *__restrict__ buckets, SegDesc *__restrict__ oversize, int64_t desc_cap,
                     unsigned long long *__restrict__ hdr, int32_t *__restrict__ flags,
                     unsigned long long *__restrict__ next)
@@ -872,7 +1077,7 @@ __global__ void __launch_bounds__(1024)
         }
         uint32_t a_and = 0xffffffffu, a_or = 0;
         for (int64_t p = threadIdx.x; p < n; p += 1024) {
-            const uint32_t k = ids[o + p] ^ kSign;
+            const uint32_t k = (uint32_t)ids[o + p] ^ kSign;
             a_and &= k;
             a_or |= k;
         }
@@ -908,7 +1113,7 @@ __global__ void __launch_bounds__(1024)
         const int shift = hb + 1 - nb_bits;
         const uint32_t mask = (1u << nb_bits) - 1u;
         for (int64_t p = threadIdx.x; p < n; p += 1024)
-            atomicAdd(&hist[((ids[o + p] ^ kSign) >> shift) & mask], 1u);
+            atomicAdd(&hist[(((uint32_t)ids[o + p] ^ kSign) >> shift) & mask], 1u);
         __syncthreads();
         if (threadIdx.x < 32) {
             uint32_t carry = 0;
@@ -933,7 +1138,7 @@ __global__ void __launch_bounds__(1024)
             s.dst = o + cursor[d];
             s.n = (int32_t)hist[d];
             s.pad = 0;
-            if (hist[d] <= (uint32_t)kCtaMax) {
+            if (hist[d] <= (uint32_t)kMidMax) {
                 const unsigned long long slot = atomicAdd(hdr + HDR_BUCKETS, 1ull);
                 if ((int64_t)slot < desc_cap)
                     buckets[slot] = s;
@@ -949,20 +1154,20 @@ __global__ void __launch_bounds__(1024)
         }
         __syncthreads();
         for (int64_t p = threadIdx.x; p < n; p += 1024) {
-            const uint32_t k = ids[o + p] ^ kSign;
-            const uint32_t pos = atomicAdd(&cursor[(k >> shift) & mask], 1u);
-            scratch[t + pos] = k;
+            const int32_t id = ids[o + p];
+            const uint32_t pos = atomicAdd(&cursor[(((uint32_t)id ^ kSign) >> shift) & mask], 1u);
+            scratch[t + pos] = id;
         }
         __syncthreads();
     }
 }
 
 // Fallback for buckets longer than kCtaMax (heavily skewed ids): LSD radix
-// sort through global memory from the bucket's scratch range (keys) to its
+// sort through global memory from the bucket's scratch range to its
 // place in the output, ping-ponging between the two.
 __global__ void __launch_bounds__(256)
     k_sort_global(const SegDesc *__restrict__ list, const unsigned long long *__restrict__ count,
-                  int64_t list_cap, uint32_t *__restrict__ scratch, int32_t *__restrict__ ids)
+                  int64_t list_cap, int32_t *__restrict__ scratch, int32_t *__restrict__ ids)
 {
     const int64_t cnt = list_len(count, list_cap);
     __shared__ uint32_t hist[kBins], run[kBins];
@@ -970,7 +1175,7 @@ __global__ void __launch_bounds__(256)
     const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     for (int64_t b = blockIdx.x; b < cnt; b += gridDim.x) {
         const SegDesc d = list[b];
-        uint32_t *x = scratch + d.src;                            // keys (flipped)
+        uint32_t *x = reinterpret_cast<uint32_t *>(scratch) + d.src;
         uint32_t *y = reinterpret_cast<uint32_t *>(ids) + d.dst;  // output area
         const int64_t n = d.n;
         uint32_t a_and = 0xffffffffu, a_or = 0;
@@ -1002,7 +1207,7 @@ __global__ void __launch_bounds__(256)
             hist[threadIdx.x] = 0;
             __syncthreads();
             for (int64_t p = threadIdx.x; p < n; p += 256)
-                atomicAdd(&hist[(src[p] >> shift) & 0xffu], 1u);
+                atomicAdd(&hist[((src[p] ^ kSign) >> shift) & 0xffu], 1u);
             __syncthreads();
             if (threadIdx.x < 32) {
                 uint32_t carry = 0;
@@ -1027,7 +1232,7 @@ __global__ void __launch_bounds__(256)
                     const int64_t p = p0 + lane;
                     const bool ok = p < n;
                     const uint32_t k = ok ? src[p] : 0u;
-                    const int dg = ok ? (int)((k >> shift) & 0xffu) : kBins;
+                    const int dg = ok ? (int)(((k ^ kSign) >> shift) & 0xffu) : kBins;
                     const unsigned peers = __match_any_sync(RT_FULL, dg);
                     const uint32_t base = ok ? run[dg] : 0u;
                     if (ok)
@@ -1043,8 +1248,9 @@ __global__ void __launch_bounds__(256)
             src = dst;
             dst = tmp;
         }
-        for (int64_t p = threadIdx.x; p < n; p += 256)
-            y[p] = src[p] ^ kSign;
+        if (src != y)
+            for (int64_t p = threadIdx.x; p < n; p += 256)
+                y[p] = src[p];
         __syncthreads();
     }
 }
@@ -1064,15 +1270,15 @@ struct Crowded {
     int64_t cap;
 };
 
-template <int THREADS, bool BUCKETS, int ITEMS = kItems>
+template <int THREADS, int ITEMS, bool BUCKETS>
 rtree_status launch_cta(const void *list, const unsigned long long *count, int64_t list_cap,
-                        const int64_t *off, const SortSources &S, const uint32_t *scratch,
+                        const int64_t *off, const SortSources &S, const int32_t *scratch,
                         int32_t *out, const Crowded &cr, unsigned long long *next, cudaStream_t s,
                         const char *name, const LongList &lg = LongList{})
 {
     if (list_cap <= 0)
         return RTREE_OK;
-    auto kern = k_sort_cta<THREADS, BUCKETS, ITEMS>;
+    auto kern = k_sort_cta<THREADS, ITEMS, BUCKETS>;
     const size_t bytes = sizeof(CtaSmem<THREADS, ITEMS>);
     RT_TRY(set_smem(kern, bytes));
     int per_sm = 0;
@@ -1091,7 +1297,7 @@ rtree_status launch_lsd(const Crowded &cr, int32_t *out, cudaStream_t s)
 {
     if (cr.cap <= 0)
         return RTREE_OK;
-    const size_t bytes = sizeof(CtaSmem<1024>);
+    const size_t bytes = sizeof(LsdSmem);
     RT_TRY(set_smem(k_sort_lsd, bytes));
     KernelTimer kt_("sort_lsd", s);
     k_sort_lsd<<<(unsigned)sm_count(), 1024, bytes, s>>>(cr.list, cr.count, cr.cap, out);
@@ -1205,7 +1411,7 @@ rtree_status segmented_sort_gather(int32_t *out, const int64_t *offsets, int64_t
     // Every list length stays on the device; the launches below are sized
     // by upper bounds and read the actual lengths themselves, so the whole
     // sort is enqueued without a host round trip.
-    const int64_t max_large = total / (kCtaMax + 1) + 1 < nseg ? total / (kCtaMax + 1) + 1 : nseg;
+    const int64_t max_large = total / (kMidMax + 1) + 1 < nseg ? total / (kMidMax + 1) + 1 : nseg;
     const int64_t scratch_cap = total;
     const int64_t desc_cap = 2 * max_large + 4 * (scratch_cap / kCtaMax) + 256;
     DevBuf<int32_t> lists(s);
@@ -1214,7 +1420,7 @@ rtree_status segmented_sort_gather(int32_t *out, const int64_t *offsets, int64_t
     RT_TRY(lists.alloc((size_t)C_COUNT * nseg, "sort lists"));
     RT_TRY(large_tmp.alloc(nseg, "sort lists"));
     // the header, two crowded-list counters, and one claim counter per CTA-sort launch
-    constexpr int kClaims = 8;
+    constexpr int kClaims = 9;
     RT_TRY(hdr.alloc(HDR_WORDS + 2 + kClaims, "sort counters"));
     RT_CUDA(cudaMemsetAsync(hdr.p, 0, (HDR_WORDS + 2 + kClaims) * sizeof(unsigned long long), s));
     auto claim = [&](int k) { return hdr.p + HDR_WORDS + 2 + k; };
@@ -1237,9 +1443,9 @@ rtree_status segmented_sort_gather(int32_t *out, const int64_t *offsets, int64_t
     RT_TRY(crowded.alloc(cta_cap > 0 ? cta_cap : 1, "sort crowded list"));
     unsigned long long *n_crowded = hdr.p + HDR_WORDS;  // two counters after the header
     const Crowded cr1{crowded.p, n_crowded, cta_cap};
-    const bool long_path = total > kCtaMax;  // else no segment can be long
-    // the long path's buffers (segments over 40960 ids, or crowded over 16384)
-    DevBuf<uint32_t> scratch(s);
+    const bool long_path = total > kMidMax;  // else no segment can be long
+    // the long path's buffers (segments over 32768 ids, or crowded over 16384)
+    DevBuf<int32_t> scratch(s);
     DevBuf<SegDesc> buckets(s), oversize(s), crowded2(s);
     if (long_path) {
         RT_TRY(scratch.alloc(scratch_cap, "sort scratch"));
@@ -1248,7 +1454,7 @@ rtree_status segmented_sort_gather(int32_t *out, const int64_t *offsets, int64_t
         RT_TRY(crowded2.alloc(desc_cap, "sort crowded list"));
     }
     // Three side streams and the call's stream run the classes side by side:
-    //   side 2: the 40960-id CTA sort, then the long path (which it feeds);
+    //   side 2: the 32768-id CTA sort, then the long path (which it feeds);
     //   side 1: the CTA sorts up to 8192 ids;
     //   side 0: the warp sorts;
     //   stream: the CTA sort up to 16384 ids, then (after side 1) the LSD
@@ -1257,12 +1463,11 @@ rtree_status segmented_sort_gather(int32_t *out, const int64_t *offsets, int64_t
     // SMs their last CTAs leave idle.
     Fork fk;
     RT_TRY(fk.begin(s));
-    constexpr int M = kItemsMid;
     if (long_path) {
         const cudaStream_t s2 = fk.side(2);
         const LongList lg{L(C_LARGE), large_tmp.p, hdr.p};
-        RT_TRY((launch_cta<1024, false, kItemsBig>(L(C_CTA40K), H(C_CTA40K), cap_of(kCtaMax + 1), offsets, S,
-                                                   nullptr, out, cr1, claim(0), s2, "sort_cta", lg)));
+        RT_TRY((launch_cta<1024, 32, false>(L(C_CTA32K), H(C_CTA32K), cap_of(kMidMax + 1), offsets, S, nullptr, out,
+                                        cr1, claim(0), s2, "sort_cta", lg)));
         // Long segments: gather into place, MSD-partition into the scratch
         // area, then sort the buckets back into place.
         const int64_t grid = max_large < (int64_t)sms * 2 ? max_large : (int64_t)sms * 2;
@@ -1276,12 +1481,12 @@ rtree_status segmented_sort_gather(int32_t *out, const int64_t *offsets, int64_t
             KernelTimer kt_("sort_msd", s2);
             k_msd_partition<<<(unsigned)grid, 1024, 0, s2>>>(
                 L(C_LARGE), large_tmp.p, H(C_LARGE), max_large, scratch_cap, offsets,
-                reinterpret_cast<const uint32_t *>(out), scratch.p, buckets.p, oversize.p, desc_cap,
+                out, scratch.p, buckets.p, oversize.p, desc_cap,
                 hdr.p, flags, claim(7));
             RT_LAUNCH();
         }
         const Crowded cr2{crowded2.p, n_crowded + 1, desc_cap};
-        RT_TRY((launch_cta<512, true, kItemsMid>(buckets.p, H(HDR_BUCKETS), desc_cap, nullptr, S, scratch.p, out, cr2, claim(1), s2, "sort_bucket")));
+        RT_TRY((launch_cta<512, 32, true>(buckets.p, H(HDR_BUCKETS), desc_cap, nullptr, S, scratch.p, out, cr2, claim(1), s2, "sort_bucket")));
         RT_TRY(launch_lsd(cr2, out, s2));
         {
             int64_t g2 = desc_cap < (int64_t)sms * 4 ? desc_cap : (int64_t)sms * 4;
@@ -1291,11 +1496,12 @@ rtree_status segmented_sort_gather(int32_t *out, const int64_t *offsets, int64_t
             RT_LAUNCH();
         }
     }
-    RT_TRY((launch_cta<512, false, M>(L(C_CTA16K), H(C_CTA16K), cap_of(8193), offsets, S, nullptr, out, cr1, claim(2), s, "sort_cta")));
+    RT_TRY((launch_cta<512, 32, false>(L(C_CTA16K), H(C_CTA16K), cap_of(cta_ids(512, 16) + 1), offsets, S, nullptr, out, cr1, claim(2), s, "sort_cta")));
     const cudaStream_t s1 = fk.side(1), s0 = fk.side(0);
-    RT_TRY((launch_cta<256, false, M>(L(C_CTA8K), H(C_CTA8K), cap_of(4097), offsets, S, nullptr, out, cr1, claim(3), s1, "sort_cta")));
-    RT_TRY((launch_cta<128, false, M>(L(C_CTA4K), H(C_CTA4K), cap_of(2049), offsets, S, nullptr, out, cr1, claim(4), s1, "sort_cta")));
-    RT_TRY((launch_cta<64, false, M>(L(C_CTA2K), H(C_CTA2K), cap_of(257), offsets, S, nullptr, out, cr1, claim(5), s1, "sort_cta")));
+    RT_TRY((launch_cta<512, 16, false>(L(C_CTA8K), H(C_CTA8K), cap_of(cta_ids(256, 16) + 1), offsets, S, nullptr, out, cr1, claim(3), s1, "sort_cta")));
+    RT_TRY((launch_cta<256, 16, false>(L(C_CTA4K), H(C_CTA4K), cap_of(cta_ids(128, 16) + 1), offsets, S, nullptr, out, cr1, claim(4), s1, "sort_cta")));
+    RT_TRY((launch_cta<128, 16, false>(L(C_CTA2K), H(C_CTA2K), cap_of(cta_ids(64, 16) + 1), offsets, S, nullptr, out, cr1, claim(5), s1, "sort_cta")));
+    RT_TRY((launch_cta<64, 16, false>(L(C_CTA1K), H(C_CTA1K), cap_of(257), offsets, S, nullptr, out, cr1, claim(8), s1, "sort_cta")));
     RT_TRY(launch_warp<8>(L(C_W8), H(C_W8), cap_of(129), offsets, S, out, s0));
     RT_TRY(launch_warp<4>(L(C_W4), H(C_W4), cap_of(65), offsets, S, out, s0));
     RT_TRY(launch_warp<2>(L(C_W2), H(C_W2), cap_of(33), offsets, S, out, s0));

@@ -30,9 +30,10 @@
 //   COUNT    per query: ids found, and (optionally) how many came one by one
 //            from leaves and how many whole subtrees were taken;
 //   SCATTER  writes the ids themselves in traversal order (unsorted output);
-//   DESC     writes the leaf hits and, for every whole subtree, its (lo, hi)
-//            range of the tree's id array; the sorted output is then built
-//            by the segmented sort, which reads the ranges directly;
+//   DESC     writes the leaf hits and, for every whole subtree, where its run
+//            of the tree's id array starts and its place among the query's
+//            run ids; the sorted output is then built by the segmented sort,
+//            which reads the runs directly;
 //   BOUND    the count pass stopped above the leaves, sizing DESC's slots.
 // With warp per query at F = 64 and 128, DESC visits a leaf-parent's
 // intersecting leaves in place (no push, no pop) and derives each leaf's id
@@ -129,6 +130,23 @@ __device__ __forceinline__ int64_t reserve(int32_t *cursor, int n, int lane)
     if (lane == 0 && n > 0)
         r = atomicAdd(cursor, n);
     return __shfl_sync(RT_FULL, r, 0);
+}
+
+// Ids in the runs of the lower lanes of mc (len: the lane's run, 0 outside
+// mc).  Runs are nearly always whole leaves of F ids.
+template <int F>
+__device__ __forceinline__ int ids_before(unsigned mc, int len, int lane, unsigned lt)
+{
+    if (!__any_sync(RT_FULL, ((mc >> lane) & 1u) && len != F))
+        return F * __popc(mc & lt);
+    int inc = len;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int u = __shfl_up_sync(RT_FULL, inc, o);
+        if (lane >= o)
+            inc += u;
+    }
+    return inc - len;
 }
 
 // One step of a walk: pops up to K nodes from the warp's stack, tests their
@@ -241,8 +259,9 @@ __device__ __forceinline__ void select_step(const TreeDev &t, const float4 q, in
                     hi = lo + cn;
                 }
                 const int64_t o = sg.rbase + wk.rcur + __popc(mc & lt);
+                const int place = wk.cur - wk.lcur + ids_before<F>(mc, hi - lo, lane, lt);
                 if (cont && o < sg.rlim && o < io.rng_cap)
-                    io.rng_out[o] = make_int2(lo, hi);
+                    io.rng_out[o] = make_int2(lo, place);
                 wk.rcur += __popc(mc);
                 wk.cur += __reduce_add_sync(RT_FULL, (unsigned)(hi - lo));
             }
@@ -335,8 +354,11 @@ __device__ __forceinline__ void select_step(const TreeDev &t, const float4 q, in
             if (PASS == PASS_DESC) {
                 const int64_t at = WQ ? sg.rbase + reserve(io.cur_rng + qi, __popc(mc), lane) : sg.rbase + wk.rcur;
                 const int64_t o = at + __popc(mc & lt);
+                // several warps may serve a query of the work queue: its
+                // entries get their lengths here, their places afterwards
+                const int place = WQ ? hi - lo : wk.cur - wk.lcur + ids_before<F>(mc, hi - lo, lane, lt);
                 if (cont && o < sg.rlim && o < io.rng_cap)
-                    io.rng_out[o] = make_int2(lo, hi);
+                    io.rng_out[o] = make_int2(lo, place);
             }
             wk.rcur += __popc(mc);
             if (PASS == PASS_SCATTER) {
@@ -664,6 +686,32 @@ __global__ void k_wq_check(const SelIO io, int pass, int64_t Q, int32_t *__restr
     }
 }
 
+// After a work-queue descriptor pass: the lengths in the range entries become
+// places (one warp per query scans them).
+__global__ void k_wq_places(const SelIO io, int64_t Q)
+{
+    const int lane = threadIdx.x & 31;
+    const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
+    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+    for (int64_t i = warp; i < Q; i += nwarps) {
+        const int64_t r0 = io.off_rng[i], r1 = io.off_rng[i + 1] < io.rng_cap ? io.off_rng[i + 1] : io.rng_cap;
+        int place = 0;
+        for (int64_t b = r0; b < r1; b += 32) {
+            const int len = b + lane < r1 ? io.rng_out[b + lane].y : 0;
+            int inc = len;
+#pragma unroll
+            for (int o = 1; o < 32; o <<= 1) {
+                const int u = __shfl_up_sync(RT_FULL, inc, o);
+                if (lane >= o)
+                    inc += u;
+            }
+            if (b + lane < r1)
+                io.rng_out[b + lane].y = place + inc - len;
+            place += __shfl_sync(RT_FULL, inc, 31);
+        }
+    }
+}
+
 using SelectKernel = void (*)(TreeDev, const float4 *, int64_t, SelIO, unsigned long long *,
                               int32_t *, int, unsigned long long *);
 
@@ -812,6 +860,12 @@ rtree_status launch_wq(int pass, const rtree *t, const float4 *q, int64_t Q, con
         KernelTimer kt_("wq_check", s);
         int64_t b = (Q + 255) / 256;
         k_wq_check<<<(unsigned)(b > 65536 ? 65536 : b), 256, 0, s>>>(io, pass, Q, flags);
+        RT_LAUNCH();
+    }
+    if (pass == PASS_DESC) {
+        KernelTimer kt_("wq_places", s);
+        const int64_t b = (Q + 7) / 8;
+        k_wq_places<<<(unsigned)(b > 65536 ? 65536 : b), 256, 0, s>>>(io, Q);
         RT_LAUNCH();
     }
     return RTREE_OK;
