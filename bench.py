@@ -209,13 +209,12 @@ def source_sha(files, read=None):
 
 KERNEL_SOURCES = {"select_count": ["select.cu", "internal.cuh"], "select_bound": ["select.cu", "internal.cuh"],
                   "select_desc": ["select.cu", "internal.cuh"],
-                  "join_scatter": ["join.cu", "internal.cuh"],
-                  "join_pruned_count": ["join.cu", "internal.cuh"],
-                  "join_pruned_scatter": ["join.cu", "internal.cuh"],
+                  "join_levels": ["join.cu", "internal.cuh"],
+                  "join_pruned_levels": ["join.cu", "internal.cuh"],
                   "select_scatter": ["select.cu", "internal.cuh"],
                   "sort_warp": ["segsort.cu"], "sort_cta": ["segsort.cu"], "sort_gather": ["segsort.cu"],
                   "sort_msd": ["segsort.cu"], "sort_bucket": ["segsort.cu"], "sort_all": ["segsort.cu"],
-                  "scatter": ["radix_sort.cu"], "join_count": ["join.cu", "internal.cuh"]}
+                  "scatter": ["radix_sort.cu"]}
 
 
 def config_matches(kv, fanout, layout=None):
@@ -285,15 +284,15 @@ def algorithmic_bytes(stats, F, Q, seg_sizes):
 
 
 def join_roofline(st, Fr, Fs, kern, hbm, peak_kind, clk):
-    """Roofline of the join's traversal kernels (count and scatter passes of
-    every level, one launch each), from the traversal counters.
+    """Roofline of the join's traversal kernels (one pass per level), from the
+    traversal counters.
 
     Bytes: a node pair tested at equal heights reads both nodes' entries
     ((Fr + Fs) * 16 B) and two node records (32 B); a one-sided descent
-    reads the taller node's entries and the other node's box.  The scatter
-    pass also writes 8 B per child pair or result pair it emits.  Tests: a
-    node pair at equal heights takes Fr * Fs predicate tests, a one-sided
-    descent F tests.  The issue-slot side needs instruction counts from ncu
+    reads the taller node's entries and the other node's box; 8 B are written
+    per child pair or result pair.  Tests: a node pair at equal heights decides
+    Fr * Fs pairs of children (most of them through the nodes' boxes), a
+    one-sided descent F.  The issue-slot side needs instruction counts from ncu
     (profiles/ncu_metrics.txt) and is reported when they were taken on the
     current source."""
     eq = st["pairs_equal_internal"] + st["pairs_leaf"]
@@ -306,12 +305,12 @@ def join_roofline(st, Fr, Fs, kern, hbm, peak_kind, clk):
     ms = sum(v[1] for v in kern.values())
     if ms <= 0:
         return None
-    algo = 2 * node_bytes + 8 * emitted
+    algo = node_bytes + 8 * emitted
     achieved = algo / (ms / 1e3) / 1e9
     out = {"kernels": names, "bound": "hbm", "achieved": round(achieved, 1), "peak": hbm, "unit": "GB/s",
            "frac": round(achieved / hbm, 4), "peak_kind": peak_kind, "ms_per_step": round(ms, 4),
            "algorithmic_bytes_per_step": int(algo), "node_pairs": int(visited),
-           "predicate_tests_per_s": round(2 * tests / (ms / 1e3), 1)}
+           "predicate_tests_per_s": round(tests / (ms / 1e3), 1)}
     issue = issue_fraction([n for n in names], visited, ms, clk, fanout=Fr)
     if issue:
         out["issue"] = issue
