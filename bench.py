@@ -212,8 +212,8 @@ KERNEL_SOURCES = {"select_count": ["select.cu", "internal.cuh"], "select_bound":
                   "join_levels": ["join.cu", "internal.cuh"],
                   "join_pruned_levels": ["join.cu", "internal.cuh"],
                   "select_scatter": ["select.cu", "internal.cuh"],
-                  "sort_warp": ["segsort.cu"], "sort_cta": ["segsort.cu"], "sort_gather": ["segsort.cu"],
-                  "sort_msd": ["segsort.cu"], "sort_bucket": ["segsort.cu"], "sort_all": ["segsort.cu"],
+                  "sort_warp": ["segsort.cu"], "sort_cta": ["segsort.cu"], "sort_long_gather": ["segsort.cu"],
+                  "sort_long_scatter": ["segsort.cu"], "sort_bucket": ["segsort.cu"], "sort_all": ["segsort.cu"],
                   "scatter": ["radix_sort.cu"]}
 
 
@@ -267,7 +267,7 @@ def algorithmic_bytes(stats, F, Q, seg_sizes):
     internal = (nodes - stats["leaves_visited"]) * node + whole * 16
     seg = np.asarray(seg_sizes, dtype=np.int64)
     in_range = lambda lo, hi: int(seg[(seg >= lo) & (seg <= hi)].sum())
-    warp_ids, cta_ids, large_ids = in_range(2, 256), in_range(257, 40960), in_range(40961, 1 << 62)
+    warp_ids, cta_ids, large_ids = in_range(2, 256), in_range(257, 32256), in_range(32257, 1 << 62)
     return {
         "select_count": float(traverse + Q * (16 + 3 * 4)),
         "select_bound": float(internal + Q * (16 + 3 * 4)),
@@ -275,11 +275,11 @@ def algorithmic_bytes(stats, F, Q, seg_sizes):
         "select_scatter": float(traverse + Q * (16 + 16) + hits * 8),
         "sort_warp": float(warp_ids * 8),
         "sort_cta": float(cta_ids * 8),
-        "sort_gather": float(large_ids * 8),
-        "sort_msd": float(large_ids * 16),
+        "sort_long_gather": float(large_ids * 8),
+        "sort_long_scatter": float(large_ids * 8),
         "sort_bucket": float(large_ids * 8),
         # the whole segmented sort as one span (its class kernels run side by side)
-        "sort_all": float((warp_ids + cta_ids + large_ids) * 8 + large_ids * 24),
+        "sort_all": float((warp_ids + cta_ids + large_ids) * 8 + large_ids * 16),
     }
 
 
@@ -523,7 +523,8 @@ def run_ours(args):
         breakdown[name] = entry
     # the sort's class kernels overlap on side streams, so their event times
     # are not additive: the sort counts as one unit timed by its span
-    overlapped = {"sort_warp", "sort_cta", "sort_gather", "sort_msd", "sort_bucket"} if "sort_all" in kern else set()
+    overlapped = {"sort_warp", "sort_cta", "sort_long_plan", "sort_long_gather", "sort_long_split", "sort_long_scatter",
+                  "sort_bucket"} if "sort_all" in kern else set()
     dominant = max((k for k in kern if k in algo and k not in overlapped), key=lambda k: kern[k][1])
     n_l, ms = kern[dominant]
     ms_step = ms / args.steps  # the kernel's time in one step, all its launches

@@ -7,17 +7,17 @@
 //   2..256 ids    one warp: gather into shared memory, then a bitonic network
 //                 on 1-8 keys per lane in registers (shuffles across lanes,
 //                 swaps inside a lane);
-//   257..32768  one CTA of 64-1024 threads (32 ids each), entirely in shared
+//   257..32256  one CTA of 64-1024 threads (16 or 32 ids each), entirely in shared
 //                 memory: asynchronous copies in, buckets by value (one id
 //                 each on average) counted with byte counters, and every id's
 //                 rank among its bucket's neighbours gives its place in the
 //                 output (cta_bucket_sort); ids in bands are bucketed again
 //                 through equalized buckets, and what overflows those too
 //                 (heavily repeated ids) goes to a stable LSD radix sort
-//                 (8-bit digits), or above 16384 ids to the next path;
-//   > 32768       gathered into place, partitioned by its top differing bits
-//                 into buckets of about 8K ids (MSD step through a scratch
-//                 area), each bucket then sorted like a mid-size segment.
+//                 (8-bit digits);
+//   above         cut into units for all CTAs, partitioned by value into
+//                 buckets of about 8K ids through a scratch area, each bucket
+//                 then sorted like a mid-size segment.
 // Each class runs as a persistent grid whose CTAs claim segments from an
 // atomic counter, so CTAs that drew long segments do not hold up the rest.
 // LSD passes whose digit is equal for all keys are skipped (from the AND and
@@ -33,14 +33,15 @@ namespace rt {
 namespace {
 
 constexpr int kBins = 256;
-constexpr int kItems = 16;              // keys per thread of the LSD fallback (1024 threads)
-constexpr int kCtaMax = 1024 * kItems;  // 16384: longest segment the LSD fallback takes
+constexpr int kLsdItems = 16;           // keys per thread of the LSD fallback (1024 threads); twice
+                                        // that for its longest segments
 constexpr uint32_t kSign = 0x80000000u;
 
 // The ids a CTA sort takes: 252 per warp and eight ids a lane (see the
 // transposition in cta_bucket_sort).
 constexpr int cta_ids(int threads, int items) { return threads / 32 * (items / 8) * 252; }
-constexpr int kMidMax = cta_ids(512, 32);  // longest segment below the largest class: 16128
+constexpr int kMidMax = cta_ids(512, 32);   // longest segment below the largest class: 16128
+constexpr int kCtaTop = cta_ids(1024, 32);  // longest segment of a CTA sort: 32256
 
 // Segment classes (index into the class lists).
 enum {
@@ -49,7 +50,7 @@ enum {
     C_LARGE,                          // MSD partition first
     C_COUNT
 };
-enum { HDR_SCRATCH = C_COUNT, HDR_BUCKETS, HDR_OVERSIZE, HDR_WORDS };
+enum { HDR_SCRATCH = C_COUNT, HDR_BUCKETS, HDR_OVERSIZE, HDR_UNITS, HDR_WORDS };
 
 struct SegDesc {
     int64_t src;  // offset of the input keys
@@ -70,7 +71,7 @@ __device__ __forceinline__ int class_of(int64_t n)
     if (n <= cta_ids(256, 16)) return C_CTA4K;
     if (n <= cta_ids(512, 16)) return C_CTA8K;
     if (n <= kMidMax) return C_CTA16K;
-    if (n <= cta_ids(1024, 32)) return C_CTA32K;
+    if (n <= kCtaTop) return C_CTA32K;
     return C_LARGE;
 }
 
@@ -708,27 +709,11 @@ __device__ __forceinline__ void push_crowded(SegDesc *list, unsigned long long *
         list[slot] = SegDesc{dst, dst, n, 0};
 }
 
-// The MSD path's segment list, its scratch offsets and the header counters.
-struct LongList {
-    int32_t *list;
-    int64_t *tmp;
-    unsigned long long *hdr;
-};
-
-// Lists segment seg (n ids) for the MSD path, with a scratch range of its own.
-__device__ __forceinline__ void push_large(const LongList &lg, int32_t seg, int64_t n)
-{
-    const unsigned long long slot = atomicAdd(lg.hdr + C_LARGE, 1ull);
-    lg.list[slot] = seg;
-    lg.tmp[slot] = (int64_t)atomicAdd(lg.hdr + HDR_SCRATCH, (unsigned long long)n);
-}
-
 constexpr int cta_per_sm(int threads, int items) { return (items <= 16 ? 1536 : 1024) / threads; }
 
 // One CTA per listed segment.  BUCKETS: the list holds SegDesc entries whose
 // ids sit in `scratch`; otherwise segment ids whose ids are gathered from S.
-// A segment of more than 16384 ids whose buckets overflow goes to the MSD
-// path.  CTAs claim list entries from the counter *next (zero at launch), so
+// CTAs claim list entries from the counter *next (zero at launch), so
 // a CTA that drew short segments takes more.
 template <int THREADS, int ITEMS, bool BUCKETS>
 __global__ void __launch_bounds__(THREADS, cta_per_sm(THREADS, ITEMS))
@@ -736,7 +721,7 @@ __global__ void __launch_bounds__(THREADS, cta_per_sm(THREADS, ITEMS))
                int64_t list_cap, const int64_t *__restrict__ off, SortSources S,
                const int32_t *__restrict__ scratch, int32_t *__restrict__ out,
                SegDesc *__restrict__ crowded, unsigned long long *__restrict__ n_crowded,
-               int64_t crowded_cap, LongList lg, unsigned long long *__restrict__ next)
+               int64_t crowded_cap, unsigned long long *__restrict__ next)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     using Smem = CtaSmem<THREADS, ITEMS>;
@@ -828,19 +813,16 @@ __global__ void __launch_bounds__(THREADS, cta_per_sm(THREADS, ITEMS))
             load_fields();
         }
         store_piece();
-        if (!ok && threadIdx.x == 0) {
-            if (THREADS == 1024)  // the long path follows on this class's stream
-                push_large(lg, m.seg, m.n);
-            else
-                push_crowded(crowded, n_crowded, crowded_cap, m.dst, m.n);
-        }
+        if (!ok && threadIdx.x == 0)
+            push_crowded(crowded, n_crowded, crowded_cap, m.dst, m.n);
     }
 }
 
 // Shared memory of the LSD fallback.
+template <int ITEMS>
 struct LsdSmem {
     static constexpr int W = 32;
-    uint32_t buf[1024 * kItems];
+    uint32_t buf[1024 * ITEMS];
     uint32_t wcnt[W][kBins];
     uint32_t dcount[kBins];
     uint32_t dstart[kBins];
@@ -848,7 +830,8 @@ struct LsdSmem {
 };
 
 // Block-wide AND and OR of the keys' bits; every thread gets AND ^ OR.
-__device__ __forceinline__ uint32_t block_diff(LsdSmem &sm, uint32_t a_and, uint32_t a_or)
+template <int ITEMS>
+__device__ __forceinline__ uint32_t block_diff(LsdSmem<ITEMS> &sm, uint32_t a_and, uint32_t a_or)
 {
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     a_and = __reduce_and_sync(RT_FULL, a_and);
@@ -867,10 +850,10 @@ __device__ __forceinline__ uint32_t block_diff(LsdSmem &sm, uint32_t a_and, uint
 // Ranks the keys held in registers for one LSD pass; on return pos[i] is the
 // position of key[i] in the pass's output order.  Warp w owns keys
 // [w*run, (w+1)*run), taken 32 at a time.
-template <int THREADS>
-__device__ __forceinline__ void rank_pass(LsdSmem &sm, const uint32_t (&key)[kItems],
+template <int THREADS, int ITEMS>
+__device__ __forceinline__ void rank_pass(LsdSmem<ITEMS> &sm, const uint32_t (&key)[ITEMS],
                                           int rounds, int run, int n, int shift,
-                                          uint32_t (&pos)[kItems])
+                                          uint32_t (&pos)[ITEMS])
 {
     constexpr int W = THREADS / 32;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
@@ -879,7 +862,7 @@ __device__ __forceinline__ void rank_pass(LsdSmem &sm, const uint32_t (&key)[kIt
         (&sm.wcnt[0][0])[i] = 0;
     __syncthreads();
 #pragma unroll
-    for (int i = 0; i < kItems; ++i) {
+    for (int i = 0; i < ITEMS; ++i) {
         if (i >= rounds)
             break;
         const bool ok = w * run + i * 32 + lane < n;
@@ -922,7 +905,7 @@ __device__ __forceinline__ void rank_pass(LsdSmem &sm, const uint32_t (&key)[kIt
     }
     __syncthreads();
 #pragma unroll
-    for (int i = 0; i < kItems; ++i) {
+    for (int i = 0; i < ITEMS; ++i) {
         if (i >= rounds)
             break;
         if (w * run + i * 32 + lane < n) {
@@ -932,17 +915,18 @@ __device__ __forceinline__ void rank_pass(LsdSmem &sm, const uint32_t (&key)[kIt
     }
 }
 
-// Stable LSD radix sort of n <= 16384 ids in place at ids[0 .. n).
-__device__ __forceinline__ void cta_lsd_sort(LsdSmem &sm, int32_t *__restrict__ ids, int n)
+// Stable LSD radix sort of n <= 1024 * ITEMS ids in place at ids[0 .. n).
+template <int ITEMS>
+__device__ __forceinline__ void cta_lsd_sort(LsdSmem<ITEMS> &sm, int32_t *__restrict__ ids, int n)
 {
     constexpr int THREADS = 1024, W = 32;
     const int w = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int run = ((n + W * 32 - 1) / (W * 32)) * 32;
     const int rounds = run / 32;
-    uint32_t key[kItems], pos[kItems];
+    uint32_t key[ITEMS], pos[ITEMS];
     uint32_t a_and = 0xffffffffu, a_or = 0;
 #pragma unroll
-    for (int i = 0; i < kItems; ++i) {
+    for (int i = 0; i < ITEMS; ++i) {
         key[i] = 0;
         const int p = w * run + i * 32 + lane;
         if (i < rounds && p < n) {
@@ -959,9 +943,9 @@ __device__ __forceinline__ void cta_lsd_sort(LsdSmem &sm, int32_t *__restrict__ 
     for (int shift = 0; shift <= last; shift += 8) {
         if (((diff >> shift) & 0xffu) == 0)
             continue;
-        rank_pass<THREADS>(sm, key, rounds, run, n, shift, pos);
+        rank_pass<THREADS, ITEMS>(sm, key, rounds, run, n, shift, pos);
 #pragma unroll
-        for (int i = 0; i < kItems; ++i)
+        for (int i = 0; i < ITEMS; ++i)
             if (i < rounds && w * run + i * 32 + lane < n)
                 sm.buf[pos[i]] = key[i];
         __syncthreads();
@@ -970,7 +954,7 @@ __device__ __forceinline__ void cta_lsd_sort(LsdSmem &sm, int32_t *__restrict__ 
                 ids[p] = (int32_t)(sm.buf[p] ^ kSign);
         } else {
 #pragma unroll
-            for (int i = 0; i < kItems; ++i) {
+            for (int i = 0; i < ITEMS; ++i) {
                 const int p = w * run + i * 32 + lane;
                 if (i < rounds && p < n)
                     key[i] = sm.buf[p];
@@ -980,189 +964,324 @@ __device__ __forceinline__ void cta_lsd_sort(LsdSmem &sm, int32_t *__restrict__ 
     }
 }
 
-// Segments whose buckets were crowded, sorted in place by LSD radix.
-// Persistent: the list length is read on the device.
+// Segments whose buckets were crowded, sorted in place by LSD radix: those of
+// least .. 1024 * ITEMS ids.  Persistent: the list length is read on the device.
+template <int ITEMS>
 __global__ void __launch_bounds__(1024, 1)
     k_sort_lsd(const SegDesc *__restrict__ list, const unsigned long long *__restrict__ count,
-               int64_t cap, int32_t *__restrict__ out)
+               int64_t cap, int least, int32_t *__restrict__ out)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    LsdSmem &sm = *reinterpret_cast<LsdSmem *>(smem_raw);
-    int64_t cnt = (int64_t)*count;
-    if (cnt > cap)
-        cnt = cap;
+    LsdSmem<ITEMS> &sm = *reinterpret_cast<LsdSmem<ITEMS> *>(smem_raw);
+    const int64_t cnt = list_len(count, cap);
     for (int64_t b = blockIdx.x; b < cnt; b += gridDim.x) {
         const SegDesc d = list[b];
-        if (d.n > 1024 * kItems)
-            continue;
-        cta_lsd_sort(sm, out + d.dst, d.n);
+        if (d.n >= least && d.n <= 1024 * ITEMS)
+            cta_lsd_sort(sm, out + d.dst, d.n);
     }
 }
 
-// ------------------------------------------------------------ MSD step
-// Gathers each long segment into its place in `out` (unsorted).
-__global__ void __launch_bounds__(1024)
-    k_gather_large(const int32_t *__restrict__ list, const unsigned long long *__restrict__ count,
-                   int64_t list_cap, const int64_t *__restrict__ tmp_off, int64_t scratch_cap,
-                   const int64_t *__restrict__ off, SortSources S, int32_t *__restrict__ out,
-                   unsigned long long *__restrict__ next)
+// ------------------------------------------------------------ long segments
+// A segment too long for a CTA sort is cut into units of kUnit ids that any CTA can
+// take (with a CTA per segment a batch of a few dozen windows left most SMs
+// idle), and partitioned by value into buckets a CTA sort takes:
+//   k_long_plan     per segment: the ids' range from a sample, its units;
+//   k_long_gather   per unit: ids into their place in the output (unsorted),
+//                   and counted into the segment's kBinsLong value bins;
+//   k_long_split    per segment: consecutive bins become buckets of about
+//                   kBucketIds ids, listed for the CTA sort;
+//   k_long_scatter  per unit: ids to their buckets in the scratch area.
+// Ids outside the sample's range go to the end bins.
+// 40 windows of 185K ids on average: 200 us for their whole sort, 630 us with
+// one CTA a segment for the gather and the partition; a plan batch with 800
+// such windows among 100K queries: 2.26 ms, before 2.66.
+// 4096 ids a unit: its CTA (21 or 31 KB of shared memory) fits beside the
+// persistent CTAs of the large sort classes, which leave 41 KB of an SM; units
+// of 8192 waited for those to finish and ended the sort late.
+constexpr int kUnit = 4096;
+constexpr int kBinsLong = 1024;
+constexpr int kBucketIds = 8192;
+constexpr int kSample = 2048;
+
+struct LongSeg {
+    int64_t add;     // value map: bin = (id * mult + add) >> 32, clamped
+    int32_t mult;
+    int32_t pad;
+};
+struct Unit {
+    int32_t slot;  // in the long segments' list
+    int32_t part;  // which kUnit ids of it
+};
+
+__device__ __forceinline__ int bin_of(const LongSeg &g, int id)
 {
+    const int b = (int)(((int64_t)id * g.mult + g.add) >> 32);
+    return max(0, min(kBinsLong - 1, b));
+}
+
+__global__ void __launch_bounds__(256)
+    k_long_plan(const int32_t *__restrict__ list, const unsigned long long *__restrict__ count, int64_t list_cap,
+                const int64_t *__restrict__ tmp_off, int64_t scratch_cap, const int64_t *__restrict__ off,
+                SortSources S, LongSeg *__restrict__ segs, uint32_t *__restrict__ hist, Unit *__restrict__ units,
+                int64_t unit_cap, unsigned long long *__restrict__ hdr, int32_t *__restrict__ flags)
+{
+    __shared__ int red[2][8];
+    __shared__ unsigned long long first;
     const int64_t cnt = list_len(count, list_cap);
-    __shared__ long long claim;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (;;) {
-        if (threadIdx.x == 0)
-            claim = (long long)atomicAdd(next, 1ull);
-        __syncthreads();
-        const int64_t b = claim;
-        __syncthreads();
-        if (b >= cnt)
-            break;
+    for (int64_t b = blockIdx.x; b < cnt; b += gridDim.x) {
         const int32_t i = list[b];
-        int32_t *dst = out + off[i];
-        if (tmp_off[b] + (off[i + 1] - off[i]) > scratch_cap)
-            continue;  // over the scratch capacity: reported by k_msd_partition
-        const int64_t l0 = S.off_leaf[i], l1 = leaf_end(S, i);
-        if (S.leaf + l0 != dst)
-            for (int64_t e = l0 + threadIdx.x; e < l1; e += 1024)
-                dst[e - l0] = S.leaf[e];
-        if (!S.rng)
-            continue;
-        const int64_t r0 = S.off_rng[i], r1 = S.off_rng[i + 1];
-        const int64_t nl = l1 - l0;
-        const int nrl = (int)(off[i + 1] - off[i] - nl);
-        for (int64_t r = r0 + w; r < r1; r += 32) {
-            const int2 g = S.rng[r];
-            const int e = r + 1 < r1 ? S.rng[r + 1].y : nrl;
-            for (int x = lane; x < e - g.y; x += 32)
-                dst[nl + g.y + x] = __ldg(S.tree_ids + g.x + x);
+        const int64_t n = off[i + 1] - off[i];
+        const int64_t l0 = S.off_leaf[i], nl = leaf_end(S, i) - l0;
+        const int64_t r0 = S.rng ? S.off_rng[i] : 0, nr = S.rng ? S.off_rng[i + 1] - r0 : 0;
+        int lo = INT_MAX, hi = INT_MIN;
+        for (int k = threadIdx.x; k < kSample; k += 256) {
+            if (nr > 0) {  // an id of every few runs
+                const int v = S.tree_ids[S.rng[r0 + nr * k / kSample].x];
+                lo = min(lo, v), hi = max(hi, v);
+            }
+            if (nl > 0) {
+                const int v = S.leaf[l0 + nl * k / kSample];
+                lo = min(lo, v), hi = max(hi, v);
+            }
         }
-    }
-}
-
-// One CTA per listed long segment (over 32768 ids, or over 16384 with crowded
-// buckets): partitions its keys by their top b differing bits (2^b buckets
-// of about kCtaMax/2) into the scratch area and lists every bucket for the
-// CTA sort (or, if a bucket is still too long, for the global LSD fallback).
-__global__ void __launch_bounds__(1024)
-    k_msd_partition(const int32_t *__restrict__ list, const int64_t *__restrict__ tmp_off,
-                    const unsigned long long *__restrict__ count, int64_t list_cap,
-                    int64_t scratch_cap, const int64_t *__restrict__ off,
-                    const int32_t *__restrict__ ids, int32_t *__restrict__ scratch,
-                    SegDesc *__restrict__ buckets, SegDesc *__restrict__ oversize, int64_t desc_cap,
-                    unsigned long long *__restrict__ hdr, int32_t *__restrict__ flags,
-                    unsigned long long *__restrict__ next)
-{
-    const int64_t cnt = list_len(count, list_cap);
-    __shared__ uint32_t hist[kBins], cursor[kBins];
-    __shared__ uint32_t red_and[32], red_or[32];
-    __shared__ long long claim;
-    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-    for (;;) {
-        if (threadIdx.x == 0)
-            claim = (long long)atomicAdd(next, 1ull);
-        __syncthreads();
-        const int64_t b = claim;
-        __syncthreads();
-        if (b >= cnt)
-            break;
-        const int32_t seg = list[b];
-        const int64_t o = off[seg];
-        const int64_t n = off[seg + 1] - o;
-        const int64_t t = tmp_off[b];
-        if (t + n > scratch_cap) {  // cannot happen when the scratch holds all ids
-            if (threadIdx.x == 0)
+        lo = __reduce_min_sync(RT_FULL, lo);
+        hi = __reduce_max_sync(RT_FULL, hi);
+        if ((threadIdx.x & 31) == 0) {
+            red[0][threadIdx.x >> 5] = lo;
+            red[1][threadIdx.x >> 5] = hi;
+        }
+        for (int k = threadIdx.x; k < kBinsLong; k += 256)
+            hist[b * kBinsLong + k] = 0;
+        const bool fits = tmp_off[b] + n <= scratch_cap;  // always, when the scratch holds all ids
+        const int64_t nu = fits ? (n + kUnit - 1) / kUnit : 0;
+        if (threadIdx.x == 0) {
+            first = atomicAdd(hdr + HDR_UNITS, (unsigned long long)nu);
+            if (!fits)
                 atomicOr(flags, 1);
-            continue;
-        }
-        uint32_t a_and = 0xffffffffu, a_or = 0;
-        for (int64_t p = threadIdx.x; p < n; p += 1024) {
-            const uint32_t k = (uint32_t)ids[o + p] ^ kSign;
-            a_and &= k;
-            a_or |= k;
-        }
-#pragma unroll
-        for (int d = 16; d > 0; d >>= 1) {
-            a_and &= __shfl_xor_sync(RT_FULL, a_and, d);
-            a_or |= __shfl_xor_sync(RT_FULL, a_or, d);
-        }
-        if (lane == 0) {
-            red_and[w] = a_and;
-            red_or[w] = a_or;
-        }
-        if (threadIdx.x < kBins)
-            hist[threadIdx.x] = 0;
-        __syncthreads();
-        a_and = 0xffffffffu;
-        a_or = 0;
-        for (int x = 0; x < 32; ++x) {
-            a_and &= red_and[x];
-            a_or |= red_or[x];
-        }
-        const uint32_t diff = a_and ^ a_or;
-        if (diff == 0) {  // all equal: nothing to do
-            __syncthreads();
-            continue;
-        }
-        const int hb = 31 - __clz(diff);
-        int nb_bits = 1;
-        while (nb_bits < 8 && (n >> nb_bits) > kCtaMax / 2)
-            ++nb_bits;
-        if (nb_bits > hb + 1)
-            nb_bits = hb + 1;
-        const int shift = hb + 1 - nb_bits;
-        const uint32_t mask = (1u << nb_bits) - 1u;
-        for (int64_t p = threadIdx.x; p < n; p += 1024)
-            atomicAdd(&hist[(((uint32_t)ids[o + p] ^ kSign) >> shift) & mask], 1u);
-        __syncthreads();
-        if (threadIdx.x < 32) {
-            uint32_t carry = 0;
-            for (int c = 0; c < kBins; c += 32) {
-                const uint32_t v = hist[c + lane];
-                uint32_t inc = v;
-#pragma unroll
-                for (int q = 1; q < 32; q <<= 1) {
-                    const uint32_t u = __shfl_up_sync(RT_FULL, inc, q);
-                    if (lane >= q)
-                        inc += u;
-                }
-                cursor[c + lane] = carry + inc - v;
-                carry += __shfl_sync(RT_FULL, inc, 31);
-            }
         }
         __syncthreads();
-        if (threadIdx.x < kBins && hist[threadIdx.x] > 0) {
-            const uint32_t d = threadIdx.x;
-            SegDesc s;
-            s.src = t + cursor[d];
-            s.dst = o + cursor[d];
-            s.n = (int32_t)hist[d];
-            s.pad = 0;
-            if (hist[d] <= (uint32_t)kMidMax) {
-                const unsigned long long slot = atomicAdd(hdr + HDR_BUCKETS, 1ull);
-                if ((int64_t)slot < desc_cap)
-                    buckets[slot] = s;
-                else
-                    atomicOr(flags, 2);
-            } else {
-                const unsigned long long slot = atomicAdd(hdr + HDR_OVERSIZE, 1ull);
-                if ((int64_t)slot < desc_cap)
-                    oversize[slot] = s;
-                else
-                    atomicOr(flags, 2);
-            }
+        for (int64_t u = threadIdx.x; u < nu; u += 256) {
+            if ((int64_t)first + u < unit_cap)
+                units[first + u] = Unit{(int32_t)b, (int32_t)u};
+            else
+                atomicOr(flags, 2);
         }
-        __syncthreads();
-        for (int64_t p = threadIdx.x; p < n; p += 1024) {
-            const int32_t id = ids[o + p];
-            const uint32_t pos = atomicAdd(&cursor[(((uint32_t)id ^ kSign) >> shift) & mask], 1u);
-            scratch[t + pos] = id;
+        if (threadIdx.x == 0) {
+            for (int x = 0; x < 8; ++x)
+                lo = min(lo, red[0][x]), hi = max(hi, red[1][x]);
+            const BucketMap m = bucket_map(kBinsLong, lo, hi, nullptr);
+            segs[b] = LongSeg{m.add, m.mult, 0};
         }
         __syncthreads();
     }
 }
 
-// Fallback for buckets longer than kCtaMax (heavily skewed ids): LSD radix
+// The last range of rng[0 .. nr) that starts at or before place p (ranges
+// ascend; the first starts at 0), found by the warp 32 probes at a time.
+__device__ __forceinline__ int64_t range_at(const int2 *__restrict__ rng, int64_t nr, int p, int lane)
+{
+    int64_t lo = 0, hi = nr;  // the answer is in [lo, hi)
+    while (hi - lo > 1) {
+        const int64_t step = (hi - lo + 31) / 32;
+        const int64_t q = lo + lane * step;
+        const unsigned m = __ballot_sync(RT_FULL, q < hi && rng[q].y <= p);
+        const int64_t at = lo + (31 - __clz(m)) * step;  // lane 0's probe always holds
+        hi = min(at + step, hi);
+        lo = at;
+    }
+    return lo;
+}
+
+constexpr int kLongThreads = 256;
+
+__global__ void __launch_bounds__(kLongThreads, 6)
+    k_long_gather(const int32_t *__restrict__ list, const Unit *__restrict__ units,
+                  const unsigned long long *__restrict__ n_units, int64_t unit_cap, const int64_t *__restrict__ off,
+                  SortSources S, const LongSeg *__restrict__ segs, uint32_t *__restrict__ hist,
+                  int32_t *__restrict__ out)
+{
+    __shared__ __align__(16) uint32_t buf[kUnit];
+    __shared__ uint32_t bins[kBinsLong];
+    constexpr int W = kLongThreads / 32;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t cnt = list_len(n_units, unit_cap);
+    for (int64_t u = blockIdx.x; u < cnt; u += gridDim.x) {
+        const Unit un = units[u];
+        const int32_t i = list[un.slot];
+        const int64_t o = off[i], n = off[i + 1] - o;
+        const int64_t p0 = (int64_t)un.part * kUnit, p1 = min(p0 + kUnit, n);
+        const int64_t l0 = S.off_leaf[i], nl = leaf_end(S, i) - l0, nrl = n - nl;
+        for (int k = threadIdx.x; k < kBinsLong; k += kLongThreads)
+            bins[k] = 0;
+        if (p1 > nrl) {  // leaf hits of the unit
+            const int64_t a = max(p0, nrl);
+            copy_async(buf + (a - p0), S.leaf + l0 + (a - nrl), (int)(p1 - a), threadIdx.x, kLongThreads);
+        }
+        if (p0 < nrl) {  // runs of the unit, a warp one after another
+            const int64_t r0 = S.off_rng[i], nr = S.off_rng[i + 1] - r0;
+            const int2 *rng = S.rng + r0;
+            const int end = (int)min(p1, nrl);
+            const int64_t first = range_at(rng, nr, (int)p0, lane), last = range_at(rng, nr, end - 1, lane);
+            const int per = (int)((last - first + W) / W);  // runs of a warp
+            const int64_t mine = min(first + (w + 1) * (int64_t)per, last + 1);
+            for (int64_t rb = first + w * (int64_t)per; rb < mine; rb += 32) {
+                const int2 g = rb + lane < nr ? rng[rb + lane] : make_int2(0, (int)nrl);
+                const int after = rb + 32 < nr ? rng[rb + 32].y : (int)nrl;
+                const int cnt = (int)min(mine - rb, (int64_t)32);
+                for (int j = lane >> 4; j < cnt + (lane >> 4); j += 2) {  // 16 lanes a run
+                    const int k = min(j, 31);
+                    const int lo = __shfl_sync(RT_FULL, g.x, k), st = __shfl_sync(RT_FULL, g.y, k);
+                    const int nx = __shfl_sync(RT_FULL, g.y, (k + 1) & 31);
+                    const int a = max(st, (int)p0), e = min(k < 31 ? nx : after, end);
+                    if (j < cnt && e > a)
+                        copy_async(buf + (a - (int)p0), S.tree_ids + lo + (a - st), e - a, lane & 15, 16);
+                }
+            }
+        }
+        cp_async_wait();
+        __syncthreads();
+        const LongSeg sg = segs[un.slot];
+        const int len = (int)(p1 - p0);
+        for (int p = threadIdx.x; p < len; p += kLongThreads) {
+            const int v = (int)buf[p];
+            atomicAdd(&bins[bin_of(sg, v)], 1u);
+            out[o + p0 + p] = v;
+        }
+        __syncthreads();
+        for (int k = threadIdx.x; k < kBinsLong; k += kLongThreads)
+            if (bins[k])
+                atomicAdd(hist + (int64_t)un.slot * kBinsLong + k, bins[k]);
+        __syncthreads();
+    }
+}
+
+// hist becomes the buckets' write cursors, table the bins' buckets.
+__global__ void __launch_bounds__(kBinsLong)
+    k_long_split(const int32_t *__restrict__ list, const unsigned long long *__restrict__ count, int64_t list_cap,
+                 const int64_t *__restrict__ tmp_off, int64_t scratch_cap, const int64_t *__restrict__ off,
+                 uint32_t *__restrict__ hist, uint16_t *__restrict__ table, SegDesc *__restrict__ buckets,
+                 SegDesc *__restrict__ oversize, int64_t desc_cap, unsigned long long *__restrict__ hdr,
+                 int32_t *__restrict__ flags)
+{
+    __shared__ uint32_t wsum[32], wfirst[32];
+    __shared__ uint32_t starts[kBinsLong + 1];
+    const int t = threadIdx.x;
+    const int64_t cnt = list_len(count, list_cap);
+    for (int64_t b = blockIdx.x; b < cnt; b += gridDim.x) {
+        const int32_t seg = list[b];
+        const int64_t o = off[seg], n = off[seg + 1] - o, tmp = tmp_off[b];
+        if (tmp + n > scratch_cap)
+            continue;
+        const uint32_t c = hist[b * kBinsLong + t];
+        int total;
+        const uint32_t pre = (uint32_t)block_scan_int<kBinsLong>(wsum, (int)c, &total);
+        // a bucket starts where another multiple of kBucketIds has been passed
+        starts[t] = pre;
+        __syncthreads();
+        const bool head = t == 0 || pre / kBucketIds != starts[t - 1] / kBucketIds;
+        int nb;
+        const int k = block_scan_int<kBinsLong>(wfirst, head ? 1 : 0, &nb) + (head ? 0 : -1);  // this bin's bucket
+        __syncthreads();
+        if (head)
+            starts[k] = pre;
+        if (t == 0)
+            starts[nb] = (uint32_t)n;
+        table[b * kBinsLong + t] = (uint16_t)k;
+        __syncthreads();
+        if (t < nb) {
+            const uint32_t s0 = starts[t], len = starts[t + 1] - s0;
+            hist[b * kBinsLong + t] = s0;
+            if (len > 0) {
+                const SegDesc d{tmp + s0, o + s0, (int32_t)len, 0};
+                const bool fits = len <= (uint32_t)kMidMax;
+                const unsigned long long slot = atomicAdd(hdr + (fits ? HDR_BUCKETS : HDR_OVERSIZE), 1ull);
+                if ((int64_t)slot < desc_cap)
+                    (fits ? buckets : oversize)[slot] = d;
+                else
+                    atomicOr(flags, 2);
+            }
+        }
+        __syncthreads();
+    }
+}
+
+__global__ void __launch_bounds__(kLongThreads, 6)
+    k_long_scatter(const int32_t *__restrict__ list, const Unit *__restrict__ units,
+                   const unsigned long long *__restrict__ n_units, int64_t unit_cap, const int64_t *__restrict__ off,
+                   const int64_t *__restrict__ tmp_off, const LongSeg *__restrict__ segs,
+                   uint32_t *__restrict__ cursors, const uint16_t *__restrict__ table,
+                   const int32_t *__restrict__ ids, int32_t *__restrict__ scratch)
+{
+    __shared__ int32_t buf[kUnit];
+    __shared__ uint16_t tab[kBinsLong];
+    __shared__ uint32_t cnt_[kBinsLong];   // ids per bucket, then their cursors in buf
+    __shared__ uint16_t from[kBinsLong];   // buckets' starts in buf
+    __shared__ uint32_t to[kBinsLong];     // ... and in the segment's scratch
+    __shared__ uint32_t wsum[32];
+    constexpr int PER = kUnit / kLongThreads;
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+    const int64_t total = list_len(n_units, unit_cap);
+    for (int64_t u = blockIdx.x; u < total; u += gridDim.x) {
+        const Unit un = units[u];
+        const int32_t seg = list[un.slot];
+        const int64_t o = off[seg], n = off[seg + 1] - o, tmp = tmp_off[un.slot];
+        const int64_t p0 = (int64_t)un.part * kUnit;
+        const int len = (int)min((int64_t)kUnit, n - p0);
+        const LongSeg sg = segs[un.slot];
+        const int nb = table[(int64_t)un.slot * kBinsLong + kBinsLong - 1] + 1;
+        int v[PER];
+#pragma unroll
+        for (int k = 0; k < PER; ++k) {
+            const int p = k * kLongThreads + threadIdx.x;
+            v[k] = p < len ? ids[o + p0 + p] : 0;
+        }
+        for (int k = threadIdx.x; k < kBinsLong; k += kLongThreads)
+            tab[k] = table[(int64_t)un.slot * kBinsLong + k];
+        for (int k = threadIdx.x; k < nb; k += kLongThreads)
+            cnt_[k] = 0;
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < PER; ++k)
+            if (k * kLongThreads + (int)threadIdx.x < len)
+                atomicAdd(&cnt_[tab[bin_of(sg, v[k])]], 1u);
+        __syncthreads();
+        // a few buckets a thread: places in buf, and a reservation in the scratch
+        constexpr int MINE = kBinsLong / kLongThreads;
+        const int k0 = MINE * threadIdx.x;
+        uint32_t c[MINE], mine = 0;
+#pragma unroll
+        for (int k = 0; k < MINE; ++k) {
+            c[k] = k0 + k < nb ? cnt_[k0 + k] : 0u;
+            mine += c[k];
+        }
+        int sum;
+        uint32_t at = (uint32_t)block_scan_int<kLongThreads>(wsum, (int)mine, &sum);
+#pragma unroll
+        for (int k = 0; k < MINE; ++k) {
+            if (k0 + k < nb) {
+                from[k0 + k] = (uint16_t)at;
+                cnt_[k0 + k] = at;
+                to[k0 + k] = c[k] ? atomicAdd(cursors + (int64_t)un.slot * kBinsLong + k0 + k, c[k]) : 0u;
+                at += c[k];
+            }
+        }
+        __syncthreads();
+#pragma unroll
+        for (int k = 0; k < PER; ++k)
+            if (k * kLongThreads + (int)threadIdx.x < len)
+                buf[atomicAdd(&cnt_[tab[bin_of(sg, v[k])]], 1u)] = v[k];
+        __syncthreads();
+        for (int k = w; k < nb; k += kLongThreads / 32) {  // cnt_[k] is now the run's end
+            const uint32_t f = from[k], e = cnt_[k];
+            int32_t *dst = scratch + tmp + to[k];
+            for (uint32_t p = f + lane; p < e; p += 32)
+                dst[p - f] = buf[p];
+        }
+        __syncthreads();
+    }
+}
+
+// Fallback for buckets longer than kMidMax (heavily skewed ids): LSD radix
 // sort through global memory from the bucket's scratch range to its
 // place in the output, ping-ponging between the two.
 __global__ void __launch_bounds__(256)
@@ -1274,7 +1393,7 @@ template <int THREADS, int ITEMS, bool BUCKETS>
 rtree_status launch_cta(const void *list, const unsigned long long *count, int64_t list_cap,
                         const int64_t *off, const SortSources &S, const int32_t *scratch,
                         int32_t *out, const Crowded &cr, unsigned long long *next, cudaStream_t s,
-                        const char *name, const LongList &lg = LongList{})
+                        const char *name)
 {
     if (list_cap <= 0)
         return RTREE_OK;
@@ -1288,21 +1407,32 @@ rtree_status launch_cta(const void *list, const unsigned long long *count, int64
         grid = list_cap;
     KernelTimer kt_(name, s);
     kern<<<(unsigned)grid, THREADS, bytes, s>>>(list, count, list_cap, off, S, scratch, out, cr.list,
-                                                cr.count, cr.cap, lg, next);
+                                                cr.count, cr.cap, next);
     RT_LAUNCH();
     return RTREE_OK;
 }
 
-rtree_status launch_lsd(const Crowded &cr, int32_t *out, cudaStream_t s)
+template <int ITEMS>
+rtree_status launch_lsd_of(const Crowded &cr, int least, int32_t *out, cudaStream_t s)
 {
-    if (cr.cap <= 0)
-        return RTREE_OK;
-    const size_t bytes = sizeof(LsdSmem);
-    RT_TRY(set_smem(k_sort_lsd, bytes));
+    const size_t bytes = sizeof(LsdSmem<ITEMS>);
+    RT_TRY(set_smem(k_sort_lsd<ITEMS>, bytes));
+    const int64_t grid = cr.cap < sm_count() ? cr.cap : sm_count();
     KernelTimer kt_("sort_lsd", s);
-    k_sort_lsd<<<(unsigned)sm_count(), 1024, bytes, s>>>(cr.list, cr.count, cr.cap, out);
+    k_sort_lsd<ITEMS><<<(unsigned)grid, 1024, bytes, s>>>(cr.list, cr.count, cr.cap, least, out);
     RT_LAUNCH();
     return RTREE_OK;
+}
+
+// The crowded segments of up to max_len ids.
+rtree_status launch_lsd(const Crowded &cr, int64_t max_len, int32_t *out, cudaStream_t s)
+{
+    constexpr int small = 1024 * kLsdItems;
+    static_assert(kCtaTop <= 2 * small, "the LSD fallback takes every CTA sort's segments");
+    if (cr.cap <= 0)
+        return RTREE_OK;
+    RT_TRY(launch_lsd_of<kLsdItems>(cr, 0, out, s));
+    return max_len > small ? launch_lsd_of<2 * kLsdItems>(cr, small + 1, out, s) : RTREE_OK;
 }
 
 template <int K>
@@ -1411,9 +1541,11 @@ rtree_status segmented_sort_gather(int32_t *out, const int64_t *offsets, int64_t
     // Every list length stays on the device; the launches below are sized
     // by upper bounds and read the actual lengths themselves, so the whole
     // sort is enqueued without a host round trip.
-    const int64_t max_large = total / (kMidMax + 1) + 1 < nseg ? total / (kMidMax + 1) + 1 : nseg;
+    const int64_t max_large = total / (kCtaTop + 1) + 1 < nseg ? total / (kCtaTop + 1) + 1 : nseg;
     const int64_t scratch_cap = total;
-    const int64_t desc_cap = 2 * max_large + 4 * (scratch_cap / kCtaMax) + 256;
+    // buckets: one per kBucketIds ids begun, and the last of each segment
+    const int64_t desc_cap = 2 * max_large + scratch_cap / kBucketIds + 256;
+    const int64_t unit_cap = max_large + scratch_cap / kUnit;
     DevBuf<int32_t> lists(s);
     DevBuf<int64_t> large_tmp(s);
     DevBuf<unsigned long long> hdr(s);
@@ -1443,51 +1575,67 @@ rtree_status segmented_sort_gather(int32_t *out, const int64_t *offsets, int64_t
     RT_TRY(crowded.alloc(cta_cap > 0 ? cta_cap : 1, "sort crowded list"));
     unsigned long long *n_crowded = hdr.p + HDR_WORDS;  // two counters after the header
     const Crowded cr1{crowded.p, n_crowded, cta_cap};
-    const bool long_path = total > kMidMax;  // else no segment can be long
-    // the long path's buffers (segments over 32768 ids, or crowded over 16384)
+    const bool long_path = total > kCtaTop;  // else no segment can be long
+    // the long path's buffers (segments over 32256 ids)
     DevBuf<int32_t> scratch(s);
     DevBuf<SegDesc> buckets(s), oversize(s), crowded2(s);
+    DevBuf<LongSeg> long_segs(s);
+    DevBuf<uint32_t> long_hist(s);
+    DevBuf<uint16_t> long_table(s);
+    DevBuf<Unit> units(s);
     if (long_path) {
         RT_TRY(scratch.alloc(scratch_cap, "sort scratch"));
         RT_TRY(buckets.alloc(desc_cap, "sort buckets"));
         RT_TRY(oversize.alloc(desc_cap, "sort buckets"));
         RT_TRY(crowded2.alloc(desc_cap, "sort crowded list"));
+        RT_TRY(long_segs.alloc(max_large, "sort long segments"));
+        RT_TRY(long_hist.alloc(max_large * kBinsLong, "sort long bins"));
+        RT_TRY(long_table.alloc(max_large * kBinsLong, "sort long bins"));
+        RT_TRY(units.alloc(unit_cap, "sort units"));
     }
     // Three side streams and the call's stream run the classes side by side:
-    //   side 2: the 32768-id CTA sort, then the long path (which it feeds);
-    //   side 1: the CTA sorts up to 8192 ids;
-    //   side 0: the warp sorts;
-    //   stream: the CTA sort up to 16384 ids, then (after side 1) the LSD
-    //           fallback for crowded segments of all CTA classes up to 16384.
-    // The largest kernels are enqueued first so that smaller ones fill the
-    // SMs their last CTAs leave idle.
+    //   side 2: the long path, a chain of small kernels, first to start;
+    //   stream: the 32256-id CTA sort, the largest;
+    //   side 1: the CTA sorts up to 16128 ids;
+    //   side 0: those up to 2016 ids and the warp sort;
+    // then, after all of them, the LSD fallback for crowded segments.  Larger
+    // kernels are enqueued first so that smaller ones fill the SMs their last
+    // CTAs leave idle.
     Fork fk;
     RT_TRY(fk.begin(s));
+    const cudaStream_t s0 = fk.side(0), s1 = fk.side(1), s2 = fk.side(2);
     if (long_path) {
-        const cudaStream_t s2 = fk.side(2);
-        const LongList lg{L(C_LARGE), large_tmp.p, hdr.p};
-        RT_TRY((launch_cta<1024, 32, false>(L(C_CTA32K), H(C_CTA32K), cap_of(kMidMax + 1), offsets, S, nullptr, out,
-                                        cr1, claim(0), s2, "sort_cta", lg)));
-        // Long segments: gather into place, MSD-partition into the scratch
-        // area, then sort the buckets back into place.
-        const int64_t grid = max_large < (int64_t)sms * 2 ? max_large : (int64_t)sms * 2;
+        const unsigned per_seg = (unsigned)(max_large < (int64_t)sms * 4 ? max_large : (int64_t)sms * 4);
+        const unsigned per_unit = (unsigned)(unit_cap < (int64_t)sms * 6 ? unit_cap : (int64_t)sms * 6);
         {
-            KernelTimer kt_("sort_gather", s2);
-            k_gather_large<<<(unsigned)grid, 1024, 0, s2>>>(L(C_LARGE), H(C_LARGE), max_large, large_tmp.p,
-                                                            scratch_cap, offsets, S, out, claim(6));
+            KernelTimer kt_("sort_long_plan", s2);
+            k_long_plan<<<per_seg, 256, 0, s2>>>(L(C_LARGE), H(C_LARGE), max_large, large_tmp.p, scratch_cap, offsets, S,
+                                                 long_segs.p, long_hist.p, units.p, unit_cap, hdr.p, flags);
             RT_LAUNCH();
         }
         {
-            KernelTimer kt_("sort_msd", s2);
-            k_msd_partition<<<(unsigned)grid, 1024, 0, s2>>>(
-                L(C_LARGE), large_tmp.p, H(C_LARGE), max_large, scratch_cap, offsets,
-                out, scratch.p, buckets.p, oversize.p, desc_cap,
-                hdr.p, flags, claim(7));
+            KernelTimer kt_("sort_long_gather", s2);
+            k_long_gather<<<per_unit, kLongThreads, 0, s2>>>(L(C_LARGE), units.p, H(HDR_UNITS), unit_cap, offsets, S,
+                                                             long_segs.p, long_hist.p, out);
+            RT_LAUNCH();
+        }
+        {
+            KernelTimer kt_("sort_long_split", s2);
+            k_long_split<<<per_seg, kBinsLong, 0, s2>>>(L(C_LARGE), H(C_LARGE), max_large, large_tmp.p, scratch_cap,
+                                                        offsets, long_hist.p, long_table.p, buckets.p, oversize.p,
+                                                        desc_cap, hdr.p, flags);
+            RT_LAUNCH();
+        }
+        {
+            KernelTimer kt_("sort_long_scatter", s2);
+            k_long_scatter<<<per_unit, kLongThreads, 0, s2>>>(L(C_LARGE), units.p, H(HDR_UNITS), unit_cap, offsets,
+                                                              large_tmp.p, long_segs.p, long_hist.p, long_table.p, out,
+                                                              scratch.p);
             RT_LAUNCH();
         }
         const Crowded cr2{crowded2.p, n_crowded + 1, desc_cap};
         RT_TRY((launch_cta<512, 32, true>(buckets.p, H(HDR_BUCKETS), desc_cap, nullptr, S, scratch.p, out, cr2, claim(1), s2, "sort_bucket")));
-        RT_TRY(launch_lsd(cr2, out, s2));
+        RT_TRY(launch_lsd(cr2, kMidMax, out, s2));
         {
             int64_t g2 = desc_cap < (int64_t)sms * 4 ? desc_cap : (int64_t)sms * 4;
             KernelTimer kt_("sort_global", s2);
@@ -1496,19 +1644,18 @@ rtree_status segmented_sort_gather(int32_t *out, const int64_t *offsets, int64_t
             RT_LAUNCH();
         }
     }
-    RT_TRY((launch_cta<512, 32, false>(L(C_CTA16K), H(C_CTA16K), cap_of(cta_ids(512, 16) + 1), offsets, S, nullptr, out, cr1, claim(2), s, "sort_cta")));
-    const cudaStream_t s1 = fk.side(1), s0 = fk.side(0);
+    RT_TRY((launch_cta<1024, 32, false>(L(C_CTA32K), H(C_CTA32K), cap_of(kMidMax + 1), offsets, S, nullptr, out, cr1, claim(0), s, "sort_cta")));
+    RT_TRY((launch_cta<512, 32, false>(L(C_CTA16K), H(C_CTA16K), cap_of(cta_ids(512, 16) + 1), offsets, S, nullptr, out, cr1, claim(2), s1, "sort_cta")));
     RT_TRY((launch_cta<512, 16, false>(L(C_CTA8K), H(C_CTA8K), cap_of(cta_ids(256, 16) + 1), offsets, S, nullptr, out, cr1, claim(3), s1, "sort_cta")));
     RT_TRY((launch_cta<256, 16, false>(L(C_CTA4K), H(C_CTA4K), cap_of(cta_ids(128, 16) + 1), offsets, S, nullptr, out, cr1, claim(4), s1, "sort_cta")));
-    RT_TRY((launch_cta<128, 16, false>(L(C_CTA2K), H(C_CTA2K), cap_of(cta_ids(64, 16) + 1), offsets, S, nullptr, out, cr1, claim(5), s1, "sort_cta")));
-    RT_TRY((launch_cta<64, 16, false>(L(C_CTA1K), H(C_CTA1K), cap_of(257), offsets, S, nullptr, out, cr1, claim(8), s1, "sort_cta")));
+    RT_TRY((launch_cta<128, 16, false>(L(C_CTA2K), H(C_CTA2K), cap_of(cta_ids(64, 16) + 1), offsets, S, nullptr, out, cr1, claim(5), s0, "sort_cta")));
+    RT_TRY((launch_cta<64, 16, false>(L(C_CTA1K), H(C_CTA1K), cap_of(257), offsets, S, nullptr, out, cr1, claim(8), s0, "sort_cta")));
     RT_TRY(launch_warp<8>(L(C_W8), H(C_W8), cap_of(129), offsets, S, out, s0));
     RT_TRY(launch_warp<4>(L(C_W4), H(C_W4), cap_of(65), offsets, S, out, s0));
     RT_TRY(launch_warp<2>(L(C_W2), H(C_W2), cap_of(33), offsets, S, out, s0));
     RT_TRY(launch_warp<1>(L(C_W1), H(C_W1), cap_of(2), offsets, S, out, s0));
-    RT_TRY(fk.wait(1));
-    RT_TRY(launch_lsd(cr1, out, s));
-    return fk.join();
+    RT_TRY(fk.join());
+    return launch_lsd(cr1, total, out, s);
 }
 
 rtree_status segmented_sort(int32_t *ids, const int64_t *offsets, int64_t nseg, int64_t total,
