@@ -301,8 +301,9 @@ __device__ __forceinline__ float4 load_entry_t(const float *__restrict__ mbr, in
 }
 
 // ------------------------------------------------------ host-side helpers
-// Exclusive scan; out has n+1 entries and out[n] is the total.
-rtree_status scan_exclusive(const int32_t *in, int64_t *out, int64_t n, cudaStream_t s);
+// Exclusive scan; out has n+1 entries and out[n] is the total.  most
+// (optional, int32 inputs >= 0): raised to the largest input.
+rtree_status scan_exclusive(const int32_t *in, int64_t *out, int64_t n, cudaStream_t s, int32_t *most = nullptr);
 rtree_status scan_exclusive(const uint32_t *in, uint32_t *out, int64_t n, cudaStream_t s);
 rtree_status scan_exclusive(const int64_t *in, int64_t *out, int64_t n, cudaStream_t s);
 
@@ -391,10 +392,11 @@ struct SortSources {
 // of the segments' lengths (it sizes the scratch), and segments ending past
 // out_cap (default: total) in `out` are skipped.  Offsets may be absolute
 // positions in a larger `out`, so a run of segments can be sorted on its
-// own.  Device-side capacity problems set bits in *flags.
+// own.  No segment is longer than max_len: classes of longer ones are not
+// launched.  Device-side capacity problems set bits in *flags.
 rtree_status segmented_sort_gather(int32_t *out, const int64_t *off, int64_t nseg, int64_t total,
                                    const SortSources &src, cudaStream_t s, int32_t *flags,
-                                   int64_t out_cap = -1);
+                                   int64_t out_cap = -1, int64_t max_len = INT64_MAX);
 
 // Sorts every segment ids[offsets[i] .. offsets[i+1]) ascending, in place.
 rtree_status segmented_sort(int32_t *ids, const int64_t *offsets, int64_t nseg, int64_t total,

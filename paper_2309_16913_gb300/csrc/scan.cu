@@ -51,18 +51,31 @@ __device__ __forceinline__ T block_excl_scan(T v, T &total)
     return r;
 }
 
+// Raises *most to the warp's largest value (one atomic a warp).
+__device__ __forceinline__ void raise(int32_t *most, int32_t v)
+{
+    v = __reduce_max_sync(RT_FULL, v);
+    if ((threadIdx.x & 31) == 0 && v > 0)
+        atomicMax(most, v);
+}
+
 template <typename Tin, typename Tout>
 __global__ void __launch_bounds__(kThreads) k_tile_reduce(const Tin *__restrict__ in, int64_t n,
-                                                          Tout *__restrict__ sums)
+                                                          Tout *__restrict__ sums, int32_t *__restrict__ most)
 {
     const int64_t base = (int64_t)blockIdx.x * kTile;
     Tout acc = 0;
+    Tin big = 0;
 #pragma unroll
     for (int i = 0; i < kItems; ++i) {
         int64_t k = base + i * kThreads + threadIdx.x;
-        if (k < n)
+        if (k < n) {
             acc += (Tout)in[k];
+            big = in[k] > big ? in[k] : big;
+        }
     }
+    if (most)
+        raise(most, (int32_t)big);
     Tout total;
     block_excl_scan<Tout>(acc, total);
     if (threadIdx.x == 0)
@@ -74,7 +87,7 @@ __global__ void __launch_bounds__(kThreads) k_tile_reduce(const Tin *__restrict_
 template <typename Tin, typename Tout>
 __global__ void __launch_bounds__(kThreads) k_tile_scan(const Tin *__restrict__ in, int64_t n,
                                                         const Tout *__restrict__ tile_base,
-                                                        Tout *__restrict__ out)
+                                                        Tout *__restrict__ out, int32_t *__restrict__ most)
 {
     __shared__ Tout sm[kTile];
     const int64_t base = (int64_t)blockIdx.x * kTile;
@@ -86,12 +99,15 @@ __global__ void __launch_bounds__(kThreads) k_tile_scan(const Tin *__restrict__ 
     }
     __syncthreads();
     Tout v[kItems];
-    Tout run = 0;
+    Tout run = 0, big = 0;
 #pragma unroll
     for (int i = 0; i < kItems; ++i) {
         v[i] = sm[threadIdx.x * kItems + i];
         run += v[i];
+        big = v[i] > big ? v[i] : big;
     }
+    if (most)
+        raise(most, (int32_t)big);
     Tout total;
     Tout pre = block_excl_scan<Tout>(run, total);
     const Tout tb = tile_base ? tile_base[blockIdx.x] : Tout(0);
@@ -114,7 +130,7 @@ __global__ void __launch_bounds__(kThreads) k_tile_scan(const Tin *__restrict__ 
 }
 
 template <typename Tin, typename Tout>
-rtree_status scan_impl(const Tin *in, Tout *out, int64_t n, cudaStream_t s)
+rtree_status scan_impl(const Tin *in, Tout *out, int64_t n, cudaStream_t s, int32_t *most = nullptr)
 {
     if (n <= 0) {
         RT_CUDA(cudaMemsetAsync(out, 0, sizeof(Tout), s));
@@ -126,7 +142,7 @@ rtree_status scan_impl(const Tin *in, Tout *out, int64_t n, cudaStream_t s)
     if (tiles == 1) {
         {
             KernelTimer kt_("tile_scan", s);
-            k_tile_scan<Tin, Tout><<<1, kThreads, 0, s>>>(in, n, nullptr, out);
+            k_tile_scan<Tin, Tout><<<1, kThreads, 0, s>>>(in, n, nullptr, out, most);
             RT_LAUNCH();
         }
         return RTREE_OK;
@@ -136,13 +152,13 @@ rtree_status scan_impl(const Tin *in, Tout *out, int64_t n, cudaStream_t s)
     RT_TRY(sums_scan.alloc(tiles + 1, "scan tile offsets"));
     {
         KernelTimer kt_("tile_reduce", s);
-        k_tile_reduce<Tin, Tout><<<(unsigned)tiles, kThreads, 0, s>>>(in, n, sums.p);
+        k_tile_reduce<Tin, Tout><<<(unsigned)tiles, kThreads, 0, s>>>(in, n, sums.p, most);
         RT_LAUNCH();
     }
     RT_TRY((scan_impl<Tout, Tout>(sums.p, sums_scan.p, tiles, s)));
     {
         KernelTimer kt_("tile_scan", s);
-        k_tile_scan<Tin, Tout><<<(unsigned)tiles, kThreads, 0, s>>>(in, n, sums_scan.p, out);
+        k_tile_scan<Tin, Tout><<<(unsigned)tiles, kThreads, 0, s>>>(in, n, sums_scan.p, out, nullptr);
         RT_LAUNCH();
     }
     return RTREE_OK;
@@ -150,9 +166,9 @@ rtree_status scan_impl(const Tin *in, Tout *out, int64_t n, cudaStream_t s)
 
 }  // namespace
 
-rtree_status scan_exclusive(const int32_t *in, int64_t *out, int64_t n, cudaStream_t s)
+rtree_status scan_exclusive(const int32_t *in, int64_t *out, int64_t n, cudaStream_t s, int32_t *most)
 {
-    return scan_impl<int32_t, int64_t>(in, out, n, s);
+    return scan_impl<int32_t, int64_t>(in, out, n, s, most);
 }
 rtree_status scan_exclusive(const uint32_t *in, uint32_t *out, int64_t n, cudaStream_t s)
 {

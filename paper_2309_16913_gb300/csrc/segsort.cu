@@ -35,6 +35,7 @@ namespace {
 constexpr int kBins = 256;
 constexpr int kLsdItems = 16;           // keys per thread of the LSD fallback (1024 threads); twice
                                         // that for its longest segments
+constexpr int kWarpMax = 256;           // longest segment one warp sorts
 constexpr uint32_t kSign = 0x80000000u;
 
 // The ids a CTA sort takes: 252 per warp and eight ids a lane (see the
@@ -45,7 +46,7 @@ constexpr int kCtaTop = cta_ids(1024, 32);  // longest segment of a CTA sort: 32
 
 // Segment classes (index into the class lists).
 enum {
-    C_W1 = 0, C_W2, C_W4, C_W8,       // warp sorts, 32*K ids
+    C_WARP = 0,  // warp sort
     C_CTA1K, C_CTA2K, C_CTA4K, C_CTA8K, C_CTA16K, C_CTA32K,  // CTA sorts
     C_LARGE,                          // MSD partition first
     C_COUNT
@@ -62,10 +63,7 @@ struct SegDesc {
 __device__ __forceinline__ int class_of(int64_t n)
 {
     if (n <= 1) return -1;
-    if (n <= 32) return C_W1;
-    if (n <= 64) return C_W2;
-    if (n <= 128) return C_W4;
-    if (n <= 256) return C_W8;
+    if (n <= kWarpMax) return C_WARP;
     if (n <= cta_ids(64, 16)) return C_CTA1K;
     if (n <= cta_ids(128, 16)) return C_CTA2K;
     if (n <= cta_ids(256, 16)) return C_CTA4K;
@@ -81,18 +79,23 @@ __device__ __forceinline__ int64_t leaf_end(const SortSources &S, int64_t i)
     return S.leaf_len ? S.off_leaf[i] + S.leaf_len[i] : S.off_leaf[i + 1];
 }
 
-// Segments of length 1 are written directly (class -1 otherwise).
-__global__ void k_classify(const int64_t *__restrict__ off, int64_t nseg, int32_t *__restrict__ lists,
-                           int64_t stride, int64_t *__restrict__ large_tmp,
-                           unsigned long long *__restrict__ hdr, SortSources S,
-                           int32_t *__restrict__ out, int64_t out_cap)
+// Lists every segment under its class (segments of one id are written
+// directly).  A block takes 256 segments at a time and reserves each class's
+// list entries once: with a reservation per warp the few counters, each hit by
+// every warp, took 174 us for a million segments (17 us now).
+constexpr int kClassThreads = 256;
+__global__ void __launch_bounds__(kClassThreads)
+    k_classify(const int64_t *__restrict__ off, int64_t nseg, int32_t *__restrict__ lists, int64_t stride,
+               int64_t *__restrict__ large_tmp, unsigned long long *__restrict__ hdr, SortSources S,
+               int32_t *__restrict__ out, int64_t out_cap)
 {
-    const int lane = threadIdx.x & 31;
+    constexpr int W = kClassThreads / 32;
+    __shared__ uint32_t before[W][C_COUNT];  // entries of the warps before
+    __shared__ unsigned long long base[C_COUNT];
+    const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
     const unsigned lt = lanemask_lt();
-    const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
-    const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
-    for (int64_t b = warp * 32; b < nseg; b += nwarps * 32) {
-        const int64_t i = b + lane;
+    for (int64_t b = blockIdx.x * (int64_t)kClassThreads; b < nseg; b += (int64_t)gridDim.x * kClassThreads) {
+        const int64_t i = b + threadIdx.x;
         int64_t len = i < nseg ? off[i + 1] - off[i] : 0;
         // a segment whose output or sources reach past a buffer's capacity is
         // skipped (the caller sees the totals exceed the capacities)
@@ -109,22 +112,34 @@ __global__ void k_classify(const int64_t *__restrict__ off, int64_t nseg, int32_
                 v = S.tree_ids[S.rng[S.off_rng[i]].x];
             out[off[i]] = v;
         }
+        unsigned mine = 0;  // the lanes of this one's class
         for (int c = 0; c < C_COUNT; ++c) {
             const unsigned m = __ballot_sync(RT_FULL, cls == c);
-            if (!m)
-                continue;
-            const int leader = __ffs(m) - 1;
-            unsigned long long base = 0;
-            if (lane == leader)
-                base = atomicAdd(hdr + c, (unsigned long long)__popc(m));
-            base = __shfl_sync(RT_FULL, base, leader);
-            if (cls == c) {
-                const int64_t slot = (int64_t)base + __popc(m & lt);
-                lists[c * stride + slot] = (int32_t)i;
-                if (c == C_LARGE)
-                    large_tmp[slot] = (int64_t)atomicAdd(hdr + HDR_SCRATCH, (unsigned long long)len);
-            }
+            if (lane == 0)
+                before[w][c] = __popc(m);
+            if (cls == c)
+                mine = m;
         }
+        __syncthreads();
+        if (threadIdx.x < C_COUNT) {
+            const int c = threadIdx.x;
+            uint32_t sum = 0;
+            for (int x = 0; x < W; ++x) {
+                const uint32_t k = before[x][c];
+                before[x][c] = sum;
+                sum += k;
+            }
+            if (sum)
+                base[c] = atomicAdd(hdr + c, (unsigned long long)sum);
+        }
+        __syncthreads();
+        if (cls >= 0) {
+            const int64_t slot = (int64_t)base[cls] + before[w][cls] + __popc(mine & lt);
+            lists[cls * stride + slot] = (int32_t)i;
+            if (cls == C_LARGE)
+                large_tmp[slot] = (int64_t)atomicAdd(hdr + HDR_SCRATCH, (unsigned long long)len);
+        }
+        __syncthreads();
     }
 }
 
@@ -171,16 +186,64 @@ __device__ __forceinline__ int64_t list_len(const unsigned long long *count, int
     return c < cap ? c : cap;
 }
 
-// Bitonic sort of up to 32*K signed ids; element e = k*32 + lane (striped).
+// Bitonic sort of up to 32*K signed ids, element e = k*32 + lane (striped),
+// from sm[0 .. n) to out[0 .. n).
 template <int K>
+__device__ __forceinline__ void warp_network(const int32_t *sm, int32_t *__restrict__ out, int n, int lane)
+{
+    constexpr int N = 32 * K;
+    int v[K];
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        const int e = k * 32 + lane;
+        v[k] = e < n ? sm[e] : INT_MAX;
+    }
+#pragma unroll
+    for (int size = 2; size <= N; size <<= 1) {
+#pragma unroll
+        for (int stride = size >> 1; stride > 0; stride >>= 1) {
+            if (stride >= 32) {  // partner in the same lane, register k ^ (stride/32)
+                const int ks = stride / 32;
+#pragma unroll
+                for (int k = 0; k < K; ++k) {
+                    if (k & ks)
+                        continue;
+                    const int e = k * 32 + lane;
+                    const bool up = (e & size) == 0;
+                    const int a = v[k], b = v[k | ks];
+                    v[k] = up ? min(a, b) : max(a, b);
+                    v[k | ks] = up ? max(a, b) : min(a, b);
+                }
+            } else {  // partner in lane ^ stride, same register
+#pragma unroll
+                for (int k = 0; k < K; ++k) {
+                    const int e = k * 32 + lane;
+                    const int other = __shfl_xor_sync(RT_FULL, v[k], stride);
+                    const bool up = (e & size) == 0;
+                    const bool lower = (lane & stride) == 0;
+                    v[k] = (lower == up) ? min(v[k], other) : max(v[k], other);
+                }
+            }
+        }
+    }
+#pragma unroll
+    for (int k = 0; k < K; ++k) {
+        const int e = k * 32 + lane;
+        if (e < n)
+            out[e] = v[k];
+    }
+}
+
+// Segments of 2..kWarpMax ids, one warp each.  One kernel for all lengths
+// (each takes the network of its size): four kernels, most of them with little
+// to do, cost a small batch four launches.
 __global__ void __launch_bounds__(256) k_sort_warp(const int32_t *__restrict__ list,
                                                    const unsigned long long *__restrict__ count,
                                                    int64_t cap, const int64_t *__restrict__ off,
                                                    SortSources S, int32_t *__restrict__ out)
 {
-    constexpr int N = 32 * K;
     const int64_t cnt = list_len(count, cap);
-    __shared__ int32_t stage[8][N];
+    __shared__ int32_t stage[8][kWarpMax];
     const int lane = threadIdx.x & 31;
     int32_t *sm = stage[threadIdx.x >> 5];
     const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
@@ -190,47 +253,15 @@ __global__ void __launch_bounds__(256) k_sort_warp(const int32_t *__restrict__ l
         const int64_t o = off[seg];
         const int n = (int)(off[seg + 1] - o);
         warp_gather(sm, S, seg, n, lane);
-        int v[K];
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            const int e = k * 32 + lane;
-            v[k] = e < n ? sm[e] : INT_MAX;
-        }
+        if (n <= 32)
+            warp_network<1>(sm, out + o, n, lane);
+        else if (n <= 64)
+            warp_network<2>(sm, out + o, n, lane);
+        else if (n <= 128)
+            warp_network<4>(sm, out + o, n, lane);
+        else
+            warp_network<8>(sm, out + o, n, lane);
         __syncwarp();
-#pragma unroll
-        for (int size = 2; size <= N; size <<= 1) {
-#pragma unroll
-            for (int stride = size >> 1; stride > 0; stride >>= 1) {
-                if (stride >= 32) {  // partner in the same lane, register k ^ (stride/32)
-                    const int ks = stride / 32;
-#pragma unroll
-                    for (int k = 0; k < K; ++k) {
-                        if (k & ks)
-                            continue;
-                        const int e = k * 32 + lane;
-                        const bool up = (e & size) == 0;
-                        const int a = v[k], b = v[k | ks];
-                        v[k] = up ? min(a, b) : max(a, b);
-                        v[k | ks] = up ? max(a, b) : min(a, b);
-                    }
-                } else {  // partner in lane ^ stride, same register
-#pragma unroll
-                    for (int k = 0; k < K; ++k) {
-                        const int e = k * 32 + lane;
-                        const int other = __shfl_xor_sync(RT_FULL, v[k], stride);
-                        const bool up = (e & size) == 0;
-                        const bool lower = (lane & stride) == 0;
-                        v[k] = (lower == up) ? min(v[k], other) : max(v[k], other);
-                    }
-                }
-            }
-        }
-#pragma unroll
-        for (int k = 0; k < K; ++k) {
-            const int e = k * 32 + lane;
-            if (e < n)
-                out[o + e] = v[k];
-        }
     }
 }
 
@@ -1435,7 +1466,6 @@ rtree_status launch_lsd(const Crowded &cr, int64_t max_len, int32_t *out, cudaSt
     return max_len > small ? launch_lsd_of<2 * kLsdItems>(cr, small + 1, out, s) : RTREE_OK;
 }
 
-template <int K>
 rtree_status launch_warp(const int32_t *list, const unsigned long long *count, int64_t list_cap,
                          const int64_t *off, const SortSources &S, int32_t *out, cudaStream_t s)
 {
@@ -1446,7 +1476,7 @@ rtree_status launch_warp(const int32_t *list, const unsigned long long *count, i
     if (blocks > cap)
         blocks = cap;
     KernelTimer kt_("sort_warp", s);
-    k_sort_warp<K><<<(unsigned)blocks, 256, 0, s>>>(list, count, list_cap, off, S, out);
+    k_sort_warp<<<(unsigned)blocks, 256, 0, s>>>(list, count, list_cap, off, S, out);
     RT_LAUNCH();
     return RTREE_OK;
 }
@@ -1528,10 +1558,13 @@ struct Fork {
 }  // namespace
 
 rtree_status segmented_sort_gather(int32_t *out, const int64_t *offsets, int64_t nseg, int64_t total,
-                                   const SortSources &S, cudaStream_t s, int32_t *flags, int64_t out_cap)
+                                   const SortSources &S, cudaStream_t s, int32_t *flags, int64_t out_cap,
+                                   int64_t max_len)
 {
     if (nseg <= 0 || total <= 0)
         return RTREE_OK;
+    if (max_len > total)
+        max_len = total;
     if (out_cap < 0)
         out_cap = total;
     if (nseg >= (int64_t)INT32_MAX)
@@ -1568,14 +1601,17 @@ rtree_status segmented_sort_gather(int32_t *out, const int64_t *offsets, int64_t
     }
     auto L = [&](int c) { return lists.p + (int64_t)c * nseg; };
     auto H = [&](int c) { return hdr.p + c; };
-    // a class can hold at most total / (its smallest length) segments
-    auto cap_of = [&](int64_t min_len) { return total / min_len < nseg ? total / min_len : nseg; };
+    // a class can hold at most total / (its smallest length) segments, and
+    // none if no segment is that long
+    auto cap_of = [&](int64_t min_len) {
+        return min_len > max_len ? 0 : total / min_len < nseg ? total / min_len : nseg;
+    };
     const int64_t cta_cap = cap_of(257);
     DevBuf<SegDesc> crowded(s);
     RT_TRY(crowded.alloc(cta_cap > 0 ? cta_cap : 1, "sort crowded list"));
     unsigned long long *n_crowded = hdr.p + HDR_WORDS;  // two counters after the header
     const Crowded cr1{crowded.p, n_crowded, cta_cap};
-    const bool long_path = total > kCtaTop;  // else no segment can be long
+    const bool long_path = max_len > kCtaTop;  // else no segment can be long
     // the long path's buffers (segments over 32256 ids)
     DevBuf<int32_t> scratch(s);
     DevBuf<SegDesc> buckets(s), oversize(s), crowded2(s);
@@ -1593,6 +1629,8 @@ rtree_status segmented_sort_gather(int32_t *out, const int64_t *offsets, int64_t
         RT_TRY(long_table.alloc(max_large * kBinsLong, "sort long bins"));
         RT_TRY(units.alloc(unit_cap, "sort units"));
     }
+    if (cta_cap == 0)  // short segments only: one kernel more
+        return launch_warp(L(C_WARP), H(C_WARP), cap_of(2), offsets, S, out, s);
     // Three side streams and the call's stream run the classes side by side:
     //   side 2: the long path, a chain of small kernels, first to start;
     //   stream: the 32256-id CTA sort, the largest;
@@ -1650,12 +1688,9 @@ rtree_status segmented_sort_gather(int32_t *out, const int64_t *offsets, int64_t
     RT_TRY((launch_cta<256, 16, false>(L(C_CTA4K), H(C_CTA4K), cap_of(cta_ids(128, 16) + 1), offsets, S, nullptr, out, cr1, claim(4), s1, "sort_cta")));
     RT_TRY((launch_cta<128, 16, false>(L(C_CTA2K), H(C_CTA2K), cap_of(cta_ids(64, 16) + 1), offsets, S, nullptr, out, cr1, claim(5), s0, "sort_cta")));
     RT_TRY((launch_cta<64, 16, false>(L(C_CTA1K), H(C_CTA1K), cap_of(257), offsets, S, nullptr, out, cr1, claim(8), s0, "sort_cta")));
-    RT_TRY(launch_warp<8>(L(C_W8), H(C_W8), cap_of(129), offsets, S, out, s0));
-    RT_TRY(launch_warp<4>(L(C_W4), H(C_W4), cap_of(65), offsets, S, out, s0));
-    RT_TRY(launch_warp<2>(L(C_W2), H(C_W2), cap_of(33), offsets, S, out, s0));
-    RT_TRY(launch_warp<1>(L(C_W1), H(C_W1), cap_of(2), offsets, S, out, s0));
+    RT_TRY(launch_warp(L(C_WARP), H(C_WARP), cap_of(2), offsets, S, out, s0));
     RT_TRY(fk.join());
-    return launch_lsd(cr1, total, out, s);
+    return launch_lsd(cr1, max_len, out, s);
 }
 
 rtree_status segmented_sort(int32_t *ids, const int64_t *offsets, int64_t nseg, int64_t total,

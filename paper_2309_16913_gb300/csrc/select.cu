@@ -906,11 +906,11 @@ rtree_status range_select_bounded(const rtree *t, const float4 *queries, int64_t
     RT_TRY(cnt.alloc(Q, "select counts"));
     RT_TRY(cnt_leaf.alloc(Q, "select counts"));
     RT_TRY(cnt_rng.alloc(Q, "select counts"));
-    RT_TRY(flags.alloc(2, "select flags"));  // [0] select passes, [1] sort
+    RT_TRY(flags.alloc(3, "select flags"));  // [0] select passes, [1] sort, [2] the longest result
     RT_TRY(ctr.alloc(2, "select work counters"));
     RT_TRY(off_leaf.alloc(Q + 1, "select offsets"));
     RT_TRY(off_rng.alloc(Q + 1, "select offsets"));
-    RT_CUDA(cudaMemsetAsync(flags.p, 0, 2 * sizeof(int32_t), s));
+    RT_CUDA(cudaMemsetAsync(flags.p, 0, 3 * sizeof(int32_t), s));
     RT_CUDA(cudaMemsetAsync(ctr.p, 0, 2 * sizeof(unsigned long long), s));
     if (order == RTREE_ORDER_HILBERT) {
         RT_TRY(perm.alloc(Q, "query order"));
@@ -961,21 +961,23 @@ rtree_status range_select_bounded(const rtree *t, const float4 *queries, int64_t
     so.counts = cnt.p;            // exact ids per query
     so.counts_leaf = cnt_leaf.p;  // exact leaf hits (the bounds are scanned already)
     RT_TRY(launch(PASS_DESC, t, queries, Q, so, ctr.p + 1, flags.p, s));
-    RT_TRY(scan_exclusive(cnt.p, off.p, Q, s));
-    // host read 2 of 2: the total (it sizes the result and is returned)
-    int64_t total = 0;
+    RT_TRY(scan_exclusive(cnt.p, off.p, Q, s, flags.p + 2));
+    // host read 2 of 2: the total (it sizes the result and is returned) and the
+    // longest result (it says which sort classes are needed)
+    int64_t total = 0, longest = 0;
     {
         PostList pl{};
         pl.src[0] = off.p + Q;
         pl.words[0] = 2;
         pl.at[0] = 0;
         pl.src[1] = flags.p;
-        pl.words[1] = 1;
+        pl.words[1] = 3;
         pl.at[1] = 2;
         pl.n = 2;
-        uint32_t w[3];
-        RT_TRY(read_words(pl, s, w, 3));
+        uint32_t w[5];
+        RT_TRY(read_words(pl, s, w, 5));
         total = word64(w);
+        longest = (int32_t)w[4];
         if (w[2])
             return fail(RTREE_EINTERNAL, "select descriptor pass reported device flags 0x%x", w[2]);
     }
@@ -988,7 +990,7 @@ rtree_status range_select_bounded(const rtree *t, const float4 *queries, int64_t
     src.rng = rng.p;
     src.off_rng = off_rng.p;
     src.tree_ids = t->ids;
-    RT_TRY(segmented_sort_gather(ids.p, off.p, Q, total, src, s, flags.p + 1));
+    RT_TRY(segmented_sort_gather(ids.p, off.p, Q, total, src, s, flags.p + 1, -1, longest));
     // the sort runs on in the order of s; its flags reach the result's status
     RT_TRY(post_result_status(flags.p, s, res));
     res->total = total;
