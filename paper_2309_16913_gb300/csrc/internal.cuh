@@ -342,10 +342,29 @@ struct SelIO {
     const uint32_t *order;
 };
 
+// Large queries (warp per query, sorted).  BOUND lists the queries with many
+// leaves to visit and writes counts[q] = -1 - (place in the list); the
+// large-query kernels make their descriptors, and DESC only reports their
+// counts.  (Not part of SelIO: the descriptor pass without large queries ran 5%
+// slower with these fields among its arguments.)
+struct LargeIO {
+    int32_t *list;               // the listed queries; null: none are listed
+    unsigned long long *n;       // [0] queries listed, [1] tasks reserved for them
+    int64_t cap, task_cap;       // of the list and of the tasks
+    int leaves;                  // a query is large from this many leaves to visit
+    int parent_base;             // first node of the level above the leaves
+    int32_t *hits;               // DESC: leaf hits of each listed query,
+    unsigned long long *runs;    // and its {runs: high half, ids in them}
+    unsigned long long *tasks;   // {place in the list, node}
+    unsigned long long *n_tasks;
+    const int64_t *total;        // DESC: the batch's leaf-hit slots; the listed queries are
+    int64_t budget;              // treated apart only if there are fewer than budget
+};
+
 // Caller-owned buffers for a select enqueued without host synchronization
 // (q = number of queries): per-query counts [q], offsets [q+1], the leaf-hit,
 // range and id outputs with their capacities, work-queue cursors [2q],
-// flags [2] (select, sort) and work counters [2].  After the stream finishes,
+// flags [2] (select, sort) and work counters [4].  After the stream finishes,
 // off[q], off_leaf[q] and off_rng[q] hold the totals; a total above its
 // capacity means the outputs are incomplete.
 struct SelectBuffers {
@@ -360,6 +379,10 @@ struct SelectBuffers {
     int32_t *cursors;
     int32_t *flags;
     unsigned long long *ctr;
+    int32_t *large;              // [large_cap] large queries, warp per query
+    unsigned long long *large_cur;  // [2 * large_cap + 1] their cursors, the number of tasks
+    unsigned long long *tasks;   // [task_cap]
+    int64_t large_cap, task_cap;
     unsigned long long *wq_ctl;  // 3 words, work-queue mapping
     unsigned long long *wq_items;
     long long wq_cap;

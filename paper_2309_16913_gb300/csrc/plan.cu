@@ -91,6 +91,9 @@ rtree_status allocate(rtree_plan *p)
     const int64_t LC = 2 * C + 4 * (int64_t)p->tree->fanout * Q;
     p->leaf_cap = LC;
     const long long wq_cap = Q + (Q > (1 << 20) ? Q : (1 << 20));
+    // large queries whose traversal is shared out; those past these limits are
+    // walked by one warp each
+    const int64_t large_cap = Q < 16384 ? Q : 16384, task_cap = 1 << 18;
     struct Piece {
         void **dst;
         size_t bytes;
@@ -109,7 +112,10 @@ rtree_status allocate(rtree_plan *p)
         {reinterpret_cast<void **>(&b.ids), (size_t)C * 4},
         {reinterpret_cast<void **>(&b.cursors), (size_t)Q * 8},
         {reinterpret_cast<void **>(&b.flags), 8},
-        {reinterpret_cast<void **>(&b.ctr), 16},
+        {reinterpret_cast<void **>(&b.ctr), 32},
+        {reinterpret_cast<void **>(&b.large), (size_t)large_cap * 4},
+        {reinterpret_cast<void **>(&b.large_cur), (size_t)(2 * large_cap + 1) * 8},
+        {reinterpret_cast<void **>(&b.tasks), (size_t)task_cap * 8},
         {reinterpret_cast<void **>(&b.wq_ctl), 24},
         {reinterpret_cast<void **>(&b.wq_items), (size_t)wq_cap * 8},
     };
@@ -137,6 +143,8 @@ rtree_status allocate(rtree_plan *p)
     }
     b.rng_cap = b.ids_cap = C;
     b.leaf_cap = LC;
+    b.large_cap = large_cap;
+    b.task_cap = task_cap;
     b.wq_cap = wq_cap;
     RT_CUDA(cudaHostAlloc(reinterpret_cast<void **>(&p->host), 64, cudaHostAllocMapped | cudaHostAllocPortable));
     memset(p->host, 0, 64);

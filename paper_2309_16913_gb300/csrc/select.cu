@@ -54,8 +54,23 @@ constexpr int kThreads = kWarps * 32;
 // child that is not inside the query is not visited but reserves F slots (an
 // upper bound on its hits); whole subtrees are counted exactly.  It sizes a
 // descriptor pass whose leaf-hit slots are such bounds.
-enum { PASS_COUNT = 0, PASS_SCATTER = 1, PASS_DESC = 2, PASS_BOUND = 3 };
+// PASS_DESC_LARGE names DESC beside large queries where a kernel is picked.
+enum { PASS_COUNT = 0, PASS_SCATTER = 1, PASS_DESC = 2, PASS_BOUND = 3, PASS_DESC_LARGE = 4 };
 enum { FLAG_STACK = 1, FLAG_COUNT_MISMATCH = 2, FLAG_TIMEOUT = 4 };
+// Leaves to visit from which a query is large, in batches that leave warps
+// without a query and in larger ones (see k_large_desc).
+constexpr int kLargeFew = 32, kLargeMany = 160;
+constexpr int64_t kFewQueries = 8192;
+constexpr int64_t kSharedQueries = 1 << 18;  // captured batches up to this size are prepared for large queries
+inline int large_leaves(int64_t Q) { return Q < kFewQueries ? kLargeFew : kLargeMany; }
+// A batch with more leaves to visit than this keeps every warp busy past the
+// walk of a large query: sharing those out would only cost (2% of a million
+// queries' select).
+inline int64_t large_budget(int F) { return (int64_t)F * kLargeMany * sm_count() * 48; }
+__device__ __forceinline__ bool treat_large(const LargeIO &lg)
+{
+    return __ldg(lg.total) < lg.budget;
+}
 
 // Copies ids[lo, hi) to out[0, hi-lo) with the whole warp.
 __device__ __forceinline__ void warp_copy(int32_t *__restrict__ out,
@@ -425,12 +440,14 @@ constexpr int select_min_blocks(int F, int pass)
 }
 
 // Warp per query: each warp takes the next query from a counter and walks
-// its whole subtree.
-template <int F, int LAYOUT, int PASS>
+// its whole subtree.  LARGE (DESC only): listed large queries are left out and
+// their counts reported; an instance of its own, because at F = 64 the test
+// costs the descriptor pass registers it does not have (2.59 -> 2.72 ms).
+template <int F, int LAYOUT, int PASS, bool LARGE = false>
 __global__ void __launch_bounds__(kThreads, select_min_blocks(F, PASS))
     k_select(TreeDev t, const float4 *__restrict__ queries, int64_t Q, SelIO io,
              unsigned long long *__restrict__ next_query, int32_t *__restrict__ flags, int cap,
-             unsigned long long *__restrict__ stats)
+             unsigned long long *__restrict__ stats, LargeIO lg)
 {
     constexpr int G = F < 32 ? F : 32;
     extern __shared__ int32_t smem[];
@@ -439,6 +456,7 @@ __global__ void __launch_bounds__(kThreads, select_min_blocks(F, PASS))
     const int grp = lane / G, sub = lane % G;
     const unsigned lt = lanemask_lt();
     const LeafPart lp = PASS == PASS_DESC || PASS == PASS_BOUND ? leaf_part_of(t) : LeafPart{-1, 0, false};
+    const bool large = LARGE && treat_large(lg);
 
     for (;;) {
         unsigned long long qi = 0;
@@ -451,6 +469,20 @@ __global__ void __launch_bounds__(kThreads, select_min_blocks(F, PASS))
             qi = __ldg(io.order + qi);
         const float4 q = __ldg(queries + qi);
         const Seg sg = seg_of(io, PASS, (int64_t)qi);
+        if (LARGE && large) {
+            const int slot = -1 - io.counts[qi];
+            if (slot >= 0) {  // a large query, done by now
+                if (lane == 0) {
+                    const unsigned long long r = lg.runs[slot];
+                    const int nl = lg.hits[slot];
+                    if (nl > sg.llim - sg.lbase || (int64_t)(r >> 32) != sg.rlim - sg.rbase)
+                        atomicOr(flags, FLAG_COUNT_MISMATCH);
+                    io.counts[qi] = nl + (int32_t)(r & 0xffffffffull);
+                    io.counts_leaf[qi] = nl;
+                }
+                continue;
+            }
+        }
         Walk wk{0, 0, 0, 0, 0, false};
         int top = 0;
         if (t.nodes > 0) {
@@ -479,6 +511,17 @@ __global__ void __launch_bounds__(kThreads, select_min_blocks(F, PASS))
                     io.counts_leaf[qi] = (int32_t)wk.lcur;
                 if (io.counts_rng)
                     io.counts_rng[qi] = (int32_t)wk.rcur;
+                if (PASS == PASS_BOUND && lg.list && wk.lcur >= lg.leaves * F) {
+                    // at most 32/G nodes a step were visited, so that many tasks suffice
+                    const unsigned long long need = (unsigned long long)steps * (32 / G);
+                    if ((int64_t)(atomicAdd(lg.n + 1, need) + need) <= lg.task_cap) {
+                        const unsigned long long slot = atomicAdd(lg.n, 1ull);
+                        if ((int64_t)slot < lg.cap) {
+                            lg.list[slot] = (int32_t)qi;
+                            io.counts[qi] = -1 - (int32_t)slot;
+                        }
+                    }
+                }
             } else if (PASS == PASS_SCATTER) {
                 if (wk.cur != sg.lim - sg.base)
                     atomicOr(flags, FLAG_COUNT_MISMATCH);
@@ -712,8 +755,189 @@ __global__ void k_wq_places(const SelIO io, int64_t Q)
     }
 }
 
+// ----------------------------------------------------------- large queries
+// With one warp per query, the descriptor pass of a batch of few, large
+// queries (map windows) takes as long as the walk of the largest one, at about
+// a microsecond a leaf, while most of the GPU idles.  The queries that the
+// bound pass lists as large are shared out: k_large_expand walks each from the
+// root down to the nodes above the leaves' parents and makes every leaf-parent
+// it meets a task; k_large_desc takes the tasks, a warp each.  Output places
+// come from two cursors per query: its leaf hits, and its runs together with
+// the ids in them (one 64-bit word, so that a run's entry and its place among
+// the query's run ids are reserved at once).
+// 48 windows of 1.6% of 10M rectangles each (F = 64): 484 us in the descriptor
+// pass before, 60 us in these kernels; a plan batch with 800 such windows
+// among 100K queries 2.25 -> 1.93 ms; 1000 queries of up to 30K ids 141 -> 92 us.
+// The lines: 32 leaves is where a walk of its own (a microsecond a leaf) takes
+// as long as two kernels more; batches that fill the warps several times over
+// gain from about 160 on.
+// The runs [lo, lo + len) of the lanes of mc go to query `slot`.
+template <int F>
+__device__ __forceinline__ void large_runs(const SelIO &io, const LargeIO &lg, const Seg &sg, int64_t slot, unsigned mc, int lo, int len,
+                                           int lane, unsigned lt)
+{
+    const int before = ids_before<F>(mc, len, lane, lt);
+    const unsigned ids = __reduce_add_sync(RT_FULL, (unsigned)len);
+    unsigned long long r = 0;
+    if (lane == 0)
+        r = atomicAdd(lg.runs + slot, ((unsigned long long)__popc(mc) << 32) | ids);
+    r = __shfl_sync(RT_FULL, r, 0);
+    const int64_t o = sg.rbase + (int64_t)(r >> 32) + __popc(mc & lt);
+    if (((mc >> lane) & 1u) && o < sg.rlim && o < io.rng_cap)
+        io.rng_out[o] = make_int2(lo, (int)(r & 0xffffffffull) + before);
+}
+
+__global__ void __launch_bounds__(kThreads)
+    k_large_expand(TreeDev t, const float4 *__restrict__ queries, SelIO io, LargeIO lg,
+                   int32_t *__restrict__ flags, int cap)
+{
+    extern __shared__ int32_t smem[];
+    const int lane = threadIdx.x & 31;
+    int32_t *st = smem + (threadIdx.x >> 5) * cap;
+    const unsigned lt = lanemask_lt();
+    const int64_t nwarps = (int64_t)gridDim.x * kWarps;
+    const int64_t n = treat_large(lg) ? min((int64_t)lg.n[0], lg.cap) : 0;
+    for (int64_t slot = blockIdx.x * (int64_t)kWarps + (threadIdx.x >> 5); slot < n; slot += nwarps) {
+        const int64_t qi = lg.list[slot];
+        const float4 q = __ldg(queries + qi);
+        const Seg sg = seg_of(io, PASS_DESC, qi);
+        int top = 1;
+        if (lane == 0)
+            st[0] = 0;
+        if (lg.parent_base == 0) {  // the root is a leaf-parent
+            top = 0;
+            if (lane == 0)
+                lg.tasks[atomicAdd(lg.n_tasks, 1ull)] = (unsigned long long)slot;
+        }
+        __syncwarp();
+        for (int steps = 0; top > 0; ++steps) {
+            const int node = st[--top];
+            __syncwarp();
+            const int4 m = __ldg(t.meta + node);
+            const bool to_tasks = m.x >= lg.parent_base;  // the children are leaf-parents
+            for (int j0 = 0; j0 < m.y; j0 += 32) {
+                const int j = j0 + lane;
+                const float4 b = j < m.y ? load_entry(t.mbr, t.layout, t.fanout, node, j) : empty_box();
+                const bool hit = j < m.y && meets(b, q);
+                const bool cont = hit && inside(b, q), go = hit && !cont;
+                const unsigned mp = __ballot_sync(RT_FULL, go), mc = __ballot_sync(RT_FULL, cont);
+                if (mp && to_tasks) {
+                    unsigned long long pos = 0;
+                    if (lane == 0)
+                        pos = atomicAdd(lg.n_tasks, (unsigned long long)__popc(mp));
+                    pos = __shfl_sync(RT_FULL, pos, 0) + __popc(mp & lt);
+                    if (go && (int64_t)pos < lg.task_cap)
+                        lg.tasks[pos] = (unsigned long long)slot | ((unsigned long long)(m.x + j) << 32);
+                } else if (mp) {
+                    const int pos = top + __popc(mp & lt);
+                    if (go && pos < cap)
+                        st[pos] = m.x + j;
+                    top += __popc(mp);
+                }
+                if (mc) {
+                    int4 cm = make_int4(0, 0, 0, 0);
+                    if (cont)
+                        cm = __ldg(t.meta + m.x + j);
+                    large_runs<1>(io, lg, sg, slot, mc, cm.z, cm.w - cm.z, lane, lt);
+                }
+            }
+            __syncwarp();
+            if (top > cap || steps > t.nodes) {  // cannot happen; guarded anyway
+                if (lane == 0)
+                    atomicOr(flags, FLAG_STACK);
+                break;
+            }
+        }
+    }
+}
+
+constexpr int kHitStage = 256;
+
+template <int F, int LAYOUT>
+__global__ void __launch_bounds__(kThreads)
+    k_large_desc(TreeDev t, const float4 *__restrict__ queries, SelIO io, LargeIO lg)
+{
+    constexpr int G = F < 32 ? F : 32;  // lanes of a leaf
+    constexpr int K = 32 / G;           // leaves a step
+    constexpr int C = F / G;            // entries a lane
+    __shared__ int32_t s_hits[kWarps][kHitStage];
+    __shared__ int32_t s_leaves[kWarps][F < 32 ? 32 : F];
+    const int lane = threadIdx.x & 31;
+    int32_t *hits = s_hits[threadIdx.x >> 5], *leaves = s_leaves[threadIdx.x >> 5];
+    const int grp = lane / G, sub = lane % G;
+    const unsigned lt = lanemask_lt();
+    const LeafPart lp = leaf_part_of(t);
+    const int64_t nwarps = (int64_t)gridDim.x * kWarps;
+    const int64_t n = min((int64_t)*lg.n_tasks, lg.task_cap);
+    for (int64_t k = blockIdx.x * (int64_t)kWarps + (threadIdx.x >> 5); k < n; k += nwarps) {
+        const unsigned long long task = lg.tasks[k];
+        const int64_t slot = (int64_t)(task & 0xffffffffull);
+        const int node = (int)(task >> 32);
+        const int64_t qi = lg.list[slot];
+        const float4 q = __ldg(queries + qi);
+        const Seg sg = seg_of(io, PASS_DESC, qi);
+        const int4 m = __ldg(t.meta + node);
+        __syncwarp();  // the previous task's lists are done with
+        int todo = 0;
+#pragma unroll
+        for (int j0 = 0; j0 < F; j0 += 32) {
+            const int j = j0 + lane;
+            const float4 b = j < m.y ? load_entry_t<F, LAYOUT>(t.mbr, node, j) : empty_box();
+            const bool hit = j < m.y && meets(b, q);
+            const bool cont = hit && inside(b, q), go = hit && !cont;
+            const unsigned mp = __ballot_sync(RT_FULL, go), mc = __ballot_sync(RT_FULL, cont);
+            if (go)
+                leaves[todo + __popc(mp & lt)] = m.x + j;
+            todo += __popc(mp);
+            if (mc) {
+                int lo = 0, len = 0;
+                if (cont)
+                    leaf_span<F>(t, lp, m.x + j, lo, len);
+                large_runs<F>(io, lg, sg, slot, mc, lo, len, lane, lt);
+            }
+        }
+        __syncwarp();
+        int held = 0;
+        auto flush = [&] {
+            const int64_t at = sg.lbase + reserve(lg.hits + slot, held, lane);
+            __syncwarp();
+            for (int e = lane; e < held; e += 32)
+                if (at + e < sg.llim && at + e < io.leaf_cap)
+                    io.leaf_out[at + e] = hits[e];
+            __syncwarp();
+            held = 0;
+        };
+        for (int l0 = 0; l0 < todo; l0 += K) {
+            const bool some = l0 + grp < todo;
+            const int leaf = leaves[some ? l0 + grp : l0];
+            int first, cnt;
+            leaf_span<F>(t, lp, leaf, first, cnt);
+            float4 e[C];
+            int32_t id[C];
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                const int j = sub + c * G;
+                e[c] = load_entry_t<F, LAYOUT>(t.mbr, leaf, j);
+                id[c] = j < cnt ? __ldg(t.ids + first + j) : 0;
+            }
+#pragma unroll
+            for (int c = 0; c < C; ++c) {
+                const bool emit = some && sub + c * G < cnt && meets(e[c], q);
+                const unsigned me = __ballot_sync(RT_FULL, emit);
+                if (held + __popc(me) > kHitStage)
+                    flush();
+                if (emit)
+                    hits[held + __popc(me & lt)] = id[c];
+                held += __popc(me);
+            }
+        }
+        if (held)
+            flush();
+    }
+}
+
 using SelectKernel = void (*)(TreeDev, const float4 *, int64_t, SelIO, unsigned long long *,
-                              int32_t *, int, unsigned long long *);
+                              int32_t *, int, unsigned long long *, LargeIO);
 
 template <int F, int LAYOUT>
 SelectKernel pick_pass(int pass)
@@ -721,7 +945,8 @@ SelectKernel pick_pass(int pass)
     return pass == PASS_COUNT     ? k_select<F, LAYOUT, PASS_COUNT>
            : pass == PASS_SCATTER ? k_select<F, LAYOUT, PASS_SCATTER>
            : pass == PASS_BOUND   ? k_select<F, LAYOUT, PASS_BOUND>
-                                  : k_select<F, LAYOUT, PASS_DESC>;
+           : pass == PASS_DESC_LARGE ? k_select<F, LAYOUT, PASS_DESC, true>
+                                     : k_select<F, LAYOUT, PASS_DESC>;
 }
 
 template <int F>
@@ -755,7 +980,7 @@ const char *pass_name(int pass)
 
 rtree_status launch(int pass, const rtree *t, const float4 *q, int64_t Q, const SelIO &io,
                     unsigned long long *ctr, int32_t *flags, cudaStream_t s,
-                    unsigned long long *stats = nullptr)
+                    unsigned long long *stats = nullptr, const LargeIO &lg = LargeIO{})
 {
     SelectKernel kern = pick(t->fanout, t->layout, pass);
     if (!kern)
@@ -773,7 +998,7 @@ rtree_status launch(int pass, const rtree *t, const float4 *q, int64_t Q, const 
     if (grid > need)
         grid = need;
     KernelTimer kt_(pass_name(pass), s);
-    kern<<<(unsigned)grid, kThreads, smem, s>>>(t->view(), q, Q, io, ctr, flags, cap, stats);
+    kern<<<(unsigned)grid, kThreads, smem, s>>>(t->view(), q, Q, io, ctr, flags, cap, stats, lg);
     RT_LAUNCH();
     return RTREE_OK;
 }
@@ -871,6 +1096,71 @@ rtree_status launch_wq(int pass, const rtree *t, const float4 *q, int64_t Q, con
     return RTREE_OK;
 }
 
+using LargeKernel = void (*)(TreeDev, const float4 *, SelIO, LargeIO);
+
+template <int F>
+LargeKernel pick_large_layout(int layout)
+{
+    return layout == RTREE_LAYOUT_AOS    ? k_large_desc<F, RTREE_LAYOUT_AOS>
+           : layout == RTREE_LAYOUT_LOHI ? k_large_desc<F, RTREE_LAYOUT_LOHI>
+                                         : k_large_desc<F, RTREE_LAYOUT_SOA>;
+}
+
+LargeKernel pick_large(int F, int layout)
+{
+    switch (F) {
+    case 4: return pick_large_layout<4>(layout);
+    case 8: return pick_large_layout<8>(layout);
+    case 16: return pick_large_layout<16>(layout);
+    case 32: return pick_large_layout<32>(layout);
+    case 64: return pick_large_layout<64>(layout);
+    case 128: return pick_large_layout<128>(layout);
+    default: return nullptr;
+    }
+}
+
+// The descriptors of the listed large queries (at most n_large of them and
+// n_tasks tasks).  io: as for DESC; lg: as filled by BOUND; cur: 2 * n_large +
+// 1 words for the cursors, which it sets in lg and zeroes here.
+rtree_status launch_large(const rtree *t, const float4 *q, const SelIO &io, LargeIO &lg, int64_t n_large,
+                          int64_t n_tasks, unsigned long long *tasks, unsigned long long *cur, int32_t *flags,
+                          cudaStream_t s)
+{
+    LargeKernel kern = pick_large(t->fanout, t->layout);
+    if (!kern)
+        return fail(RTREE_EINVAL, "unsupported fanout %d", t->fanout);
+    lg.cap = n_large;
+    lg.task_cap = n_tasks;
+    lg.parent_base = t->levels > 1 ? (int)t->level_base[t->levels - 2] : 0;
+    lg.runs = cur;
+    lg.n_tasks = cur + n_large;
+    lg.hits = reinterpret_cast<int32_t *>(cur + n_large + 1);
+    lg.tasks = tasks;
+    const int cap = t->levels * (t->fanout > 32 ? t->fanout : 32);
+    const size_t smem = (size_t)kWarps * cap * sizeof(int32_t);
+    if (smem > 48 * 1024)
+        RT_CUDA(cudaFuncSetAttribute(k_large_expand, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem));
+    int per_sm = 0;
+    RT_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kern, kThreads, 0));
+    const int64_t full = (int64_t)(per_sm > 0 ? per_sm : 1) * sm_count();
+    auto grid = [&](int64_t items) {
+        const int64_t b = (items + kWarps - 1) / kWarps;
+        return (unsigned)(b < 1 ? 1 : b < full ? b : full);
+    };
+    RT_CUDA(cudaMemsetAsync(cur, 0, (2 * n_large + 1) * sizeof(unsigned long long), s));
+    {
+        KernelTimer kt_("select_large_expand", s);
+        k_large_expand<<<grid(n_large), kThreads, smem, s>>>(t->view(), q, io, lg, flags, cap);
+        RT_LAUNCH();
+    }
+    {
+        KernelTimer kt_("select_large", s);
+        kern<<<grid(n_tasks), kThreads, 0, s>>>(t->view(), q, io, lg);
+        RT_LAUNCH();
+    }
+    return RTREE_OK;
+}
+
 SelIO unlimited()
 {
     SelIO io{};
@@ -890,6 +1180,8 @@ rtree_status empty_result(int64_t Q, DevBuf<int64_t> &off, cudaStream_t s, rtree
     return RTREE_OK;
 }
 
+constexpr int64_t kMostTasks = 4 << 20;
+
 // Sorted select, warp per query.  The bound pass stops above the leaves and
 // gives each query F leaf-hit slots per intersecting leaf (whole subtrees
 // exactly); the descriptor pass fills the slots and reports every query's
@@ -903,15 +1195,18 @@ rtree_status range_select_bounded(const rtree *t, const float4 *queries, int64_t
     DevBuf<unsigned long long> ctr(s);
     DevBuf<int64_t> off_leaf(s), off_rng(s);
     DevBuf<uint32_t> perm(s);
+    DevBuf<int32_t> large(s);
+    const int64_t large_cap = Q < 65536 ? Q : 65536;
     RT_TRY(cnt.alloc(Q, "select counts"));
     RT_TRY(cnt_leaf.alloc(Q, "select counts"));
     RT_TRY(cnt_rng.alloc(Q, "select counts"));
     RT_TRY(flags.alloc(3, "select flags"));  // [0] select passes, [1] sort, [2] the longest result
-    RT_TRY(ctr.alloc(2, "select work counters"));
+    RT_TRY(ctr.alloc(4, "select work counters"));  // two passes, large queries, tasks for them
+    RT_TRY(large.alloc(large_cap, "select large queries"));
     RT_TRY(off_leaf.alloc(Q + 1, "select offsets"));
     RT_TRY(off_rng.alloc(Q + 1, "select offsets"));
     RT_CUDA(cudaMemsetAsync(flags.p, 0, 3 * sizeof(int32_t), s));
-    RT_CUDA(cudaMemsetAsync(ctr.p, 0, 2 * sizeof(unsigned long long), s));
+    RT_CUDA(cudaMemsetAsync(ctr.p, 0, 4 * sizeof(unsigned long long), s));
     if (order == RTREE_ORDER_HILBERT) {
         RT_TRY(perm.alloc(Q, "query order"));
         RT_TRY(hilbert_order(t, queries, Q, perm.p, s));
@@ -921,11 +1216,19 @@ rtree_status range_select_bounded(const rtree *t, const float4 *queries, int64_t
     io.counts_leaf = cnt_leaf.p;
     io.counts_rng = cnt_rng.p;
     io.order = perm.p;
-    RT_TRY(launch(PASS_BOUND, t, queries, Q, io, ctr.p, flags.p, s));
+    LargeIO lg{};
+    lg.list = large.p;
+    lg.n = ctr.p + 2;
+    lg.cap = large_cap;
+    lg.task_cap = kMostTasks;
+    lg.leaves = large_leaves(Q);
+    lg.total = off_leaf.p + Q;
+    lg.budget = large_budget(t->fanout);
+    RT_TRY(launch(PASS_BOUND, t, queries, Q, io, ctr.p, flags.p, s, nullptr, lg));
     RT_TRY(scan_exclusive(cnt_leaf.p, off_leaf.p, Q, s));
     RT_TRY(scan_exclusive(cnt_rng.p, off_rng.p, Q, s));
     // host read 1 of 2: the sizes of the descriptor pass's outputs and the flags
-    int64_t h[2] = {0, 0};
+    int64_t h[2] = {0, 0}, n_large = 0, n_tasks = 0;
     int32_t hflags = 0;
     {
         PostList pl{};
@@ -935,15 +1238,20 @@ rtree_status range_select_bounded(const rtree *t, const float4 *queries, int64_t
         pl.src[1] = off_rng.p + Q;
         pl.words[1] = 2;
         pl.at[1] = 2;
-        pl.src[2] = flags.p;
-        pl.words[2] = 1;
+        pl.src[2] = ctr.p + 2;
+        pl.words[2] = 4;
         pl.at[2] = 4;
-        pl.n = 3;
-        uint32_t w[5];
-        RT_TRY(read_words(pl, s, w, 5));
+        pl.src[3] = flags.p;
+        pl.words[3] = 1;
+        pl.at[3] = 8;
+        pl.n = 4;
+        uint32_t w[9];
+        RT_TRY(read_words(pl, s, w, 9));
         h[0] = word64(w);
         h[1] = word64(w + 2);
-        hflags = (int32_t)w[4];
+        n_large = word64(w + 4) < large_cap ? word64(w + 4) : large_cap;
+        n_tasks = word64(w + 6) < kMostTasks ? word64(w + 6) : kMostTasks;
+        hflags = (int32_t)w[8];
     }
     if (hflags)
         return fail(RTREE_EINTERNAL, "select bound pass reported device flags 0x%x", hflags);
@@ -960,7 +1268,15 @@ rtree_status range_select_bounded(const rtree *t, const float4 *queries, int64_t
     so.order = perm.p;
     so.counts = cnt.p;            // exact ids per query
     so.counts_leaf = cnt_leaf.p;  // exact leaf hits (the bounds are scanned already)
-    RT_TRY(launch(PASS_DESC, t, queries, Q, so, ctr.p + 1, flags.p, s));
+    DevBuf<unsigned long long> tasks(s), large_cur(s);
+    int pass = PASS_DESC;
+    if (n_large > 0 && h[0] < lg.budget) {
+        RT_TRY(tasks.alloc(n_tasks, "select tasks"));
+        RT_TRY(large_cur.alloc(2 * n_large + 1, "select cursors"));
+        RT_TRY(launch_large(t, queries, so, lg, n_large, n_tasks, tasks.p, large_cur.p, flags.p, s));
+        pass = PASS_DESC_LARGE;
+    }
+    RT_TRY(launch(pass, t, queries, Q, so, ctr.p + 1, flags.p, s, nullptr, lg));
     RT_TRY(scan_exclusive(cnt.p, off.p, Q, s, flags.p + 2));
     // host read 2 of 2: the total (it sizes the result and is returned) and the
     // longest result (it says which sort classes are needed)
@@ -1428,8 +1744,11 @@ rtree_status select_enqueue(const rtree *t, const float4 *queries, int64_t Q, in
                             const SelectBuffers &b, cudaStream_t s)
 {
     const bool wq = mapping == RTREE_MAP_WORK_QUEUE;
+    // (a graph cannot ask whether there are large queries, only prepare for them)
+    const bool share_large = !wq && Q <= kSharedQueries;
+    LargeIO lg{};
     RT_CUDA(cudaMemsetAsync(b.flags, 0, 2 * sizeof(int32_t), s));
-    RT_CUDA(cudaMemsetAsync(b.ctr, 0, 2 * sizeof(unsigned long long), s));
+    RT_CUDA(cudaMemsetAsync(b.ctr, 0, 4 * sizeof(unsigned long long), s));
     if (Q == 0 || t->nodes == 0) {
         RT_CUDA(cudaMemsetAsync(b.off, 0, (Q + 1) * sizeof(int64_t), s));
         RT_CUDA(cudaMemsetAsync(b.off_leaf, 0, (Q + 1) * sizeof(int64_t), s));
@@ -1449,7 +1768,16 @@ rtree_status select_enqueue(const rtree *t, const float4 *queries, int64_t Q, in
     } else {
         // warp per query: the bound pass (stopped above the leaves) sizes the
         // leaf-hit slots; the descriptor pass reports the exact counts
-        RT_TRY(launch(PASS_BOUND, t, queries, Q, io, b.ctr, b.flags, s));
+        if (share_large) {
+            lg.list = b.large;
+            lg.n = b.ctr + 2;
+            lg.cap = b.large_cap;
+            lg.task_cap = b.task_cap;
+            lg.leaves = large_leaves(Q);
+            lg.total = b.off_leaf + Q;
+            lg.budget = large_budget(t->fanout);
+        }
+        RT_TRY(launch(PASS_BOUND, t, queries, Q, io, b.ctr, b.flags, s, nullptr, lg));
     }
     if (wq)
         RT_TRY(scan_exclusive(b.cnt, b.off, Q, s));
@@ -1471,7 +1799,9 @@ rtree_status select_enqueue(const rtree *t, const float4 *queries, int64_t Q, in
     } else {
         so.counts = b.cnt;            // exact ids per query
         so.counts_leaf = b.cnt_leaf;  // exact leaf hits (the slot bounds are scanned already)
-        RT_TRY(launch(PASS_DESC, t, queries, Q, so, b.ctr + 1, b.flags, s));
+        if (share_large)
+            RT_TRY(launch_large(t, queries, so, lg, b.large_cap, b.task_cap, b.tasks, b.large_cur, b.flags, s));
+        RT_TRY(launch(share_large ? PASS_DESC_LARGE : PASS_DESC, t, queries, Q, so, b.ctr + 1, b.flags, s, nullptr, lg));
         RT_TRY(scan_exclusive(b.cnt, b.off, Q, s));
     }
     SortSources src{};
