@@ -169,6 +169,11 @@ void timing_add_replay(const char *name, long long launches);
 //   ids : entry ids, leaves in node order, entries in slot order.
 struct Mailbox;
 
+// From this fanout on each whole subtree is a run of its own: a leaf has ids
+// enough for one copy, and what merging them adds to the descriptor pass made
+// it slower (172 -> 189 us at F=128, 100K queries of 0.01% on 2M).
+constexpr int kRunSingly = 128;
+
 struct TreeDev {
     const float *mbr;
     const int4 *meta;
@@ -179,7 +184,11 @@ struct TreeDev {
     int32_t levels;
     int32_t fanout;
     int32_t layout;
-    int32_t sorted;  // entries of every node ascend by lx
+    // Lanes that start a run of neighbouring subtrees whatever the lane before
+    // holds: the first child's lane of each node a warp tests at once, or every
+    // lane if neighbours' entries do not follow one another (a loaded tree)
+    // or the fanout is kRunSingly or more.
+    uint32_t run_first;
     // The leaf level's one short leaf: {its position among the leaves (-1:
     // none), its count, how many leaves are short}.  With at most one short
     // leaf, leaf s holds entries [s*F - (s > pos ? F - count : 0), + F or
@@ -206,6 +215,7 @@ struct rtree {
     float4 *nbox = nullptr;
     int32_t *ids = nullptr;
     int64_t *leaf_part = nullptr;  // see TreeDev::leaf_part
+    bool chained = true;  // each subtree's entries follow those of the sibling before it
     float root_mbr[4] = {0, 0, 0, 0};  // valid once root_ready (see tree_root_box)
     bool root_ready = true;
     rt::Mailbox *root_mb = nullptr;     // the build's posted root box until it is read
@@ -225,8 +235,9 @@ struct rtree {
         v.levels = levels;
         v.fanout = fanout;
         v.layout = layout;
-        v.sorted = sorted;
         v.leaf_part = leaf_part;
+        v.run_first = !chained || fanout >= rt::kRunSingly ? 0xffffffffu : fanout == 16 ? 0x00010001u : fanout == 8 ? 0x01010101u
+                      : fanout == 4 ? 0x11111111u : 1u;
         return v;
     }
 };

@@ -213,6 +213,8 @@ struct LevelInfo {
 // Structure check of loaded metadata: counts in [1, F]; an internal node's
 // children lie in the next level; leaf entries, and every node's entry range,
 // inside [0, n).
+// bad[0]: the first node that breaks the structure.  bad[1]: cleared to 0 if some
+// node's entries do not start where those of the node before it, a sibling, end.
 __global__ void k_check_meta(const int4 *__restrict__ meta, LevelInfo L, int F, int64_t n,
                              unsigned long long *__restrict__ bad)
 {
@@ -228,8 +230,13 @@ __global__ void k_check_meta(const int4 *__restrict__ meta, LevelInfo L, int F, 
             ok = ok && m.x >= L.base[e + 1] && (int64_t)m.x + m.y <= L.base[e + 2];
         else
             ok = ok && m.x >= 0 && (int64_t)m.x + m.y <= n;
-        if (!ok)
+        if (!ok) {
             atomicMin(bad, (unsigned long long)g);
+        } else if (e + 1 < L.levels) {
+            for (int64_t c = m.x; c + 1 < (int64_t)m.x + m.y; ++c)
+                if (meta[c].w != meta[c + 1].z)
+                    bad[1] = 0;
+        }
     }
 }
 
@@ -389,8 +396,8 @@ rtree_status load_payload(FILE *f, const Header &h, rtree *t, cudaStream_t s)
     L.base[h.levels] = base;
     if (h.nodes > 0) {
         DevBuf<unsigned long long> bad(s);
-        RT_TRY(bad.alloc(1, "load check flag"));
-        RT_CUDA(cudaMemsetAsync(bad.p, 0xff, sizeof(unsigned long long), s));
+        RT_TRY(bad.alloc(2, "load check flags"));
+        RT_CUDA(cudaMemsetAsync(bad.p, 0xff, 2 * sizeof(unsigned long long), s));
         {
             KernelTimer kt_("check_meta", s);
             int64_t blocks = (h.nodes + 255) / 256;
@@ -398,11 +405,12 @@ rtree_status load_payload(FILE *f, const Header &h, rtree *t, cudaStream_t s)
                                                                                    h.n, bad.p);
             RT_LAUNCH();
         }
-        unsigned long long hb = 0;
-        RT_CUDA(cudaMemcpyAsync(&hb, bad.p, sizeof(hb), cudaMemcpyDeviceToHost, s));
+        unsigned long long hb[2] = {0, 0};
+        RT_CUDA(cudaMemcpyAsync(hb, bad.p, sizeof(hb), cudaMemcpyDeviceToHost, s));
         RT_CUDA(cudaStreamSynchronize(s));
-        if (hb != ~0ull)
-            return fail(RTREE_EINVAL, "rtree_load: node %llu breaks the tree structure", hb);
+        if (hb[0] != ~0ull)
+            return fail(RTREE_EINVAL, "rtree_load: node %llu breaks the tree structure", hb[0]);
+        t->chained = hb[1] != 0;
     }
     t->fanout = h.fanout;
     t->layout = h.layout;

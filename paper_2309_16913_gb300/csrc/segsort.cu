@@ -270,7 +270,7 @@ constexpr int kHalo = 32;          // slots kept before and after the keys (a wi
 constexpr int kNet = 5;            // ids a bucket may hold for the register network
 constexpr int kCoarse = 4;         // coarse bins per thread of the equalized buckets
 constexpr int kRetry = 12;         // a bucket this full asks for equalized buckets
-constexpr int kLongRange = 512;    // longer id runs are copied by the whole CTA
+constexpr int kLongRange = 2048;   // longer id runs are copied by the whole CTA
 
 // A segment to sort: n ids of which nl are leaf hits, nr whole subtrees.
 struct Piece {

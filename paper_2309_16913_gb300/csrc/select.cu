@@ -30,8 +30,8 @@
 //   COUNT    per query: ids found, and (optionally) how many came one by one
 //            from leaves and how many whole subtrees were taken;
 //   SCATTER  writes the ids themselves in traversal order (unsorted output);
-//   DESC     writes the leaf hits and, for every whole subtree, where its run
-//            of the tree's id array starts and its place among the query's
+//   DESC     writes the leaf hits and, for every run of whole subtrees, where
+//            it starts in the tree's id array and its place among the query's
 //            run ids; the sorted output is then built by the segmented sort,
 //            which reads the runs directly;
 //   BOUND    the count pass stopped above the leaves, sizing DESC's slots.
@@ -94,7 +94,8 @@ __device__ __forceinline__ void warp_copy(int32_t *__restrict__ out,
 struct Walk {
     int32_t cur;   // ids found, warp-uniform (a query's ids fit 31 bits)
     int32_t lcur;  // of which found one by one in leaves
-    int32_t rcur;  // whole subtrees taken
+    int32_t rcur;  // runs of whole subtrees (see run_starts)
+    int32_t n_whole;  // statistics: whole subtrees (kept apart where they are merged), nodes, leaves
     unsigned long long n_visit, n_leaf;
     bool overflow;
 };
@@ -145,6 +146,31 @@ __device__ __forceinline__ int64_t reserve(int32_t *cursor, int n, int lane)
     if (lane == 0 && n > 0)
         r = atomicAdd(cursor, n);
     return __shfl_sync(RT_FULL, r, 0);
+}
+
+// Whole subtrees are taken a run at a time: neighbouring children's subtrees
+// follow one another in the id array, so the run's first lane stands for it.
+// mc: the lanes with a whole subtree.  A window holds leaves side by side, so
+// runs are several times fewer than subtrees: 1M queries on 11M sort in
+// 7.48 ms instead of 7.65 with fewer entries to read, and the unsorted copies of
+// 100K queries on 2M (F=16) take 561 us instead of 680, being longer.
+template <int F>
+__device__ __forceinline__ unsigned run_starts(const TreeDev &t, unsigned mc)
+{
+    if (F >= kRunSingly)
+        return mc;
+    return mc & (~(mc << 1) | t.run_first);
+}
+
+// The last lane of the run that starts at lane `start` of mc.
+template <int F>
+__device__ __forceinline__ int run_last(const TreeDev &t, unsigned mc, int start)
+{
+    if (F >= kRunSingly)
+        return start;
+    // the lanes after `start` that are not in mc or start a run
+    const unsigned stop = (~mc | run_starts<F>(t, mc)) & ~((2u << start) - 1u);
+    return stop ? __ffs(stop) - 2 : 31;
 }
 
 // Ids in the runs of the lower lanes of mc (len: the lane's run, 0 outside
@@ -242,7 +268,7 @@ __device__ __forceinline__ void select_step(const TreeDev &t, const float4 q, in
                     int lo;
                     leaf_span<F>(t, lp, m.x + j, lo, n);
                 }
-                wk.rcur += __popc(mc);
+                wk.rcur += __popc(run_starts<F>(t, mc));
                 wk.cur += __reduce_add_sync(RT_FULL, (unsigned)n);
             }
         }
@@ -273,11 +299,12 @@ __device__ __forceinline__ void select_step(const TreeDev &t, const float4 q, in
                     leaf_span<F>(t, lp, m.x + j, lo, cn);
                     hi = lo + cn;
                 }
-                const int64_t o = sg.rbase + wk.rcur + __popc(mc & lt);
+                const unsigned ms = run_starts<F>(t, mc);
+                const int64_t o = sg.rbase + wk.rcur + __popc(ms & lt);
                 const int place = wk.cur - wk.lcur + ids_before<F>(mc, hi - lo, lane, lt);
-                if (cont && o < sg.rlim && o < io.rng_cap)
+                if ((F >= kRunSingly ? cont : (ms >> lane) & 1u) && o < sg.rlim && o < io.rng_cap)
                     io.rng_out[o] = make_int2(lo, place);
-                wk.rcur += __popc(mc);
+                wk.rcur += __popc(ms);
                 wk.cur += __reduce_add_sync(RT_FULL, (unsigned)(hi - lo));
             }
         }
@@ -366,23 +393,27 @@ __device__ __forceinline__ void select_step(const TreeDev &t, const float4 q, in
                 lo = cm.z;
                 hi = cm.w;
             }
+            const unsigned ms = run_starts<F>(t, mc);
             if (PASS == PASS_DESC) {
-                const int64_t at = WQ ? sg.rbase + reserve(io.cur_rng + qi, __popc(mc), lane) : sg.rbase + wk.rcur;
-                const int64_t o = at + __popc(mc & lt);
+                const int64_t at = WQ ? sg.rbase + reserve(io.cur_rng + qi, __popc(ms), lane) : sg.rbase + wk.rcur;
+                const int64_t o = at + __popc(ms & lt);
                 // several warps may serve a query of the work queue: its
                 // entries get their lengths here, their places afterwards
-                const int place = WQ ? hi - lo : wk.cur - wk.lcur + ids_before<F>(mc, hi - lo, lane, lt);
-                if (cont && o < sg.rlim && o < io.rng_cap)
+                const int place = WQ ? __shfl_sync(RT_FULL, hi, run_last<F>(t, mc, lane)) - lo
+                                     : wk.cur - wk.lcur + ids_before<F>(mc, hi - lo, lane, lt);
+                if ((F >= kRunSingly ? cont : (ms >> lane) & 1u) && o < sg.rlim && o < io.rng_cap)
                     io.rng_out[o] = make_int2(lo, place);
             }
-            wk.rcur += __popc(mc);
+            wk.rcur += __popc(ms);
+            if (F < kRunSingly && stats)
+                wk.n_whole += __popc(mc);
             if (PASS == PASS_SCATTER) {
-                unsigned mm = mc;
+                unsigned mm = ms;
                 while (mm) {
                     const int src = __ffs(mm) - 1;
                     mm &= mm - 1;
                     const int l = __shfl_sync(RT_FULL, lo, src);
-                    const int h = __shfl_sync(RT_FULL, hi, src);
+                    const int h = __shfl_sync(RT_FULL, hi, run_last<F>(t, mc, src));
                     const int64_t at = WQ ? sg.base + reserve(io.cur_ids + qi, h - l, lane) : sg.base + wk.cur;
                     const int64_t end = sg.lim < io.out_cap ? sg.lim : io.out_cap;
                     const int64_t room = end - at;
@@ -418,25 +449,28 @@ __device__ __forceinline__ Seg seg_of(const SelIO &io, int pass, int64_t qi)
     return sg;
 }
 
+template <int F>
 __device__ __forceinline__ void flush_stats(unsigned long long *stats, const Walk &wk, bool new_query)
 {
     if (new_query)
         atomicAdd(stats + 0, 1ull);
     atomicAdd(stats + 1, wk.n_visit);
     atomicAdd(stats + 2, wk.n_leaf);
-    atomicAdd(stats + 3, (unsigned long long)wk.rcur);
+    atomicAdd(stats + 3, (unsigned long long)(F >= kRunSingly ? wk.rcur : wk.n_whole));
     atomicAdd(stats + 4, (unsigned long long)wk.cur);
     atomicAdd(stats + 5, (unsigned long long)(wk.cur - wk.lcur));
 }
 
 // CTAs per SM the warp-per-query kernel is compiled for.  The descriptor
-// pass at F=64 takes six (40 registers a thread): its walk is bound by the
-// latency of dependent node loads, and the extra resident warps were
-// measured to outweigh a few spilled registers; at F=128 four (64
-// registers, no spills); elsewhere the compiler chooses.
+// pass's walk is bound by the latency of dependent node loads, so it takes the
+// warps that the registers allow with at most a few spilled: left to the
+// compiler (51 registers, five CTAs) F=16 took 209 us instead of 188, F=32 in
+// the LOHI layout 220 instead of 188 (100K queries of 0.01% on 2M), F=64 2585
+// instead of 2530 (1M queries on 11M); at F=128 the five and six CTAs that
+// need fewer than 64 registers took 185 and 196 us instead of 172.
 constexpr int select_min_blocks(int F, int pass)
 {
-    return pass != PASS_DESC ? 1 : (F == 64 ? 6 : (F == 128 ? 4 : 1));
+    return pass != PASS_DESC ? 1 : (F >= 128 ? 4 : (F >= 32 ? 7 : 6));
 }
 
 // Warp per query: each warp takes the next query from a counter and walks
@@ -483,7 +517,7 @@ __global__ void __launch_bounds__(kThreads, select_min_blocks(F, PASS))
                 continue;
             }
         }
-        Walk wk{0, 0, 0, 0, 0, false};
+        Walk wk{0, 0, 0, 0, 0, 0, false};
         int top = 0;
         if (t.nodes > 0) {
             if (lane == 0)
@@ -501,7 +535,7 @@ __global__ void __launch_bounds__(kThreads, select_min_blocks(F, PASS))
                                                 PASS == PASS_COUNT && stats != nullptr, lane, grp, sub, lt, lp);
         }
         if (PASS == PASS_COUNT && stats && lane == 0)
-            flush_stats(stats, wk, true);
+            flush_stats<F>(stats, wk, true);
         if (lane == 0) {
             if (wk.overflow)
                 atomicOr(flags, FLAG_STACK);
@@ -619,7 +653,7 @@ __global__ void __launch_bounds__(kThreads)
         const int root = (int)(word >> 32);
         const float4 q = __ldg(queries + qi);
         const Seg sg = seg_of(io, PASS, qi);
-        Walk wk{0, 0, 0, 0, 0, false};
+        Walk wk{0, 0, 0, 0, 0, 0, false};
         if (lane == 0)
             st[0] = root;
         int top = 1;
@@ -679,7 +713,7 @@ __global__ void __launch_bounds__(kThreads)
             }
         }
         if (PASS == PASS_COUNT && stats && lane == 0)
-            flush_stats(stats, wk, root == 0);
+            flush_stats<F>(stats, wk, root == 0);
         if (lane == 0) {
             if (wk.overflow)
                 atomicOr(flags, FLAG_STACK);
@@ -773,17 +807,18 @@ __global__ void k_wq_places(const SelIO io, int64_t Q)
 // gain from about 160 on.
 // The runs [lo, lo + len) of the lanes of mc go to query `slot`.
 template <int F>
-__device__ __forceinline__ void large_runs(const SelIO &io, const LargeIO &lg, const Seg &sg, int64_t slot, unsigned mc, int lo, int len,
+__device__ __forceinline__ void large_runs(const TreeDev &t, const SelIO &io, const LargeIO &lg, const Seg &sg, int64_t slot, unsigned mc, int lo, int len,
                                            int lane, unsigned lt)
 {
+    const unsigned ms = run_starts<F>(t, mc);
     const int before = ids_before<F>(mc, len, lane, lt);
     const unsigned ids = __reduce_add_sync(RT_FULL, (unsigned)len);
     unsigned long long r = 0;
     if (lane == 0)
-        r = atomicAdd(lg.runs + slot, ((unsigned long long)__popc(mc) << 32) | ids);
+        r = atomicAdd(lg.runs + slot, ((unsigned long long)__popc(ms) << 32) | ids);
     r = __shfl_sync(RT_FULL, r, 0);
-    const int64_t o = sg.rbase + (int64_t)(r >> 32) + __popc(mc & lt);
-    if (((mc >> lane) & 1u) && o < sg.rlim && o < io.rng_cap)
+    const int64_t o = sg.rbase + (int64_t)(r >> 32) + __popc(ms & lt);
+    if (((ms >> lane) & 1u) && o < sg.rlim && o < io.rng_cap)
         io.rng_out[o] = make_int2(lo, (int)(r & 0xffffffffull) + before);
 }
 
@@ -838,7 +873,7 @@ __global__ void __launch_bounds__(kThreads)
                     int4 cm = make_int4(0, 0, 0, 0);
                     if (cont)
                         cm = __ldg(t.meta + m.x + j);
-                    large_runs<1>(io, lg, sg, slot, mc, cm.z, cm.w - cm.z, lane, lt);
+                    large_runs<1>(t, io, lg, sg, slot, mc, cm.z, cm.w - cm.z, lane, lt);
                 }
             }
             __syncwarp();
@@ -893,7 +928,7 @@ __global__ void __launch_bounds__(kThreads)
                 int lo = 0, len = 0;
                 if (cont)
                     leaf_span<F>(t, lp, m.x + j, lo, len);
-                large_runs<F>(io, lg, sg, slot, mc, lo, len, lane, lt);
+                large_runs<F>(t, io, lg, sg, slot, mc, lo, len, lane, lt);
             }
         }
         __syncwarp();
