@@ -37,16 +37,6 @@ inline unsigned blocks_for(int64_t n, int per_block = kThreads)
     return (unsigned)(b < 1 ? 1 : (b > 1048576 ? 1048576 : b));
 }
 
-// float32 centre key as an order-preserving unsigned integer.
-__device__ __forceinline__ uint32_t centre_key(float lo, float hi)
-{
-    const float k = __fadd_rn(lo, hi);
-    uint32_t u = __float_as_uint(k);
-    if (k != k || (u << 1) == 0u)
-        u = 0u;  // NaN -> +0, -0 -> +0
-    return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
-}
-
 __global__ void k_validate(const float4 *__restrict__ r, int64_t n, unsigned long long *bad)
 {
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n;
@@ -182,13 +172,15 @@ __global__ void k_sort_children(const float4 *__restrict__ items, uint32_t *__re
 }
 
 // ---- small levels: one CTA builds every level of at most kSmallLevel items
-// (the upper levels of a big tree, or all of a small one), instead of a
-// dozen launches per level.  Each level is sorted twice in shared memory by
-// a bitonic network over 64-bit composite keys that end in the item index,
-// which gives exactly the stable orders of the radix path:
+// (the upper levels of a big tree, or all of a small one) in one launch; the
+// sorts by a cluster (str_order_small) are faster from about this size on (2,442
+// boxes and what is above them: 108 us here, 45 there).  Each level is sorted
+// twice in shared memory by a bitonic network over 64-bit composite keys that
+// end in the item index, which gives exactly the stable orders of the radix
+// path:
 //   (x centre key, item)  -> slab = rank / (S*F),
 //   (slab, y centre key, item) -> the packing order.
-constexpr int kSmallLevel = 4096;  // item indices fit 12 bits
+constexpr int kSmallLevel = 1024;  // item indices fit 12 bits
 
 struct SmallLevels {
     int count;                      // levels to build, bottom up
@@ -482,11 +474,13 @@ rtree_status build_tree(const float4 *rects, const int32_t *ids, int64_t n, int 
 
     {
         DevBuf<uint32_t> k0(s), v0(s), k1(s), v1(s), slab(s);
-        RT_TRY(k0.alloc(n, "build keys"));
-        RT_TRY(v0.alloc(n, "build values"));
-        RT_TRY(k1.alloc(n, "build keys"));
-        RT_TRY(v1.alloc(n, "build values"));
-        RT_TRY(slab.alloc(n, "build slabs"));
+        if (n > kSmallLevel && !str_order_is_small(n)) {
+            RT_TRY(k0.alloc(n, "build keys"));
+            RT_TRY(v0.alloc(n, "build values"));
+            RT_TRY(k1.alloc(n, "build keys"));
+            RT_TRY(v1.alloc(n, "build values"));
+            RT_TRY(slab.alloc(n, "build slabs"));
+        }
         const float4 *cur = rects;
         int64_t m = n;
         for (;;) {
@@ -527,7 +521,9 @@ rtree_status build_tree(const float4 *rects, const int32_t *ids, int64_t n, int 
             auto *pack = new DevBuf<uint32_t>(s);
             packs.push_back(pack);
             RT_TRY(pack->alloc(m, "build packing order"));
-            if (nslab > 1) {
+            if (str_order_is_small(m)) {
+                RT_TRY(str_order_small(cur, m, cap, pack->p, s));
+            } else if (nslab > 1) {
                 {
                     KernelTimer kt_("keys", s);
                     k_keys<<<blocks_for(m), kThreads, 0, s>>>(cur, m, 0, k0.p, v0.p);

@@ -269,6 +269,16 @@ __device__ __forceinline__ bool inside(float4 c, float4 q)
     return q.x <= c.x && c.z <= q.z && q.y <= c.y && c.w <= q.w;
 }
 
+// float32 centre key as an order-preserving unsigned integer.
+__device__ __forceinline__ uint32_t centre_key(float lo, float hi)
+{
+    const float k = __fadd_rn(lo, hi);
+    uint32_t u = __float_as_uint(k);
+    if (k != k || (u << 1) == 0u)
+        u = 0u;  // NaN -> +0, -0 -> +0
+    return (u & 0x80000000u) ? ~u : (u | 0x80000000u);
+}
+
 __device__ __forceinline__ float4 empty_box()
 {
     return make_float4(__int_as_float(0x7f800000), __int_as_float(0x7f800000),
@@ -326,6 +336,11 @@ rtree_status compute_leaf_part(rtree *t, cudaStream_t s);
 // Inputs are not modified; outputs must not alias inputs.
 rtree_status radix_sort_pairs(const uint32_t *kin, const uint32_t *vin, uint32_t *kout,
                               uint32_t *vout, int64_t n, int bit_lo, int bit_hi, cudaStream_t s);
+// The STR packing order of a level of m boxes in slabs of `size` items, as the
+// general path of build_tree makes it, for levels that are small.
+bool str_order_is_small(int64_t m);
+rtree_status str_order_small(const float4 *boxes, int64_t m, int64_t size, uint32_t *pack, cudaStream_t s);
+
 
 // Outputs of one select pass kernel (unused fields are null).
 struct SelIO {
