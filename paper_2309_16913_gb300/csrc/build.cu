@@ -48,40 +48,6 @@ __global__ void k_validate(const float4 *__restrict__ r, int64_t n, unsigned lon
     }
 }
 
-__global__ void k_keys(const float4 *__restrict__ boxes, int64_t m, int axis,
-                       uint32_t *__restrict__ keys, uint32_t *__restrict__ vals)
-{
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m;
-         i += (int64_t)gridDim.x * blockDim.x) {
-        const float4 b = boxes[i];
-        keys[i] = axis == 0 ? centre_key(b.x, b.z) : centre_key(b.y, b.w);
-        vals[i] = (uint32_t)i;
-    }
-}
-
-__global__ void k_slab_of(const uint32_t *__restrict__ order_x, int64_t m, int64_t cap,
-                          uint32_t *__restrict__ slab)
-{
-    const uint32_t cap32 = (uint32_t)cap;  // m < 2^31, so ranks and cap fit 32 bits
-    for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < m;
-         r += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t i = order_x[r];
-        if (i < m)
-            slab[i] = (uint32_t)r / cap32;
-    }
-}
-
-__global__ void k_gather_slab(const uint32_t *__restrict__ order_y,
-                              const uint32_t *__restrict__ slab, int64_t m,
-                              uint32_t *__restrict__ keys)
-{
-    for (int64_t p = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; p < m;
-         p += (int64_t)gridDim.x * blockDim.x) {
-        const uint32_t i = order_y[p];
-        keys[p] = i < m ? slab[i] : 0u;
-    }
-}
-
 // Bounding box of each packed node (exact min/max).  A group of G = min(F,
 // 32) lanes takes one node: each lane reduces every G-th item, then the
 // group reduces by shuffles (min/max are exact in any order).
@@ -173,7 +139,7 @@ __global__ void k_sort_children(const float4 *__restrict__ items, uint32_t *__re
 
 // ---- small levels: one CTA builds every level of at most kSmallLevel items
 // (the upper levels of a big tree, or all of a small one) in one launch; the
-// sorts by a cluster (str_order_small) are faster from about this size on (2,442
+// sorts by a cluster (str_order) are faster from about this size on (2,442
 // boxes and what is above them: 108 us here, 45 there).  Each level is sorted
 // twice in shared memory by a bitonic network over 64-bit composite keys that
 // end in the item index, which gives exactly the stable orders of the radix
@@ -382,16 +348,6 @@ int64_t ceil_sqrt(int64_t p)
     return s;
 }
 
-int bits_for(uint64_t v)  // bits needed to hold values 0..v
-{
-    int b = 0;
-    while (v) {
-        ++b;
-        v >>= 1;
-    }
-    return b;
-}
-
 // Allocates the leaf record (TreeDev::leaf_part) and fills it from the leaf
 // level's metadata, on stream s.
 rtree_status leaf_part_into(const int4 *leaf_meta, int64_t P, int F, DevBuf<int64_t> &part, cudaStream_t s)
@@ -473,14 +429,6 @@ rtree_status build_tree(const float4 *rects, const int32_t *ids, int64_t n, int 
     } cleanup{packs, boxes};
 
     {
-        DevBuf<uint32_t> k0(s), v0(s), k1(s), v1(s), slab(s);
-        if (n > kSmallLevel && !str_order_is_small(n)) {
-            RT_TRY(k0.alloc(n, "build keys"));
-            RT_TRY(v0.alloc(n, "build values"));
-            RT_TRY(k1.alloc(n, "build keys"));
-            RT_TRY(v1.alloc(n, "build values"));
-            RT_TRY(slab.alloc(n, "build slabs"));
-        }
         const float4 *cur = rects;
         int64_t m = n;
         for (;;) {
@@ -517,45 +465,10 @@ rtree_status build_tree(const float4 *rects, const int32_t *ids, int64_t n, int 
             const int64_t P = (m + F - 1) / F;
             const int64_t S = ceil_sqrt(P);
             const int64_t cap = S * F;
-            const int64_t nslab = (m + cap - 1) / cap;
             auto *pack = new DevBuf<uint32_t>(s);
             packs.push_back(pack);
             RT_TRY(pack->alloc(m, "build packing order"));
-            if (str_order_is_small(m)) {
-                RT_TRY(str_order_small(cur, m, cap, pack->p, s));
-            } else if (nslab > 1) {
-                {
-                    KernelTimer kt_("keys", s);
-                    k_keys<<<blocks_for(m), kThreads, 0, s>>>(cur, m, 0, k0.p, v0.p);
-                    RT_LAUNCH();
-                }
-                RT_TRY(radix_sort_pairs(k0.p, v0.p, k1.p, v1.p, m, 0, 32, s));
-                {
-                    KernelTimer kt_("slab_of", s);
-                    k_slab_of<<<blocks_for(m), kThreads, 0, s>>>(v1.p, m, cap, slab.p);
-                    RT_LAUNCH();
-                }
-                {
-                    KernelTimer kt_("keys", s);
-                    k_keys<<<blocks_for(m), kThreads, 0, s>>>(cur, m, 1, k0.p, v0.p);
-                    RT_LAUNCH();
-                }
-                RT_TRY(radix_sort_pairs(k0.p, v0.p, k1.p, v1.p, m, 0, 32, s));
-                {
-                    KernelTimer kt_("gather_slab", s);
-                    k_gather_slab<<<blocks_for(m), kThreads, 0, s>>>(v1.p, slab.p, m, k0.p);
-                    RT_LAUNCH();
-                }
-                RT_TRY(radix_sort_pairs(k0.p, v1.p, k1.p, pack->p, m, 0,
-                                        bits_for((uint64_t)(nslab - 1)), s));
-            } else {
-                {
-                    KernelTimer kt_("keys", s);
-                    k_keys<<<blocks_for(m), kThreads, 0, s>>>(cur, m, 1, k0.p, v0.p);
-                    RT_LAUNCH();
-                }
-                RT_TRY(radix_sort_pairs(k0.p, v0.p, k1.p, pack->p, m, 0, 32, s));
-            }
+            RT_TRY(str_order(cur, m, cap, pack->p, s));
             if (sort_children && F > 1) {
                 KernelTimer kt_("sort_children", s);
                 k_sort_children<<<blocks_for(P * 32), kThreads, 0, s>>>(cur, pack->p, m, F, P);

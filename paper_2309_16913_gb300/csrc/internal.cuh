@@ -336,10 +336,9 @@ rtree_status compute_leaf_part(rtree *t, cudaStream_t s);
 // Inputs are not modified; outputs must not alias inputs.
 rtree_status radix_sort_pairs(const uint32_t *kin, const uint32_t *vin, uint32_t *kout,
                               uint32_t *vout, int64_t n, int bit_lo, int bit_hi, cudaStream_t s);
-// The STR packing order of a level of m boxes in slabs of `size` items, as the
-// general path of build_tree makes it, for levels that are small.
-bool str_order_is_small(int64_t m);
-rtree_status str_order_small(const float4 *boxes, int64_t m, int64_t size, uint32_t *pack, cudaStream_t s);
+// The STR packing order of a level of m boxes in slabs of `size` items: by
+// (rank by x centre / size, y centre, index).
+rtree_status str_order(const float4 *boxes, int64_t m, int64_t size, uint32_t *pack, cudaStream_t s);
 
 
 // Outputs of one select pass kernel (unused fields are null).

@@ -16,6 +16,9 @@
 // ballot per digit bit and rank by lane order on top of a per-warp running
 // count), tiles are taken in order inside a CTA, and CTAs own consecutive
 // runs.
+#include <algorithm>
+#include <type_traits>
+
 #include "internal.cuh"
 
 namespace rt {
@@ -26,6 +29,7 @@ constexpr int kWarps = kThreads / 32;
 constexpr int kItems = 16;
 constexpr int kTile = kThreads * kItems;  // 4096
 constexpr int kBins = 256;
+constexpr int kWide = 1024;               // digits of up to 10 bits, where they save a pass
 constexpr int kWarpRun = 32 * kItems;     // contiguous items owned by one warp
 static_assert(kThreads == kBins, "one thread per digit");
 
@@ -39,11 +43,12 @@ __device__ __forceinline__ void run_of(int64_t ntiles, int G, int c, int64_t &t0
 // Lanes of the warp whose digit equals this lane's (all lanes valid or not
 // take part; the answer is meaningful for valid lanes), from one ballot per
 // digit bit.
+template <int BITS = 8>
 __device__ __forceinline__ unsigned peers_of(int dg, uint32_t mask, bool ok)
 {
     unsigned peers = __ballot_sync(RT_FULL, ok);
 #pragma unroll
-    for (int b = 0; b < 8; ++b) {
+    for (int b = 0; b < BITS; ++b) {
         if (!((mask >> b) & 1u))
             break;
         const unsigned m = __ballot_sync(RT_FULL, (dg >> b) & 1);
@@ -75,12 +80,13 @@ __device__ __forceinline__ uint32_t block_excl(uint32_t v, uint32_t *wsum)
     return add + inc - v;
 }
 
+template <int BINS>
 __global__ void __launch_bounds__(kThreads) k_hist(const uint32_t *__restrict__ keys, int64_t n,
                                                    int shift, uint32_t mask, int64_t ntiles, int G,
                                                    uint32_t *__restrict__ hist)
 {
-    __shared__ uint32_t h[kWarps][kBins];
-    for (int i = threadIdx.x; i < kWarps * kBins; i += kThreads)
+    __shared__ uint32_t h[kWarps][BINS];
+    for (int i = threadIdx.x; i < kWarps * BINS; i += kThreads)
         (&h[0][0])[i] = 0;
     __syncthreads();
     int64_t t0, t1;
@@ -91,12 +97,14 @@ __global__ void __launch_bounds__(kThreads) k_hist(const uint32_t *__restrict__ 
     for (int64_t k = b + threadIdx.x; k < e; k += kThreads)
         atomicAdd(&h[w][(__ldg(keys + k) >> shift) & mask], 1u);
     __syncthreads();
-    const int d = threadIdx.x;
-    uint32_t s = 0;
 #pragma unroll
-    for (int x = 0; x < kWarps; ++x)
-        s += h[x][d];
-    hist[(int64_t)d * G + blockIdx.x] = s;
+    for (int d = threadIdx.x; d < BINS; d += kThreads) {
+        uint32_t s = 0;
+#pragma unroll
+        for (int x = 0; x < kWarps; ++x)
+            s += h[x][d];
+        hist[(int64_t)d * G + blockIdx.x] = s;
+    }
 }
 
 // Per digit d (one CTA each): exclusive scan of hist[d*G .. d*G+G) into
@@ -122,30 +130,65 @@ __global__ void __launch_bounds__(kThreads) k_scan(const uint32_t *__restrict__ 
         tot[blockIdx.x] = run;
 }
 
+// What the last pass leaves.
+enum : int {
+    END_PAIRS = 0,    // the sorted keys and values
+    END_VALUES = 1,   // the values
+    END_GROUPS = 2,   // table[value] = place / size, nothing else
+    END_RELABEL = 3   // the values, and table[value] as their keys
+};
+struct RadixEnd {
+    int what;
+    uint32_t *table;
+    uint32_t size;
+};
+
+template <int BINS>
+struct ScatterSmem {
+    // counts of a tile and places in it fit 16 bits; the narrow form has room for words
+    using Count = typename std::conditional<(BINS > kBins), uint16_t, uint32_t>::type;
+    uint32_t k[kTile], v[kTile];
+    uint32_t base[BINS];  // where this CTA's next item of each digit goes
+    uint32_t wsum[kWarps];
+    Count wcnt[kWarps][BINS];
+    Count tstart[BINS];
+};
+
 // Four CTAs per SM (64 registers a thread): the tiles' loads of one CTA
-// overlap the ranking of the others.
+// overlap the ranking of the others.  A value is its own index where vin is null.
+template <int BINS, int END>
 __global__ void __launch_bounds__(kThreads, 4)
     k_scatter(const uint32_t *__restrict__ kin, const uint32_t *__restrict__ vin,
               uint32_t *__restrict__ kout, uint32_t *__restrict__ vout, int64_t n, int shift,
               uint32_t mask, const uint32_t *__restrict__ offs, const uint32_t *__restrict__ tot,
-              int64_t ntiles, int G)
+              int64_t ntiles, int G, RadixEnd end)
 {
-    __shared__ uint32_t wcnt[kWarps][kBins];
-    __shared__ uint32_t tstart[kBins];
-    __shared__ uint32_t base[kBins];  // where this CTA's next item of each digit goes
-    __shared__ uint32_t wsum[kWarps];
-    __shared__ uint32_t sk[kTile];
-    __shared__ uint32_t sv[kTile];
+    constexpr int PER = BINS / kThreads;  // digits a thread looks after
+    using Smem = ScatterSmem<BINS>;
+    using Count = typename Smem::Count;
+    extern __shared__ uint4 smem[];
+    Smem &sm = *reinterpret_cast<Smem *>(smem);
 
-    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, d = threadIdx.x;
+    const int w = threadIdx.x >> 5, lane = threadIdx.x & 31, d0 = threadIdx.x * PER;
     const unsigned lt = lanemask_lt();
     int64_t t0, t1;
     run_of(ntiles, G, blockIdx.x, t0, t1);
     // items of smaller digits come first, then this digit's items of earlier CTAs
-    base[d] = block_excl<kThreads>(tot[d], wsum) + offs[(int64_t)d * G + blockIdx.x];
+    {
+        uint32_t all = 0;
+#pragma unroll
+        for (int j = 0; j < PER; ++j)
+            all += tot[d0 + j];
+        uint32_t at = block_excl<kThreads>(all, sm.wsum);
+#pragma unroll
+        for (int j = 0; j < PER; ++j) {
+            sm.base[d0 + j] = at + offs[(int64_t)(d0 + j) * G + blockIdx.x];
+            at += tot[d0 + j];
+        }
+    }
     for (int64_t tile = t0; tile < t1; ++tile) {
-        for (int i = threadIdx.x; i < kWarps * kBins; i += kThreads)
-            (&wcnt[0][0])[i] = 0;
+        for (int i = threadIdx.x; i < (int)(sizeof(sm.wcnt) / 4); i += kThreads)
+            reinterpret_cast<uint32_t *>(&sm.wcnt[0][0])[i] = 0;
         __syncthreads();  // also: the previous tile's staging is written out
 
         const int64_t tile0 = tile * kTile;
@@ -160,25 +203,35 @@ __global__ void __launch_bounds__(kThreads, 4)
         for (int i = 0; i < kItems; ++i) {
             const bool ok = wbase + i * 32 + lane < n;
             const int dg = (int)((k[i] >> shift) & mask);
-            const unsigned peers = peers_of(dg, mask, ok);
-            const uint32_t prev = ok ? wcnt[w][dg] : 0u;
+            const unsigned peers = peers_of<(BINS > kBins ? 10 : 8)>(dg, mask, ok);
+            const uint32_t prev = ok ? sm.wcnt[w][dg] : 0u;
             rank[i] = prev + __popc(peers & lt);
             __syncwarp();
             if (ok && lane == __ffs(peers) - 1)
-                wcnt[w][dg] = prev + __popc(peers);
+                sm.wcnt[w][dg] = (Count)(prev + __popc(peers));
             __syncwarp();
         }
         __syncthreads();
 
         // per digit: exclusive prefix over warps (in place) and the tile's count
-        uint32_t cnt = 0;
+        uint32_t cnt[PER], all = 0;
 #pragma unroll
-        for (int x = 0; x < kWarps; ++x) {
-            const uint32_t c = wcnt[x][d];
-            wcnt[x][d] = cnt;
-            cnt += c;
+        for (int j = 0; j < PER; ++j) {
+            cnt[j] = 0;
+#pragma unroll
+            for (int x = 0; x < kWarps; ++x) {
+                const uint32_t c = sm.wcnt[x][d0 + j];
+                sm.wcnt[x][d0 + j] = (Count)cnt[j];
+                cnt[j] += c;
+            }
+            all += cnt[j];
         }
-        tstart[d] = block_excl<kThreads>(cnt, wsum);  // the digit runs' starts in the tile
+        uint32_t at = block_excl<kThreads>(all, sm.wsum);  // the digit runs' starts in the tile
+#pragma unroll
+        for (int j = 0; j < PER; ++j) {
+            sm.tstart[d0 + j] = (Count)at;
+            at += cnt[j];
+        }
         __syncthreads();
 
         // stage the tile in digit order: keys, then values (read only now)
@@ -186,38 +239,62 @@ __global__ void __launch_bounds__(kThreads, 4)
         for (int i = 0; i < kItems; ++i) {
             if (wbase + i * 32 + lane < n) {
                 const int dg = (int)((k[i] >> shift) & mask);
-                rank[i] += tstart[dg] + wcnt[w][dg];
-                sk[rank[i]] = k[i];
+                rank[i] += sm.tstart[dg] + sm.wcnt[w][dg];
+                sm.k[rank[i]] = k[i];
             }
         }
+        if (vin) {
 #pragma unroll
-        for (int i = 0; i < kItems; ++i) {
-            const int64_t idx = wbase + i * 32 + lane;
-            if (idx < n)
-                sv[rank[i]] = __ldg(vin + idx);
+            for (int i = 0; i < kItems; ++i) {
+                const int64_t idx = wbase + i * 32 + lane;
+                if (idx < n)
+                    sm.v[rank[i]] = __ldg(vin + idx);
+            }
+        } else {
+#pragma unroll
+            for (int i = 0; i < kItems; ++i) {
+                const int64_t idx = wbase + i * 32 + lane;
+                if (idx < n)
+                    sm.v[rank[i]] = (uint32_t)idx;
+            }
         }
         __syncthreads();
         const int tn = (int)(n - tile0 < kTile ? n - tile0 : kTile);
         for (int p = threadIdx.x; p < tn; p += kThreads) {
-            const uint32_t key = sk[p];
+            const uint32_t key = sm.k[p];
             const int dd = (int)((key >> shift) & mask);
-            const uint32_t dst = base[dd] + (uint32_t)p - tstart[dd];
+            const uint32_t dst = sm.base[dd] + (uint32_t)p - sm.tstart[dd];
             if (dst < (uint64_t)n) {
-                kout[dst] = key;
-                vout[dst] = sv[p];
+                if (END == END_PAIRS)
+                    kout[dst] = key;
+                const uint32_t value = sm.v[p];
+                if (END == END_GROUPS) {
+                    if (value < (uint64_t)n)
+                        end.table[value] = dst / end.size;
+                } else {
+                    vout[dst] = value;
+                }
+                if (END == END_RELABEL)
+                    kout[dst] = value < (uint64_t)n ? __ldg(end.table + value) : 0u;
             }
         }
         __syncthreads();
-        base[d] += cnt;
+#pragma unroll
+        for (int j = 0; j < PER; ++j)
+            sm.base[d0 + j] += cnt[j];
     }
 }
 
 // CTAs of the persistent grid: every SM full (at most one tile each).
+template <int BINS, int END>
 int grid_for(int64_t ntiles)
 {
     static const int per_sm = [] {  // initialised once, thread-safely
         int v = 0;
-        if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, k_scatter, kThreads, 0) != cudaSuccess || v < 1) {
+        if (cudaFuncSetAttribute(k_scatter<BINS, END>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                 (int)sizeof(ScatterSmem<BINS>)) != cudaSuccess ||
+            cudaOccupancyMaxActiveBlocksPerMultiprocessor(&v, k_scatter<BINS, END>, kThreads,
+                                                          sizeof(ScatterSmem<BINS>)) != cudaSuccess || v < 1) {
             cudaGetLastError();
             v = 1;
         }
@@ -225,6 +302,75 @@ int grid_for(int64_t ntiles)
     }();
     const int64_t g = (int64_t)per_sm * sm_count();
     return (int)(ntiles < g ? ntiles : g);
+}
+
+// Words of digit counts that a pass over n pairs needs.
+template <int BINS, int END>
+size_t count_words(int64_t n)
+{
+    return (size_t)BINS * (2 * grid_for<BINS, END>((n + kTile - 1) / kTile) + 1);
+}
+
+// One pass: digit (key >> shift) & mask, of at most BINS values.
+template <int BINS, int END>
+rtree_status radix_pass(const uint32_t *kin, const uint32_t *vin, uint32_t *kout, uint32_t *vout, int64_t n,
+                        int shift, uint32_t mask, const RadixEnd &end, uint32_t *counts, cudaStream_t s)
+{
+    const int64_t ntiles = (n + kTile - 1) / kTile;
+    const int G = grid_for<BINS, END>(ntiles);
+    uint32_t *hist = counts, *offs = hist + (size_t)BINS * G, *tot = offs + (size_t)BINS * G;
+    {
+        KernelTimer kt_("hist", s);
+        k_hist<BINS><<<(unsigned)G, kThreads, 0, s>>>(kin, n, shift, mask, ntiles, G, hist);
+        RT_LAUNCH();
+    }
+    {
+        KernelTimer kt_("radix_scan", s);
+        k_scan<<<BINS, kThreads, 0, s>>>(hist, G, offs, tot);
+        RT_LAUNCH();
+    }
+    KernelTimer kt_("scatter", s);
+    k_scatter<BINS, END><<<(unsigned)G, kThreads, sizeof(ScatterSmem<BINS>), s>>>(
+        kin, vin, kout, vout, n, shift, mask, offs, tot, ntiles, G, end);
+    RT_LAUNCH();
+    return RTREE_OK;
+}
+
+// All passes over the bits [bit_lo, bit_hi); the last one leaves END.
+template <int END>
+rtree_status radix_passes(const uint32_t *kin, const uint32_t *vin, uint32_t *kout, uint32_t *vout, int64_t n,
+                          int bit_lo, int bit_hi, const RadixEnd &end, cudaStream_t s)
+{
+    // ten bits at a time where that saves a pass (10M items by 9 bits: 90 us less than two
+    // passes take)
+    const int bits = bit_hi - bit_lo, wide = (bits + 9) / 10, passes = (bits + 7) / 8 > wide ? wide : (bits + 7) / 8;
+    const int digit = (bits + passes - 1) / passes;
+    DevBuf<uint32_t> tk(s), tv(s), counts(s);
+    if (passes > 1) {
+        RT_TRY(tk.alloc(n, "radix keys"));
+        RT_TRY(tv.alloc(n, "radix values"));
+    }
+    const size_t words = digit > 8 ? std::max(count_words<kWide, END>(n), count_words<kWide, END_PAIRS>(n))
+                                   : std::max(count_words<kBins, END>(n), count_words<kBins, END_PAIRS>(n));
+    RT_TRY(counts.alloc(words, "radix digit counts"));
+    // Ping-pong so that the last pass writes kout/vout.
+    uint32_t *bk[2] = {kout, tk.p}, *bv[2] = {vout, tv.p};
+    for (int p = 0; p < passes; ++p) {
+        const int shift = bit_lo + digit * p, o = (passes - 1 - p) & 1;
+        const uint32_t mask = (1u << min(digit, bit_hi - shift)) - 1u;
+        const bool last = p == passes - 1;
+        rtree_status st;
+        if (digit > 8)
+            st = last ? radix_pass<kWide, END>(kin, vin, bk[o], bv[o], n, shift, mask, end, counts.p, s)
+                      : radix_pass<kWide, END_PAIRS>(kin, vin, bk[o], bv[o], n, shift, mask, end, counts.p, s);
+        else
+            st = last ? radix_pass<kBins, END>(kin, vin, bk[o], bv[o], n, shift, mask, end, counts.p, s)
+                      : radix_pass<kBins, END_PAIRS>(kin, vin, bk[o], bv[o], n, shift, mask, end, counts.p, s);
+        RT_TRY(st);
+        kin = bk[o];
+        vin = bv[o];
+    }
+    return RTREE_OK;
 }
 
 // ---- small sorts: every pass in one launch, by a cluster of CTAs.
@@ -315,7 +461,7 @@ template <int SRC>
 __global__ void __launch_bounds__(kCThreads, 1)
     k_sort_cluster(const __grid_constant__ ClusterSort first, const __grid_constant__ ClusterSort second)
 {
-    extern __shared__ uint32_t smem[];
+    extern __shared__ uint4 smem[];
     ClusterSmem &sm = *reinterpret_cast<ClusterSmem *>(smem);
     unsigned me, C;
     asm("mov.u32 %0, %%cluster_ctarank;" : "=r"(me));
@@ -552,8 +698,8 @@ rtree_status radix_sort_pairs(const uint32_t *kin, const uint32_t *vin, uint32_t
         RT_CUDA(cudaMemcpyAsync(vout, vin, n * sizeof(uint32_t), cudaMemcpyDeviceToDevice, s));
         return RTREE_OK;
     }
-    const int passes = (bit_hi - bit_lo + 7) / 8;
     if (n <= kClusterMost && cluster_ctas() > 0) {
+        const int passes = (bit_hi - bit_lo + 7) / 8;
         DevBuf<uint32_t> tk(s), tv(s);
         if (passes > 1) {
             RT_TRY(tk.alloc(n, "radix keys"));
@@ -563,64 +709,63 @@ rtree_status radix_sort_pairs(const uint32_t *kin, const uint32_t *vin, uint32_t
                             0, (int)n, bit_lo, bit_hi, passes, 1};
         return launch_cluster<SRC_PAIRS>(a, a, 1, s);
     }
-    const int64_t ntiles = (n + kTile - 1) / kTile;
-    const int G = grid_for(ntiles);
-    DevBuf<uint32_t> tk(s), tv(s), hist(s), offs(s), tot(s);
-    if (passes > 1) {
-        RT_TRY(tk.alloc(n, "radix keys"));
-        RT_TRY(tv.alloc(n, "radix values"));
-    }
-    RT_TRY(hist.alloc((size_t)kBins * G, "radix histogram"));
-    RT_TRY(offs.alloc((size_t)kBins * G, "radix offsets"));
-    RT_TRY(tot.alloc(kBins, "radix digit totals"));
-    // Ping-pong so that the last pass writes kout/vout.
-    uint32_t *bk[2] = {kout, tk.p}, *bv[2] = {vout, tv.p};
-    int dst = (passes % 2 == 1) ? 0 : 1;
-    const uint32_t *sk = kin, *sv = vin;
-    for (int p = 0; p < passes; ++p) {
-        const int shift = bit_lo + 8 * p;
-        const int bits = min(8, bit_hi - shift);
-        const uint32_t mask = (1u << bits) - 1u;
-        {
-            KernelTimer kt_("hist", s);
-            k_hist<<<(unsigned)G, kThreads, 0, s>>>(sk, n, shift, mask, ntiles, G, hist.p);
-            RT_LAUNCH();
-        }
-        {
-            KernelTimer kt_("radix_scan", s);
-            k_scan<<<kBins, kThreads, 0, s>>>(hist.p, G, offs.p, tot.p);
-            RT_LAUNCH();
-        }
-        {
-            KernelTimer kt_("scatter", s);
-            k_scatter<<<(unsigned)G, kThreads, 0, s>>>(sk, sv, bk[dst], bv[dst], n, shift, mask, offs.p,
-                                                       tot.p, ntiles, G);
-            RT_LAUNCH();
-        }
-        sk = bk[dst];
-        sv = bv[dst];
-        dst ^= 1;
-    }
-    return RTREE_OK;
+    return radix_passes<END_PAIRS>(kin, vin, kout, vout, n, bit_lo, bit_hi, RadixEnd{END_PAIRS, nullptr, 1}, s);
 }
 
-// Levels up to this many boxes are packed by str_order_small: two clusters sort
-// the x and the y keys side by side, then one sorts the y order by slab.  A tree
+namespace {
+
+// Both centre keys of every box, read once.
+__global__ void k_keys(const float4 *__restrict__ boxes, int64_t m, uint32_t *__restrict__ kx,
+                       uint32_t *__restrict__ ky)
+{
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < m;
+         i += (int64_t)gridDim.x * blockDim.x) {
+        const float4 b = boxes[i];
+        kx[i] = centre_key(b.x, b.z);
+        ky[i] = centre_key(b.y, b.w);
+    }
+}
+
+// Slabs by the whole chip's passes: the x sort's last pass writes the items'
+// slabs, the y sort's last pass looks them up as the keys of the third sort.
+// Apart, the passes that made the keys of each axis, the slabs and the third
+// sort's keys cost a 10M-box build 200 us of 2,290.
+rtree_status str_order_large(const float4 *boxes, int64_t m, uint32_t size, int bits, uint32_t *pack, cudaStream_t s)
+{
+    DevBuf<uint32_t> kx(s), ky(s), k(s), v(s);
+    RT_TRY(kx.alloc(m, "build keys"));
+    RT_TRY(ky.alloc(m, "build keys"));
+    RT_TRY(k.alloc(m, "build keys"));
+    RT_TRY(v.alloc(m, "build values"));
+    {
+        KernelTimer kt_("keys", s);
+        const int64_t blocks = (m + kThreads - 1) / kThreads;
+        k_keys<<<(unsigned)(blocks < 1048576 ? blocks : 1048576), kThreads, 0, s>>>(boxes, m, kx.p, ky.p);
+        RT_LAUNCH();
+    }
+    if (bits == 0)  // one slab: the y order is the packing order
+        return radix_passes<END_VALUES>(ky.p, nullptr, k.p, pack, m, 0, 32, RadixEnd{END_VALUES, nullptr, 1}, s);
+    RT_TRY(radix_passes<END_GROUPS>(kx.p, nullptr, k.p, v.p, m, 0, 32, RadixEnd{END_GROUPS, kx.p, size}, s));
+    RT_TRY(radix_passes<END_RELABEL>(ky.p, nullptr, k.p, v.p, m, 0, 32, RadixEnd{END_RELABEL, kx.p, 1}, s));
+    return radix_passes<END_VALUES>(k.p, v.p, ky.p, pack, m, 0, bits, RadixEnd{END_VALUES, nullptr, 1}, s);
+}
+
+// Levels up to this many boxes are packed by clusters: two sort
+// the x and the y keys side by side, then one the y order by slab.  A tree
 // of 20K boxes (F=16) builds in 270 us instead of 449, of 150K in 360 instead of
 // 625, of 520K in 610 instead of 706; the sorts of a level use 32 SMs at most, so
 // larger ones are left to the whole chip.
 constexpr int64_t kLevelMost = (int64_t)1 << 19;
 
-bool str_order_is_small(int64_t m)
-{
-    return m <= kLevelMost && cluster_ctas() > 0;
-}
+}  // namespace
 
-rtree_status str_order_small(const float4 *boxes, int64_t m, int64_t size, uint32_t *pack, cudaStream_t s)
+rtree_status str_order(const float4 *boxes, int64_t m, int64_t size, uint32_t *pack, cudaStream_t s)
 {
     int bits = 0;
     for (int64_t v = (m + size - 1) / size - 1; v; v >>= 1)
         ++bits;
+    if (m > kLevelMost || cluster_ctas() == 0)
+        return str_order_large(boxes, m, (uint32_t)size, bits, pack, s);
     DevBuf<uint32_t> buf(s);
     RT_TRY(buf.alloc(8 * (size_t)m, "level order"));
     uint32_t *x = buf.p, *y = x + 4 * m;

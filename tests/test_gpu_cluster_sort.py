@@ -19,7 +19,8 @@ def rt():
 # 16 x 16384 = 2^18 items are one tile for each CTA of the cluster
 @pytest.mark.parametrize("kind", ["uniform", "dups"])
 @pytest.mark.parametrize("n,F", [(1024, 64), (1025, 64), (1025, 4), (1057, 128), (16 * 1024 + 1, 8), (2**18 - 31, 4),
-                                 (2**18, 16), (2**18 + 1, 32), (2**19 - 1, 4), (2**19, 128), (2**19 + 1, 16)])
+                                 (2**18, 16), (2**18 + 1, 32), (2**19 - 1, 4), (2**19, 128), (2**19 + 1, 16),
+                                 (2**19 + 1, 4), (2**21 + 1, 4), (4_200_000, 4)])  # slabs of 9, 10 and 11 bits
 def test_tree(rt, n, F, kind):
     rects = random_case(kind, n, n)
     ids = np.arange(n, dtype=np.int32)[::-1].copy()
