@@ -322,11 +322,19 @@ __device__ __forceinline__ float4 load_entry_t(const float *__restrict__ mbr, in
 }
 
 // ------------------------------------------------------ host-side helpers
-// Exclusive scan; out has n+1 entries and out[n] is the total.  most
-// (optional, int32 inputs >= 0): raised to the largest input.
-rtree_status scan_exclusive(const int32_t *in, int64_t *out, int64_t n, cudaStream_t s, int32_t *most = nullptr);
-rtree_status scan_exclusive(const uint32_t *in, uint32_t *out, int64_t n, cudaStream_t s);
-rtree_status scan_exclusive(const int64_t *in, int64_t *out, int64_t n, cudaStream_t s);
+struct PostList;
+// Exclusive scans of counts (>= 0); an out has n+1 entries and out[n] is the total.
+constexpr int kScanJobs = 3;
+struct ScanJobs {  // arrays of one length
+    int count;
+    const int32_t *in[kScanJobs];
+    int64_t *out[kScanJobs];
+    int32_t *most[kScanJobs];  // raised to the array's largest value, if given
+};
+rtree_status scan_exclusive(const ScanJobs &j, int64_t n, cudaStream_t s);
+// The same, and then a host read of words that the scans or what precedes them
+// leave (mailbox_post, mailbox_wait).
+rtree_status scan_and_read(const ScanJobs &j, int64_t n, const PostList &l, cudaStream_t s, uint32_t *out, int nwords);
 
 // Fills t->leaf_part (allocated here from the tree's allocator) from the
 // leaf level's metadata, on stream s.

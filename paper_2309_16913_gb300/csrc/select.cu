@@ -1226,7 +1226,7 @@ constexpr int64_t kMostTasks = 4 << 20;
 rtree_status range_select_bounded(const rtree *t, const float4 *queries, int64_t Q, int order,
                                   cudaStream_t s, rtree_result *res, DevBuf<int64_t> &off)
 {
-    DevBuf<int32_t> cnt(s), cnt_leaf(s), cnt_rng(s), flags(s);
+    DevBuf<int32_t> cnt(s), cnt_leaf(s), cnt_rng(s);
     DevBuf<unsigned long long> ctr(s);
     DevBuf<int64_t> off_leaf(s), off_rng(s);
     DevBuf<uint32_t> perm(s);
@@ -1235,13 +1235,14 @@ rtree_status range_select_bounded(const rtree *t, const float4 *queries, int64_t
     RT_TRY(cnt.alloc(Q, "select counts"));
     RT_TRY(cnt_leaf.alloc(Q, "select counts"));
     RT_TRY(cnt_rng.alloc(Q, "select counts"));
-    RT_TRY(flags.alloc(3, "select flags"));  // [0] select passes, [1] sort, [2] the longest result
-    RT_TRY(ctr.alloc(4, "select work counters"));  // two passes, large queries, tasks for them
+    // work counters of two passes, large queries and tasks for them; then the
+    // flags: [0] select passes, [1] sort, [2] the longest result
+    RT_TRY(ctr.alloc(6, "select work counters and flags"));
+    int32_t *flags = reinterpret_cast<int32_t *>(ctr.p + 4);
     RT_TRY(large.alloc(large_cap, "select large queries"));
     RT_TRY(off_leaf.alloc(Q + 1, "select offsets"));
     RT_TRY(off_rng.alloc(Q + 1, "select offsets"));
-    RT_CUDA(cudaMemsetAsync(flags.p, 0, 3 * sizeof(int32_t), s));
-    RT_CUDA(cudaMemsetAsync(ctr.p, 0, 4 * sizeof(unsigned long long), s));
+    RT_CUDA(cudaMemsetAsync(ctr.p, 0, 6 * sizeof(unsigned long long), s));
     if (order == RTREE_ORDER_HILBERT) {
         RT_TRY(perm.alloc(Q, "query order"));
         RT_TRY(hilbert_order(t, queries, Q, perm.p, s));
@@ -1259,9 +1260,7 @@ rtree_status range_select_bounded(const rtree *t, const float4 *queries, int64_t
     lg.leaves = large_leaves(Q);
     lg.total = off_leaf.p + Q;
     lg.budget = large_budget(t->fanout);
-    RT_TRY(launch(PASS_BOUND, t, queries, Q, io, ctr.p, flags.p, s, nullptr, lg));
-    RT_TRY(scan_exclusive(cnt_leaf.p, off_leaf.p, Q, s));
-    RT_TRY(scan_exclusive(cnt_rng.p, off_rng.p, Q, s));
+    RT_TRY(launch(PASS_BOUND, t, queries, Q, io, ctr.p, flags, s, nullptr, lg));
     // host read 1 of 2: the sizes of the descriptor pass's outputs and the flags
     int64_t h[2] = {0, 0}, n_large = 0, n_tasks = 0;
     int32_t hflags = 0;
@@ -1276,12 +1275,12 @@ rtree_status range_select_bounded(const rtree *t, const float4 *queries, int64_t
         pl.src[2] = ctr.p + 2;
         pl.words[2] = 4;
         pl.at[2] = 4;
-        pl.src[3] = flags.p;
+        pl.src[3] = flags;
         pl.words[3] = 1;
         pl.at[3] = 8;
         pl.n = 4;
         uint32_t w[9];
-        RT_TRY(read_words(pl, s, w, 9));
+        RT_TRY(scan_and_read({2, {cnt_leaf.p, cnt_rng.p}, {off_leaf.p, off_rng.p}, {}}, Q, pl, s, w, 9));
         h[0] = word64(w);
         h[1] = word64(w + 2);
         n_large = word64(w + 4) < large_cap ? word64(w + 4) : large_cap;
@@ -1308,11 +1307,10 @@ rtree_status range_select_bounded(const rtree *t, const float4 *queries, int64_t
     if (n_large > 0 && h[0] < lg.budget) {
         RT_TRY(tasks.alloc(n_tasks, "select tasks"));
         RT_TRY(large_cur.alloc(2 * n_large + 1, "select cursors"));
-        RT_TRY(launch_large(t, queries, so, lg, n_large, n_tasks, tasks.p, large_cur.p, flags.p, s));
+        RT_TRY(launch_large(t, queries, so, lg, n_large, n_tasks, tasks.p, large_cur.p, flags, s));
         pass = PASS_DESC_LARGE;
     }
-    RT_TRY(launch(pass, t, queries, Q, so, ctr.p + 1, flags.p, s, nullptr, lg));
-    RT_TRY(scan_exclusive(cnt.p, off.p, Q, s, flags.p + 2));
+    RT_TRY(launch(pass, t, queries, Q, so, ctr.p + 1, flags, s, nullptr, lg));
     // host read 2 of 2: the total (it sizes the result and is returned) and the
     // longest result (it says which sort classes are needed)
     int64_t total = 0, longest = 0;
@@ -1321,12 +1319,12 @@ rtree_status range_select_bounded(const rtree *t, const float4 *queries, int64_t
         pl.src[0] = off.p + Q;
         pl.words[0] = 2;
         pl.at[0] = 0;
-        pl.src[1] = flags.p;
+        pl.src[1] = flags;
         pl.words[1] = 3;
         pl.at[1] = 2;
         pl.n = 2;
         uint32_t w[5];
-        RT_TRY(read_words(pl, s, w, 5));
+        RT_TRY(scan_and_read({1, {cnt.p}, {off.p}, {flags + 2}}, Q, pl, s, w, 5));
         total = word64(w);
         longest = (int32_t)w[4];
         if (w[2])
@@ -1341,9 +1339,9 @@ rtree_status range_select_bounded(const rtree *t, const float4 *queries, int64_t
     src.rng = rng.p;
     src.off_rng = off_rng.p;
     src.tree_ids = t->ids;
-    RT_TRY(segmented_sort_gather(ids.p, off.p, Q, total, src, s, flags.p + 1, -1, longest));
+    RT_TRY(segmented_sort_gather(ids.p, off.p, Q, total, src, s, flags + 1, -1, longest));
     // the sort runs on in the order of s; its flags reach the result's status
-    RT_TRY(post_result_status(flags.p, s, res));
+    RT_TRY(post_result_status(flags, s, res));
     res->total = total;
     res->offsets = off.release();
     res->ids = ids.release();
@@ -1398,13 +1396,10 @@ rtree_status range_select(const rtree *t, const float4 *queries, int64_t Q, bool
     } else {
         RT_TRY(launch(PASS_COUNT, t, queries, Q, io, ctr.p, flags.p, s));
     }
-    RT_TRY(scan_exclusive(cnt.p, off.p, Q, s));
     DevBuf<int64_t> off_leaf(s), off_rng(s);
     if (sorted) {
         RT_TRY(off_leaf.alloc(Q + 1, "select offsets"));
         RT_TRY(off_rng.alloc(Q + 1, "select offsets"));
-        RT_TRY(scan_exclusive(cnt_leaf.p, off_leaf.p, Q, s));
-        RT_TRY(scan_exclusive(cnt_rng.p, off_rng.p, Q, s));
     }
     // the one host read: the total, the descriptor sizes and the flags
     int64_t h[3] = {0, 0, 0};
@@ -1428,7 +1423,8 @@ rtree_status range_select(const rtree *t, const float4 *queries, int64_t Q, bool
             pl.n = 4;
         }
         uint32_t w[7] = {};
-        RT_TRY(read_words(pl, s, w, sorted ? 7 : 3));
+        RT_TRY(scan_and_read({sorted ? 3 : 1, {cnt.p, cnt_leaf.p, cnt_rng.p}, {off.p, off_leaf.p, off_rng.p}, {}}, Q,
+                             pl, s, w, sorted ? 7 : 3));
         h[0] = word64(w);
         hflags = (int32_t)w[2];
         if (sorted) {
@@ -1602,11 +1598,7 @@ rtree_status range_select_host_begin(const rtree *t, const float4 *queries, int6
     } else {
         RT_TRY(launch(PASS_COUNT, t, queries, Q, io, ctr.p, flags.p, s));
     }
-    RT_TRY(scan_exclusive(cnt.p, off.p, Q, s));
-    if (sorted) {
-        RT_TRY(scan_exclusive(cnt_leaf.p, off_leaf.p, Q, s));
-        RT_TRY(scan_exclusive(cnt_rng.p, off_rng.p, Q, s));
-    }
+    RT_TRY(scan_exclusive({sorted ? 3 : 1, {cnt.p, cnt_leaf.p, cnt_rng.p}, {off.p, off_leaf.p, off_rng.p}, {}}, Q, s));
     MailboxRef plan;
     RT_TRY(mailbox_get(&plan.m));
     int64_t *mbd = reinterpret_cast<int64_t *>(plan.m.d);
@@ -1814,10 +1806,7 @@ rtree_status select_enqueue(const rtree *t, const float4 *queries, int64_t Q, in
         }
         RT_TRY(launch(PASS_BOUND, t, queries, Q, io, b.ctr, b.flags, s, nullptr, lg));
     }
-    if (wq)
-        RT_TRY(scan_exclusive(b.cnt, b.off, Q, s));
-    RT_TRY(scan_exclusive(b.cnt_leaf, b.off_leaf, Q, s));
-    RT_TRY(scan_exclusive(b.cnt_rng, b.off_rng, Q, s));
+    RT_TRY(scan_exclusive({wq ? 3 : 2, {b.cnt_leaf, b.cnt_rng, b.cnt}, {b.off_leaf, b.off_rng, b.off}, {}}, Q, s));
     SelIO so = unlimited();
     so.off_leaf = b.off_leaf;
     so.off_rng = b.off_rng;
@@ -1837,7 +1826,7 @@ rtree_status select_enqueue(const rtree *t, const float4 *queries, int64_t Q, in
         if (share_large)
             RT_TRY(launch_large(t, queries, so, lg, b.large_cap, b.task_cap, b.tasks, b.large_cur, b.flags, s));
         RT_TRY(launch(share_large ? PASS_DESC_LARGE : PASS_DESC, t, queries, Q, so, b.ctr + 1, b.flags, s, nullptr, lg));
-        RT_TRY(scan_exclusive(b.cnt, b.off, Q, s));
+        RT_TRY(scan_exclusive({1, {b.cnt}, {b.off}, {}}, Q, s));
     }
     SortSources src{};
     src.leaf = b.leaf;
