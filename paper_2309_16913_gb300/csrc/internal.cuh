@@ -469,6 +469,8 @@ rtree_status build_tree(const float4 *rects, const int32_t *ids, int64_t n, int 
 // completed, so such reads never queue behind large copies on a copy engine
 // (mailbox.cu).  Mailboxes come from a per-device pool.
 constexpr int kMailboxWords = 256;
+// A word behind them, set once the words of a host read are there.
+constexpr int kMailboxPosted = kMailboxWords;
 struct Mailbox {
     uint32_t *h = nullptr;  // host view
     uint32_t *d = nullptr;  // device view
@@ -497,6 +499,20 @@ rtree_status mailbox_wait(const Mailbox &m);
 // enqueued on s so far; rtree_result_wait reads them (word 0 bit 4: a
 // bounded device wait ran out; any other bit: a consistency check failed).
 rtree_status post_result_status(const int32_t *flags, cudaStream_t s, rtree_result *res);
+// Takes nwords that a kernel enqueued on s posts to m, as it marks them posted:
+// mailbox_expect comes before its launch, mailbox_take after.
+void mailbox_expect(const Mailbox &m);
+rtree_status mailbox_take(const Mailbox &m, cudaStream_t s, uint32_t *out, int nwords);
+// Device side: every thread that wrote words calls this, one CTA.
+__device__ __forceinline__ void mailbox_posted(uint32_t *dst)
+{
+    __threadfence_system();
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence_system();
+        *(volatile uint32_t *)(dst + kMailboxPosted) = 1u;
+    }
+}
 // Reads nwords <= kMailboxWords device words listed in l on the host (one
 // kernel stores them into a mailbox; the host waits for its event).
 rtree_status read_words(const PostList &l, cudaStream_t s, uint32_t *out, int nwords);

@@ -10,6 +10,7 @@
 // would serialize calls that are meant to overlap.  Mailboxes are pooled per
 // device: allocating page-locked memory synchronizes the device, so it only
 // happens the first time a mailbox is needed.
+#include <chrono>
 #include <mutex>
 #include <vector>
 
@@ -22,14 +23,16 @@ std::mutex g_mu;
 std::vector<Mailbox> g_free[64];
 std::vector<Mailbox> g_deferred[64];  // handed back while a post into them may still be pending
 
-__global__ void k_post(PostList l, uint32_t *__restrict__ dst)
+__global__ void k_post(const __grid_constant__ PostList l, uint32_t *__restrict__ dst, bool mark)
 {
     const int i = threadIdx.x;
-    if (i >= l.n)
-        return;
-    const uint32_t *src = static_cast<const uint32_t *>(l.src[i]);
-    for (int w = 0; w < l.words[i]; ++w)
-        dst[l.at[i] + w] = src[w];
+    if (i < l.n) {
+        const uint32_t *src = static_cast<const uint32_t *>(l.src[i]);
+        for (int w = 0; w < l.words[i]; ++w)
+            dst[l.at[i] + w] = src[w];
+    }
+    if (mark)
+        mailbox_posted(dst);
 }
 
 }  // namespace
@@ -61,7 +64,7 @@ rtree_status mailbox_get(Mailbox *m)
     Mailbox n;
     n.device = dev;
     void *h = nullptr;
-    RT_CUDA(cudaHostAlloc(&h, kMailboxWords * sizeof(uint32_t), cudaHostAllocMapped | cudaHostAllocPortable));
+    RT_CUDA(cudaHostAlloc(&h, (kMailboxWords + 4) * sizeof(uint32_t), cudaHostAllocMapped | cudaHostAllocPortable));
     n.h = static_cast<uint32_t *>(h);
     void *d = nullptr;
     cudaError_t e = cudaHostGetDevicePointer(&d, h, 0);
@@ -98,7 +101,7 @@ rtree_status post_words(const PostList &l, uint32_t *dst, cudaStream_t s)
 {
     if (l.n > 0) {
         KernelTimer kt_("mailbox_post", s);
-        k_post<<<1, 32, 0, s>>>(l, dst);
+        k_post<<<1, 32, 0, s>>>(l, dst, false);
         RT_LAUNCH();
     }
     return RTREE_OK;
@@ -145,10 +148,35 @@ rtree_status read_words(const PostList &l, cudaStream_t s, uint32_t *out, int nw
 {
     MailboxRef mb;
     RT_TRY(mailbox_get(&mb.m));
-    RT_TRY(mailbox_post(mb.m, l, s));
-    RT_TRY(mailbox_wait(mb.m));
+    mailbox_expect(mb.m);
+    {
+        KernelTimer kt_("mailbox_post", s);
+        k_post<<<1, 32, 0, s>>>(l, mb.m.d, true);
+        RT_LAUNCH();
+    }
+    return mailbox_take(mb.m, s, out, nwords);
+}
+
+void mailbox_expect(const Mailbox &m)
+{
+    __atomic_store_n(m.h + kMailboxPosted, 0u, __ATOMIC_RELEASE);
+}
+
+// The words are looked for in the mailbox itself, and the event is waited for
+// only if they do not come soon: it is complete some microseconds later.
+rtree_status mailbox_take(const Mailbox &m, cudaStream_t s, uint32_t *out, int nwords)
+{
+    RT_CUDA(cudaEventRecord(m.ev, s));
+    const auto until = std::chrono::steady_clock::now() + std::chrono::microseconds(200);
+    bool there = false;
+    do {
+        for (int i = 0; i < 64 && !there; ++i)
+            there = __atomic_load_n(m.h + kMailboxPosted, __ATOMIC_ACQUIRE) != 0;
+    } while (!there && std::chrono::steady_clock::now() < until);
+    if (!there)
+        RT_TRY(mailbox_wait(m));
     for (int i = 0; i < nwords; ++i)
-        out[i] = ((const volatile uint32_t *)mb.m.h)[i];
+        out[i] = ((const volatile uint32_t *)m.h)[i];
     return RTREE_OK;
 }
 

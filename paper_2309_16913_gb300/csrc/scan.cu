@@ -173,6 +173,7 @@ __global__ void __launch_bounds__(kThreads) k_scan_post(const __grid_constant__ 
         for (int w = 0; w < l.words[i]; ++w)
             dst[l.at[i] + w] = src[w];
     }
+    mailbox_posted(dst);
 }
 
 template <typename Tin>
@@ -237,16 +238,13 @@ rtree_status scan_and_read(const ScanJobs &j, int64_t n, const PostList &l, cuda
     }
     MailboxRef mb;
     RT_TRY(mailbox_get(&mb.m));
+    mailbox_expect(mb.m);
     {
         KernelTimer kt_("scan_post", s);
         k_scan_post<<<1, kThreads, 0, s>>>(j, (int)n, l, mb.m.d);
         RT_LAUNCH();
     }
-    RT_TRY(mailbox_post(mb.m, PostList{}, s));  // the event alone
-    RT_TRY(mailbox_wait(mb.m));
-    for (int i = 0; i < nwords; ++i)
-        out[i] = ((const volatile uint32_t *)mb.m.h)[i];
-    return RTREE_OK;
+    return mailbox_take(mb.m, s, out, nwords);
 }
 
 }  // namespace rt
