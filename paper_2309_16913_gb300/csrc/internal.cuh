@@ -329,7 +329,10 @@ struct ScanJobs {  // arrays of one length
     int count;
     const int32_t *in[kScanJobs];
     int64_t *out[kScanJobs];
-    int32_t *most[kScanJobs];  // raised to the array's largest value, if given
+    // if given: [0] is raised to the array's largest value, and the sum of its
+    // values above `over` is added to the 64-bit word at [2]
+    int32_t *most[kScanJobs];
+    int32_t over;
 };
 rtree_status scan_exclusive(const ScanJobs &j, int64_t n, cudaStream_t s);
 // The same, and then a host read of words that the scans or what precedes them
@@ -449,10 +452,12 @@ struct SortSources {
 // out_cap (default: total) in `out` are skipped.  Offsets may be absolute
 // positions in a larger `out`, so a run of segments can be sorted on its
 // own.  No segment is longer than max_len: classes of longer ones are not
-// launched.  Device-side capacity problems set bits in *flags.
+// launched.  Segments longer than kSortWhole hold at most long_ids ids (default:
+// total); they alone need scratch.  Device-side capacity problems set bits in *flags.
+constexpr int kSortWhole = 32256;  // ids that one CTA sorts; longer segments are split
 rtree_status segmented_sort_gather(int32_t *out, const int64_t *off, int64_t nseg, int64_t total,
                                    const SortSources &src, cudaStream_t s, int32_t *flags,
-                                   int64_t out_cap = -1, int64_t max_len = INT64_MAX);
+                                   int64_t out_cap = -1, int64_t max_len = INT64_MAX, int64_t long_ids = -1);
 
 // Sorts every segment ids[offsets[i] .. offsets[i+1]) ascending, in place.
 rtree_status segmented_sort(int32_t *ids, const int64_t *offsets, int64_t nseg, int64_t total,

@@ -51,12 +51,14 @@ __device__ __forceinline__ T block_excl_scan(T v, T &total)
     return r;
 }
 
-// Raises *most to the warp's largest value (one atomic a warp).
-__device__ __forceinline__ void raise(int32_t *most, int32_t v)
+// Notes a thread's largest value and the sum of those above j.over (ScanJobs::most).
+__device__ __forceinline__ void note(int32_t *most, int32_t v, int64_t above)
 {
     v = __reduce_max_sync(RT_FULL, v);
     if ((threadIdx.x & 31) == 0 && v > 0)
         atomicMax(most, v);
+    if (above > 0)  // seldom
+        atomicAdd(reinterpret_cast<unsigned long long *>(most + 2), (unsigned long long)above);
 }
 
 // The arrays of one launch (blockIdx.y): base, if given, is each tile's start.
@@ -65,7 +67,8 @@ struct Scans {
     const Tin *in[kScanJobs];
     int64_t *out[kScanJobs];
     const int64_t *base[kScanJobs];
-    int32_t *most[kScanJobs];  // raised to the largest value, if given
+    int32_t *most[kScanJobs];
+    int32_t over;
 };
 
 template <typename Tin>
@@ -73,7 +76,7 @@ __global__ void __launch_bounds__(kThreads) k_tile_reduce(const __grid_constant_
 {
     const Tin *__restrict__ in = j.in[blockIdx.y];
     const int64_t base = (int64_t)blockIdx.x * kTile;
-    int64_t acc = 0;
+    int64_t acc = 0, above = 0;
     Tin big = 0;
 #pragma unroll
     for (int i = 0; i < kItems; ++i) {
@@ -81,10 +84,11 @@ __global__ void __launch_bounds__(kThreads) k_tile_reduce(const __grid_constant_
         if (k < n) {
             acc += (int64_t)in[k];
             big = in[k] > big ? in[k] : big;
+            above += in[k] > j.over ? (int64_t)in[k] : 0;
         }
     }
     if (j.most[blockIdx.y])
-        raise(j.most[blockIdx.y], (int32_t)big);
+        note(j.most[blockIdx.y], (int32_t)big, above);
     int64_t total;
     block_excl_scan<int64_t>(acc, total);
     if (threadIdx.x == 0)
@@ -106,15 +110,16 @@ __global__ void __launch_bounds__(kThreads) k_tile_scan(const __grid_constant__ 
         sm[p] = k < n ? (int64_t)in[k] : 0;
     }
     __syncthreads();
-    int64_t v[kItems], run = 0, big = 0;
+    int64_t v[kItems], run = 0, big = 0, above = 0;
 #pragma unroll
     for (int i = 0; i < kItems; ++i) {
         v[i] = sm[threadIdx.x * kItems + i];
         run += v[i];
         big = v[i] > big ? v[i] : big;
+        above += v[i] > j.over ? v[i] : 0;
     }
     if (j.most[blockIdx.y])
-        raise(j.most[blockIdx.y], (int32_t)big);
+        note(j.most[blockIdx.y], (int32_t)big, above);
     int64_t total;
     int64_t pre = block_excl_scan<int64_t>(run, total);
     const int64_t tb = j.base[blockIdx.y] ? j.base[blockIdx.y][blockIdx.x] : 0;
@@ -145,7 +150,7 @@ __global__ void __launch_bounds__(kThreads) k_scan_post(const __grid_constant__ 
     for (int a = 0; a < j.count; ++a) {
         const int32_t *__restrict__ in = j.in[a];
         const int k0 = threadIdx.x * kItems;
-        int64_t v[kItems], run = 0;
+        int64_t v[kItems], run = 0, above = 0;
         int32_t big = 0;
 #pragma unroll
         for (int i = 0; i < kItems; ++i) {
@@ -153,9 +158,10 @@ __global__ void __launch_bounds__(kThreads) k_scan_post(const __grid_constant__ 
             v[i] = run;
             run += x;
             big = x > big ? x : big;
+            above += x > j.over ? x : 0;
         }
         if (j.most[a])
-            raise(j.most[a], big);
+            note(j.most[a], big, above);
         int64_t total;
         const int64_t pre = block_excl_scan<int64_t>(run, total);
 #pragma unroll
@@ -227,6 +233,7 @@ rtree_status scan_exclusive(const ScanJobs &j, int64_t n, cudaStream_t s)
         jobs.out[a] = j.out[a];
         jobs.most[a] = j.most[a];
     }
+    jobs.over = j.over;
     return scan_impl<int32_t>(jobs, j.count, n, s);
 }
 

@@ -43,12 +43,13 @@ constexpr uint32_t kSign = 0x80000000u;
 constexpr int cta_ids(int threads, int items) { return threads / 32 * (items / 8) * 252; }
 constexpr int kMidMax = cta_ids(512, 32);   // longest segment below the largest class: 16128
 constexpr int kCtaTop = cta_ids(1024, 32);  // longest segment of a CTA sort: 32256
+static_assert(kCtaTop == kSortWhole, "the caller counts the ids that need scratch");
 
 // Segment classes (index into the class lists).
 enum {
     C_WARP = 0,  // warp sort
     C_CTA1K, C_CTA2K, C_CTA4K, C_CTA8K, C_CTA16K, C_CTA32K,  // CTA sorts
-    C_LARGE,                          // MSD partition first
+    C_LARGE,                          // split into buckets first
     C_COUNT
 };
 enum { HDR_SCRATCH = C_COUNT, HDR_BUCKETS, HDR_OVERSIZE, HDR_UNITS, HDR_WORDS };
@@ -1559,7 +1560,7 @@ struct Fork {
 
 rtree_status segmented_sort_gather(int32_t *out, const int64_t *offsets, int64_t nseg, int64_t total,
                                    const SortSources &S, cudaStream_t s, int32_t *flags, int64_t out_cap,
-                                   int64_t max_len)
+                                   int64_t max_len, int64_t long_ids)
 {
     if (nseg <= 0 || total <= 0)
         return RTREE_OK;
@@ -1574,8 +1575,8 @@ rtree_status segmented_sort_gather(int32_t *out, const int64_t *offsets, int64_t
     // Every list length stays on the device; the launches below are sized
     // by upper bounds and read the actual lengths themselves, so the whole
     // sort is enqueued without a host round trip.
-    const int64_t max_large = total / (kCtaTop + 1) + 1 < nseg ? total / (kCtaTop + 1) + 1 : nseg;
-    const int64_t scratch_cap = total;
+    const int64_t scratch_cap = long_ids < 0 || long_ids > total ? total : long_ids;
+    const int64_t max_large = scratch_cap / (kCtaTop + 1) + 1 < nseg ? scratch_cap / (kCtaTop + 1) + 1 : nseg;
     // buckets: one per kBucketIds ids begun, and the last of each segment
     const int64_t desc_cap = 2 * max_large + scratch_cap / kBucketIds + 256;
     const int64_t unit_cap = max_large + scratch_cap / kUnit;

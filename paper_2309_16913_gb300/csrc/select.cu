@@ -1236,13 +1236,14 @@ rtree_status range_select_bounded(const rtree *t, const float4 *queries, int64_t
     RT_TRY(cnt_leaf.alloc(Q, "select counts"));
     RT_TRY(cnt_rng.alloc(Q, "select counts"));
     // work counters of two passes, large queries and tasks for them; then the
-    // flags: [0] select passes, [1] sort, [2] the longest result
-    RT_TRY(ctr.alloc(6, "select work counters and flags"));
+    // flags: [0] select passes, [1] sort, [2] the longest result, [4], [5] the
+    // ids of results that the sort must split
+    RT_TRY(ctr.alloc(7, "select work counters and flags"));
     int32_t *flags = reinterpret_cast<int32_t *>(ctr.p + 4);
     RT_TRY(large.alloc(large_cap, "select large queries"));
     RT_TRY(off_leaf.alloc(Q + 1, "select offsets"));
     RT_TRY(off_rng.alloc(Q + 1, "select offsets"));
-    RT_CUDA(cudaMemsetAsync(ctr.p, 0, 6 * sizeof(unsigned long long), s));
+    RT_CUDA(cudaMemsetAsync(ctr.p, 0, 7 * sizeof(unsigned long long), s));
     if (order == RTREE_ORDER_HILBERT) {
         RT_TRY(perm.alloc(Q, "query order"));
         RT_TRY(hilbert_order(t, queries, Q, perm.p, s));
@@ -1312,21 +1313,23 @@ rtree_status range_select_bounded(const rtree *t, const float4 *queries, int64_t
     }
     RT_TRY(launch(pass, t, queries, Q, so, ctr.p + 1, flags, s, nullptr, lg));
     // host read 2 of 2: the total (it sizes the result and is returned) and the
-    // longest result (it says which sort classes are needed)
-    int64_t total = 0, longest = 0;
+    // longest result and the ids in long ones (they say which sort classes are
+    // needed and size the scratch)
+    int64_t total = 0, longest = 0, long_ids = 0;
     {
         PostList pl{};
         pl.src[0] = off.p + Q;
         pl.words[0] = 2;
         pl.at[0] = 0;
         pl.src[1] = flags;
-        pl.words[1] = 3;
+        pl.words[1] = 6;
         pl.at[1] = 2;
         pl.n = 2;
-        uint32_t w[5];
-        RT_TRY(scan_and_read({1, {cnt.p}, {off.p}, {flags + 2}}, Q, pl, s, w, 5));
+        uint32_t w[8];
+        RT_TRY(scan_and_read({1, {cnt.p}, {off.p}, {flags + 2}, kSortWhole}, Q, pl, s, w, 8));
         total = word64(w);
         longest = (int32_t)w[4];
+        long_ids = word64(w + 6);
         if (w[2])
             return fail(RTREE_EINTERNAL, "select descriptor pass reported device flags 0x%x", w[2]);
     }
@@ -1339,7 +1342,7 @@ rtree_status range_select_bounded(const rtree *t, const float4 *queries, int64_t
     src.rng = rng.p;
     src.off_rng = off_rng.p;
     src.tree_ids = t->ids;
-    RT_TRY(segmented_sort_gather(ids.p, off.p, Q, total, src, s, flags + 1, -1, longest));
+    RT_TRY(segmented_sort_gather(ids.p, off.p, Q, total, src, s, flags + 1, -1, longest, long_ids));
     // the sort runs on in the order of s; its flags reach the result's status
     RT_TRY(post_result_status(flags, s, res));
     res->total = total;
