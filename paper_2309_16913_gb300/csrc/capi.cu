@@ -59,7 +59,58 @@ void setup_device_pool(int dev)
     done[dev] = true;
 }
 
-rtree_status dmalloc(void **p, size_t bytes, cudaStream_t s, const char *what)
+namespace {
+// The pool of large results on the current device (null: the default one).
+// It keeps freed blocks up to a quarter of the device's memory.
+cudaMemPool_t result_pool()
+{
+    static std::mutex mu;
+    static cudaMemPool_t pools[64] = {};
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64)
+        return nullptr;
+    std::lock_guard<std::mutex> g(mu);
+    if (!pools[dev]) {
+        cudaMemPoolProps props{};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = dev;
+        size_t idle = 0, all = 0;
+        cudaMemPool_t pool = nullptr;
+        if (cudaMemGetInfo(&idle, &all) == cudaSuccess && cudaMemPoolCreate(&pool, &props) == cudaSuccess) {
+            uint64_t keep = all / 4;
+            cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+            pools[dev] = pool;
+        }
+        cudaGetLastError();
+    }
+    return pools[dev];
+}
+
+// Gives what the pools keep for later calls back to the device.
+void trim_pools(cudaStream_t s)
+{
+    cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
+    int dev = 0;
+    cudaMemPool_t pool = nullptr;
+    if (cudaStreamIsCapturing(s, &capturing) == cudaSuccess && capturing == cudaStreamCaptureStatusNone &&
+        cudaGetDevice(&dev) == cudaSuccess && cudaDeviceSynchronize() == cudaSuccess) {
+        if (cudaDeviceGetDefaultMemPool(&pool, dev) == cudaSuccess)
+            cudaMemPoolTrimTo(pool, 0);
+        if ((pool = result_pool()))
+            cudaMemPoolTrimTo(pool, 0);
+    }
+    cudaGetLastError();
+}
+}  // namespace
+
+// Where no free block of a pool is large enough, the pool maps one together, at
+// a cost that grows with its size, and a caller that drops a result after the
+// next call makes large blocks of scratch and of results change places.  Three
+// batches of 1M queries on 11M rectangles in turn, 1.4G ids each, took 12.9 to
+// 16.3 ms a call, one of them alone 11.0.  With sizes in steps and results apart
+// both take 11.0.
+rtree_status dmalloc(void **p, size_t bytes, cudaStream_t s, const char *what, Block kind)
 {
     *p = nullptr;
     long long c = g_alloc_countdown.load();
@@ -76,7 +127,21 @@ rtree_status dmalloc(void **p, size_t bytes, cudaStream_t s, const char *what)
             return fail(RTREE_ENOMEM, "the tree's allocator returned no memory: %zu bytes for %s", bytes, what);
         return RTREE_OK;
     }
-    cudaError_t e = cudaMallocAsync(p, bytes, s);
+    size_t step = 1;
+    cudaMemPool_t pool = nullptr;
+    if (kind != EXACT && bytes >= ((size_t)64 << 20)) {
+        while (step <= bytes >> 5)
+            step <<= 1;
+        if (kind == RESULT)
+            pool = result_pool();
+    }
+    const size_t size = (bytes + step - 1) / step * step;
+    cudaError_t e = pool ? cudaMallocFromPoolAsync(p, size, pool, s) : cudaMallocAsync(p, size, s);
+    if (e == cudaErrorMemoryAllocation) {  // once more without what is kept, and exactly
+        cudaGetLastError();
+        trim_pools(s);
+        e = cudaMallocAsync(p, bytes, s);
+    }
     if (e == cudaErrorMemoryAllocation) {
         cudaGetLastError();
         *p = nullptr;

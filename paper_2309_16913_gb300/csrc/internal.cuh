@@ -54,7 +54,10 @@ struct AllocScope {
 // Device memory from t_alloc, usable in the order of stream s.  A host-side
 // counter can make the k-th allocation fail (fault injection for tests; no
 // GPU fault is involved).
-rtree_status dmalloc(void **p, size_t bytes, cudaStream_t s, const char *what);
+// Blocks of 64 MB and more that are not EXACT may be up to a sixteenth larger;
+// results come from a pool of their own.
+enum Block { EXACT, SCRATCH, RESULT };
+rtree_status dmalloc(void **p, size_t bytes, cudaStream_t s, const char *what, Block kind = EXACT);
 // Keeps freed blocks in the device's default pool between calls (once per device).
 void setup_device_pool(int dev);
 // Releases a tree's device arrays (not the struct): after the whole device
@@ -97,10 +100,10 @@ struct DevBuf {
     DevBuf(const DevBuf &) = delete;
     DevBuf &operator=(const DevBuf &) = delete;
     ~DevBuf() { reset(); }
-    rtree_status alloc(size_t n, const char *what)
+    rtree_status alloc(size_t n, const char *what, Block kind = EXACT)
     {
         reset();
-        return dmalloc(reinterpret_cast<void **>(&p), (n ? n : 1) * sizeof(T), s, what);
+        return dmalloc(reinterpret_cast<void **>(&p), (n ? n : 1) * sizeof(T), s, what, kind);
     }
     void reset()
     {

@@ -1621,7 +1621,7 @@ rtree_status segmented_sort_gather(int32_t *out, const int64_t *offsets, int64_t
     DevBuf<uint16_t> long_table(s);
     DevBuf<Unit> units(s);
     if (long_path) {
-        RT_TRY(scratch.alloc(scratch_cap, "sort scratch"));
+        RT_TRY(scratch.alloc(scratch_cap, "sort scratch", long_ids >= 0 ? SCRATCH : EXACT));
         RT_TRY(buckets.alloc(desc_cap, "sort buckets"));
         RT_TRY(oversize.alloc(desc_cap, "sort buckets"));
         RT_TRY(crowded2.alloc(desc_cap, "sort crowded list"));

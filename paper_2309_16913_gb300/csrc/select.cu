@@ -1293,8 +1293,8 @@ rtree_status range_select_bounded(const rtree *t, const float4 *queries, int64_t
 
     DevBuf<int32_t> leaf(s);
     DevBuf<int2> rng(s);
-    RT_TRY(leaf.alloc(h[0], "select leaf hits"));
-    RT_TRY(rng.alloc(h[1], "select whole subtrees"));
+    RT_TRY(leaf.alloc(h[0], "select leaf hits", SCRATCH));
+    RT_TRY(rng.alloc(h[1], "select whole subtrees", SCRATCH));
     SelIO so = unlimited();
     so.off_leaf = off_leaf.p;
     so.off_rng = off_rng.p;
@@ -1334,7 +1334,7 @@ rtree_status range_select_bounded(const rtree *t, const float4 *queries, int64_t
             return fail(RTREE_EINTERNAL, "select descriptor pass reported device flags 0x%x", w[2]);
     }
     DevBuf<int32_t> ids(s);
-    RT_TRY(ids.alloc(total, "select ids"));
+    RT_TRY(ids.alloc(total, "select ids", RESULT));
     SortSources src{};
     src.leaf = leaf.p;
     src.off_leaf = off_leaf.p;
@@ -1447,7 +1447,7 @@ rtree_status range_select(const rtree *t, const float4 *queries, int64_t Q, bool
     }
 
     DevBuf<int32_t> ids(s);
-    RT_TRY(ids.alloc(total, "select ids"));
+    RT_TRY(ids.alloc(total, "select ids", RESULT));
     if (!sorted) {
         SelIO so = unlimited();
         so.offsets = off.p;
@@ -1462,8 +1462,8 @@ rtree_status range_select(const rtree *t, const float4 *queries, int64_t Q, bool
     } else {
         DevBuf<int32_t> leaf(s);
         DevBuf<int2> rng(s);
-        RT_TRY(leaf.alloc(h[1], "select leaf hits"));
-        RT_TRY(rng.alloc(h[2], "select whole subtrees"));
+        RT_TRY(leaf.alloc(h[1], "select leaf hits", SCRATCH));
+        RT_TRY(rng.alloc(h[2], "select whole subtrees", SCRATCH));
         SelIO so = unlimited();
         so.off_leaf = off_leaf.p;
         so.off_rng = off_rng.p;
@@ -1639,10 +1639,10 @@ rtree_status range_select_host_begin(const rtree *t, const float4 *queries, int6
     DevBuf<int32_t> ids(s), cursors(s), leaf(s);
     DevBuf<int2> rng(s);
     DevBuf<uint32_t> cperm(s);
-    RT_TRY(ids.alloc(total, "select ids"));
+    RT_TRY(ids.alloc(total, "select ids", RESULT));
     if (sorted) {
-        RT_TRY(leaf.alloc(leaf_total, "select leaf hits"));
-        RT_TRY(rng.alloc(rng_total, "select whole subtrees"));
+        RT_TRY(leaf.alloc(leaf_total, "select leaf hits", SCRATCH));
+        RT_TRY(rng.alloc(rng_total, "select whole subtrees", SCRATCH));
     }
     if (wq) {
         RT_TRY(cursors.alloc(2 * Q, "select cursors"));
