@@ -253,8 +253,8 @@ def algorithmic_bytes(stats, F, Q, seg_sizes):
     Node visit: F entry MBRs (16 B each, unused slots included) + 16 B of node
     metadata.  Whole subtree: 16 B metadata read + 8 B (lo, hi) written.  Leaf
     hit: 4 B id read + 4 B written.  Sorting an id: 4 B gathered + 4 B written
-    (segments over 40960 ids take the MSD path, which adds three reads and one
-    write for the split).
+    (segments over 32256 ids are first gathered and scattered into buckets,
+    which adds two reads and two writes).
     The bound pass visits the internal nodes only; the descriptor pass after
     it also writes two exact counts per query.
     """
@@ -539,8 +539,8 @@ def run_ours(args):
         roofline["traffic_note"] = traffic_note
     if dominant.startswith("sort_"):
         roofline["note"] = ("sort_all = the whole segmented sort (warp, CTA and long-segment classes on side "
-                            "streams), wall time of its span; 8 B per id (gathered + written), 24 B more per id of "
-                            "segments over 40960; bound by shared-memory work and per-segment latency, not by HBM "
+                            "streams), wall time of its span; 8 B per id (gathered + written), 16 B more per id of "
+                            "segments over 32256; bound by shared-memory work and per-segment latency, not by HBM "
                             "(ncu: 45-53% issue active, a few % of DRAM peak)")
     # the node-test kernels, each against HBM (ncu DRAM bytes) and issue slots
     roofline_node_test = node_test_roofline(kern, algo, stats, args.steps, hbm, peak_kind, clk, F, layout)

@@ -481,10 +481,10 @@ enum { RTREE_PRUNE_AUTO = 0, /* prune when both trees have sorted children */
 /* How the node pairs of the traversal are scheduled (same pairs either way). */
 enum { RTREE_JOIN_AUTO = 0,   /* the library's choice (RTREE_JOIN_LEVELS: faster on the joins measured;
                                  the queue's counters see one atomic per node pair or more, while a
-                                 level costs one launch and one host read) */
+                                 level costs one launch) */
        RTREE_JOIN_LEVELS = 1, /* one launch per tree level over that level's node pairs, the pairs
-                                 found on one level being the next level's work (count, scan and
-                                 scatter per level; the call returns when its work has finished) */
+                                 found on one level being the next level's work (one pass a level;
+                                 the call returns when its work has finished) */
        RTREE_JOIN_QUEUE = 2 };/* a persistent grid pulls node pairs from a device work queue and
                                  publishes the qualifying child pairs to it; a count pass, one host
                                  read of the total, a scatter pass and the pair sort.  The call
