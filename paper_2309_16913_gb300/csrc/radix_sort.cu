@@ -17,6 +17,7 @@
 // count), tiles are taken in order inside a CTA, and CTAs own consecutive
 // runs.
 #include <algorithm>
+#include <mutex>
 #include <type_traits>
 
 #include "internal.cuh"
@@ -32,6 +33,28 @@ constexpr int kBins = 256;
 constexpr int kWide = 1024;               // digits of up to 10 bits, where they save a pass
 constexpr int kWarpRun = 32 * kItems;     // contiguous items owned by one warp
 static_assert(kThreads == kBins, "one thread per digit");
+
+// A number of each device, worked out at its first use there: how many CTAs of a
+// kernel fit, after the kernel's attributes have been set (which CUDA keeps per
+// device too, so a number of the whole process would leave the others without).
+class PerDevice {
+    static constexpr int kMaxDev = 64;
+    std::once_flag once_[kMaxDev];
+    int value_[kMaxDev] = {};
+
+public:
+    template <typename F>
+    int get(F f)
+    {
+        int dev = 0;
+        if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= kMaxDev) {
+            cudaGetLastError();
+            return f();
+        }
+        std::call_once(once_[dev], [&] { value_[dev] = f(); });
+        return value_[dev];
+    }
+};
 
 // Tiles [t0, t1) of CTA c out of G (balanced: they differ by at most one).
 __device__ __forceinline__ void run_of(int64_t ntiles, int G, int c, int64_t &t0, int64_t &t1)
@@ -289,7 +312,8 @@ __global__ void __launch_bounds__(kThreads, 4)
 template <int BINS, int END>
 int grid_for(int64_t ntiles)
 {
-    static const int per_sm = [] {  // initialised once, thread-safely
+    static PerDevice ctas;
+    const int per_sm = ctas.get([] {
         int v = 0;
         if (cudaFuncSetAttribute(k_scatter<BINS, END>, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                  (int)sizeof(ScatterSmem<BINS>)) != cudaSuccess ||
@@ -299,7 +323,7 @@ int grid_for(int64_t ntiles)
             v = 1;
         }
         return v;
-    }();
+    });
     const int64_t g = (int64_t)per_sm * sm_count();
     return (int)(ntiles < g ? ntiles : g);
 }
@@ -660,16 +684,16 @@ bool cluster_fits(int C)
     return false;
 }
 
-// CTAs a cluster can have (16, 8, or 0 if there is none).
+// CTAs a cluster can have on the current device (16, 8, or 0 if there is none).
 int cluster_ctas()
 {
-    static const int most = [] {  // initialised once, thread-safely
+    static PerDevice most;
+    return most.get([] {
         for (int c = kCluster; c >= 8; c >>= 1)
             if (cluster_fits<SRC_PAIRS>(c) && cluster_fits<SRC_BOXES>(c) && cluster_fits<SRC_TABLE>(c))
                 return c;
         return 0;
-    }();
-    return most;
+    });
 }
 
 template <int SRC>
