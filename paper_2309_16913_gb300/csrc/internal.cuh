@@ -360,7 +360,7 @@ struct SelIO {
     int32_t *counts;          // COUNT: ids per query
     int32_t *counts_leaf;     // COUNT, optional: ids found one by one in leaves
     int32_t *counts_rng;      // COUNT, optional: whole subtrees taken
-    const int64_t *offsets;   // SCATTER: CSR offsets of the ids
+    const int64_t *offsets;   // SCATTER, and DESC of the work queue: CSR offsets of the ids
     int32_t *out;             // SCATTER: the ids, traversal order
     const int64_t *off_leaf;  // DESC: offsets of the leaf hits
     const int64_t *off_rng;   // DESC: offsets of the whole-subtree ranges
@@ -370,7 +370,7 @@ struct SelIO {
     // pass), because several warps may emit results for one query.
     int32_t *cur_ids;         // SCATTER
     int32_t *cur_leaf;        // DESC
-    int32_t *cur_rng;         // DESC
+    int32_t *cur_rng;         // DESC; negative in the end: the query is to be left out
     // Buffer capacities (entries); writes at or past them are dropped.  Only
     // the graph-captured plan sizes buffers before knowing the totals.
     int64_t out_cap;
@@ -446,6 +446,7 @@ struct SortSources {
     const int32_t *tree_ids;
     int64_t leaf_cap;  // 0: unchecked; else segments reaching past are skipped
     int64_t rng_cap;
+    const int32_t *left_out;  // if set, segments with a negative value are skipped
 };
 
 // Writes segment i's ids, sorted ascending (signed), to

@@ -99,8 +99,9 @@ __global__ void __launch_bounds__(kClassThreads)
         const int64_t i = b + threadIdx.x;
         int64_t len = i < nseg ? off[i + 1] - off[i] : 0;
         // a segment whose output or sources reach past a buffer's capacity is
-        // skipped (the caller sees the totals exceed the capacities)
-        if (len > 0 && (off[i + 1] > out_cap ||
+        // skipped (the caller sees the totals exceed the capacities), and so is
+        // one whose sources are not all there (the caller's flags say so)
+        if (len > 0 && (off[i + 1] > out_cap || (S.left_out && S.left_out[i] < 0) ||
                         (S.leaf_cap && leaf_end(S, i) > S.leaf_cap) ||
                         (S.rng && S.rng_cap && S.off_rng[i + 1] > S.rng_cap)))
             len = 0;

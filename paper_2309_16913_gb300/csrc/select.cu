@@ -765,15 +765,23 @@ __global__ void k_wq_check(const SelIO io, int pass, int64_t Q, int32_t *__restr
 
 // After a work-queue descriptor pass: the lengths in the range entries become
 // places (one warp per query scans them).
-__global__ void k_wq_places(const SelIO io, int64_t Q)
+// A pass that gave up waiting leaves slots unset, and one behind a count pass
+// that gave up has slots for some of the runs only.  The sort copies from where
+// the entries say, so a query whose entries are not all there, or whose runs and
+// leaf hits do not make up its ids, is left out of it (cur_rng < 0).
+__global__ void k_wq_places(const SelIO io, int64_t Q, int32_t *__restrict__ flags)
 {
     const int lane = threadIdx.x & 31;
     const int64_t warp = (blockIdx.x * (int64_t)blockDim.x + threadIdx.x) >> 5;
     const int64_t nwarps = ((int64_t)gridDim.x * blockDim.x) >> 5;
     for (int64_t i = warp; i < Q; i += nwarps) {
-        const int64_t r0 = io.off_rng[i], r1 = io.off_rng[i + 1] < io.rng_cap ? io.off_rng[i + 1] : io.rng_cap;
+        const int64_t r0 = io.off_rng[i], r1 = io.off_rng[i + 1];
+        const int64_t nl = io.off_leaf[i + 1] - io.off_leaf[i], n = io.offsets[i + 1] - io.offsets[i];
+        if (r1 > io.rng_cap)
+            continue;  // the sort leaves it out by itself
+        const bool all = io.cur_rng[i] == r1 - r0 && io.cur_leaf[i] == nl;
         int place = 0;
-        for (int64_t b = r0; b < r1; b += 32) {
+        for (int64_t b = r0; all && b < r1; b += 32) {
             const int len = b + lane < r1 ? io.rng_out[b + lane].y : 0;
             int inc = len;
 #pragma unroll
@@ -785,6 +793,11 @@ __global__ void k_wq_places(const SelIO io, int64_t Q)
             if (b + lane < r1)
                 io.rng_out[b + lane].y = place + inc - len;
             place += __shfl_sync(RT_FULL, inc, 31);
+        }
+        __syncwarp();
+        if (lane == 0 && !(all && place == n - nl)) {
+            io.cur_rng[i] = -1;
+            atomicOr(flags, FLAG_COUNT_MISMATCH);
         }
     }
 }
@@ -1125,7 +1138,7 @@ rtree_status launch_wq(int pass, const rtree *t, const float4 *q, int64_t Q, con
     if (pass == PASS_DESC) {
         KernelTimer kt_("wq_places", s);
         const int64_t b = (Q + 7) / 8;
-        k_wq_places<<<(unsigned)(b > 65536 ? 65536 : b), 256, 0, s>>>(io, Q);
+        k_wq_places<<<(unsigned)(b > 65536 ? 65536 : b), 256, 0, s>>>(io, Q, flags);
         RT_LAUNCH();
     }
     return RTREE_OK;
@@ -1471,6 +1484,7 @@ rtree_status range_select(const rtree *t, const float4 *queries, int64_t Q, bool
         so.rng_out = rng.p;
         so.order = perm.p;
         if (wq) {
+            so.offsets = off.p;
             so.cur_leaf = cursors.p;
             so.cur_rng = cursors.p + Q;
             RT_TRY(launch_wq(PASS_DESC, t, queries, Q, so, flags.p, s));
@@ -1483,6 +1497,7 @@ rtree_status range_select(const rtree *t, const float4 *queries, int64_t Q, bool
         src.rng = rng.p;
         src.off_rng = off_rng.p;
         src.tree_ids = t->ids;
+        src.left_out = so.cur_rng;
         RT_TRY(segmented_sort_gather(ids.p, off.p, Q, total, src, s, flags.p + 1));
     }
     // the second pass (and sort) run on in the order of s; their flags reach
@@ -1699,6 +1714,7 @@ rtree_status range_select_host_begin(const rtree *t, const float4 *queries, int6
             so.leaf_out = leaf.p;
             so.rng_out = rng.p;
             if (wq) {
+                so.offsets = off.p + c0;
                 so.cur_leaf = cursors.p + c0;
                 so.cur_rng = cursors.p + Q + c0;
                 RT_TRY(launch_wq(PASS_DESC, t, qk, qc, so, flags.p, s));
@@ -1711,6 +1727,7 @@ rtree_status range_select_host_begin(const rtree *t, const float4 *queries, int6
             src.rng = rng.p;
             src.off_rng = off_rng.p + c0;
             src.tree_ids = t->ids;
+            src.left_out = so.cur_rng;
             RT_TRY(segmented_sort_gather(ids.p, off.p + c0, qc, boff[k + 1] - boff[k], src, s,
                                          flags.p + 1, total));
         }
@@ -1819,6 +1836,7 @@ rtree_status select_enqueue(const rtree *t, const float4 *queries, int64_t Q, in
     so.rng_cap = b.rng_cap;
     if (wq) {
         RT_CUDA(cudaMemsetAsync(b.cursors, 0, 2 * Q * sizeof(int32_t), s));
+        so.offsets = b.off;
         so.cur_leaf = b.cursors;
         so.cur_rng = b.cursors + Q;
         RT_TRY(launch_wq(PASS_DESC, t, queries, Q, so, b.flags, s, nullptr, b.wq_items, b.wq_cap,
@@ -1840,6 +1858,7 @@ rtree_status select_enqueue(const rtree *t, const float4 *queries, int64_t Q, in
     src.tree_ids = t->ids;
     src.leaf_cap = b.leaf_cap;
     src.rng_cap = b.rng_cap;
+    src.left_out = so.cur_rng;
     return segmented_sort_gather(b.ids, b.off, Q, b.ids_cap, src, s, b.flags + 1);
 }
 
