@@ -87,14 +87,16 @@ cudaMemPool_t result_pool()
     return pools[dev];
 }
 
-// Gives what the pools keep for later calls back to the device.
+// Gives what the pools keep for later calls back to the device, what was freed
+// on s included.  (Waiting for the whole device would end the capture of any
+// stream that another thread is recording.)
 void trim_pools(cudaStream_t s)
 {
     cudaStreamCaptureStatus capturing = cudaStreamCaptureStatusNone;
     int dev = 0;
     cudaMemPool_t pool = nullptr;
     if (cudaStreamIsCapturing(s, &capturing) == cudaSuccess && capturing == cudaStreamCaptureStatusNone &&
-        cudaGetDevice(&dev) == cudaSuccess && cudaDeviceSynchronize() == cudaSuccess) {
+        cudaGetDevice(&dev) == cudaSuccess && cudaStreamSynchronize(s) == cudaSuccess) {
         if (cudaDeviceGetDefaultMemPool(&pool, dev) == cudaSuccess)
             cudaMemPoolTrimTo(pool, 0);
         if ((pool = result_pool()))
