@@ -33,7 +33,14 @@
  * (rtree_allocator_t); every device buffer the library allocates for that
  * tree -- the tree itself, the scratch of calls on it, and their results --
  * is taken from it and given back to it.  NULL selects cudaMallocAsync and
- * cudaFreeAsync on the call's stream (the device's default memory pool).
+ * cudaFreeAsync on the call's stream (the device's default memory pool, whose
+ * release threshold the library raises so that it keeps freed blocks).  Select
+ * results of 64 MB and more then come from a memory pool of the library's own,
+ * which keeps freed blocks up to a quarter of the device's memory: rtree_trim
+ * gives them back.  A caller who sets the default pool's release threshold to
+ * another value, or makes another pool the device's current one, has those
+ * results from that pool as well, from the next call on.  Blocks of 64 MB and
+ * more may be up to a sixteenth larger than what they hold.
  *
  * Errors.  Every call returns an rtree_status; on failure no output is
  * produced (output handles are set to NULL) and rtree_last_error() describes
@@ -164,11 +171,11 @@ typedef struct rtree_allocator {
  * rects: n*4 floats, ids: n int32 (NULL -> ids 0..n-1); host or device.
  * n = 0 builds a valid empty tree.  n must be < 2^31.
  * The inputs are copied; the caller keeps ownership and may free them once
- * the call returns.  alloc: the tree's device-memory hook (NULL: the default
- * pool).  *out receives the tree (free with rtree_free).  The call returns
- * once the inputs have been checked on the device (one host read) and the
- * packing is enqueued on `stream`; work enqueued on `stream` afterwards may
- * use the tree.
+ * the call returns.  alloc: the tree's device-memory hook (NULL: the device's
+ * memory pools, see above).  *out receives the tree (free with rtree_free).
+ * The call returns once the inputs have been checked on the device (one host
+ * read) and the packing is enqueued on `stream`; work enqueued on `stream`
+ * afterwards may use the tree.
  * Errors: RTREE_EINVAL for a NaN coordinate, xmin > xmax or ymin > ymax in
  * any row, an unsupported fanout/layout, an allocator with a NULL function,
  * or NULL out; RTREE_ENOMEM.
@@ -540,6 +547,13 @@ RTREE_API void rtree_result_free(rtree_result_t *res);
  * other streams is not waited for.  The handle is invalid on return.  NULL
  * is ignored. */
 RTREE_API void rtree_result_free_async(rtree_result_t *res, void *stream);
+
+/* Gives back to the device what the library's pool of large results on
+ * `device` (< 0: the current one) keeps for later calls.  (The default memory
+ * pool is the caller's to trim: cudaMemPoolTrimTo.)  Does not wait for the
+ * device: blocks freed in a stream's order go once that stream has got there.
+ * Errors: RTREE_EINVAL (no such device). */
+RTREE_API rtree_status rtree_trim(int device);
 
 /* Description of the last failure on this host thread ("" if none). */
 RTREE_API const char *rtree_last_error(void);

@@ -43,6 +43,9 @@ rtree_status fail(rtree_status st, const char *fmt, ...)
 
 void clear_error() { g_err.clear(); }
 
+static constexpr uint64_t kKeepAll = UINT64_MAX;    // the release threshold given to the default pool
+static constexpr size_t kLarge = (size_t)64 << 20;  // bytes from which a block is large
+
 void setup_device_pool(int dev)
 {
     static std::mutex mu;
@@ -52,7 +55,7 @@ void setup_device_pool(int dev)
         return;
     cudaMemPool_t pool;
     if (cudaDeviceGetDefaultMemPool(&pool, dev) == cudaSuccess) {
-        uint64_t keep = UINT64_MAX;  // keep freed blocks in the pool between calls
+        uint64_t keep = kKeepAll;  // keep freed blocks in the pool between calls
         cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
     }
     cudaGetLastError();
@@ -60,31 +63,65 @@ void setup_device_pool(int dev)
 }
 
 namespace {
-// The pool of large results on the current device (null: the default one).
-// It keeps freed blocks up to a quarter of the device's memory.
+std::mutex g_results_mu;
+cudaMemPool_t g_results[64] = {};
+bool g_results_kept[64] = {};  // their release threshold is a quarter of the memory, else 0
+
+// Whether the caller leaves the current device's default pool to the library:
+// it is the current pool, and its release threshold is the library's.
+bool default_pool_ours(int dev)
+{
+    cudaMemPool_t current = nullptr, pool = nullptr;
+    uint64_t keep = 0;
+    const bool ours = cudaDeviceGetMemPool(&current, dev) == cudaSuccess &&
+                      cudaDeviceGetDefaultMemPool(&pool, dev) == cudaSuccess && current == pool &&
+                      cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) == cudaSuccess &&
+                      keep == kKeepAll;
+    cudaGetLastError();
+    return ours;
+}
+
+// The pool of large results on the current device (null: the current pool).
+// It keeps freed blocks up to a quarter of the device's memory.  A caller who
+// sets a pool of its own, or another release threshold for the default one, has
+// large results from that pool too, and this one then keeps nothing.
 cudaMemPool_t result_pool()
 {
-    static std::mutex mu;
-    static cudaMemPool_t pools[64] = {};
     int dev = 0;
-    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64)
+    if (cudaGetDevice(&dev) != cudaSuccess || dev < 0 || dev >= 64) {
+        cudaGetLastError();
         return nullptr;
-    std::lock_guard<std::mutex> g(mu);
-    if (!pools[dev]) {
+    }
+    const bool ours = default_pool_ours(dev);
+    std::lock_guard<std::mutex> g(g_results_mu);
+    cudaMemPool_t &pool = g_results[dev];
+    if (!pool && ours) {
         cudaMemPoolProps props{};
         props.allocType = cudaMemAllocationTypePinned;
         props.location.type = cudaMemLocationTypeDevice;
         props.location.id = dev;
-        size_t idle = 0, all = 0;
-        cudaMemPool_t pool = nullptr;
-        if (cudaMemGetInfo(&idle, &all) == cudaSuccess && cudaMemPoolCreate(&pool, &props) == cudaSuccess) {
-            uint64_t keep = all / 4;
-            cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
-            pools[dev] = pool;
-        }
-        cudaGetLastError();
+        if (cudaMemPoolCreate(&pool, &props) != cudaSuccess)
+            pool = nullptr;
     }
-    return pools[dev];
+    if (pool && ours != g_results_kept[dev]) {
+        size_t idle = 0, all = 0;
+        if (ours && cudaMemGetInfo(&idle, &all) != cudaSuccess)
+            all = 0;
+        uint64_t keep = all / 4;
+        cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep);
+        if (!ours)
+            cudaMemPoolTrimTo(pool, 0);
+        g_results_kept[dev] = ours;
+    }
+    cudaGetLastError();
+    return ours ? pool : nullptr;
+}
+
+// Gives back what the pool of large results on device dev keeps.
+cudaError_t trim_results(int dev)
+{
+    std::lock_guard<std::mutex> g(g_results_mu);
+    return g_results[dev] ? cudaMemPoolTrimTo(g_results[dev], 0) : cudaSuccess;
 }
 
 // Gives what the pools keep for later calls back to the device, what was freed
@@ -99,8 +136,8 @@ void trim_pools(cudaStream_t s)
         cudaGetDevice(&dev) == cudaSuccess && cudaStreamSynchronize(s) == cudaSuccess) {
         if (cudaDeviceGetDefaultMemPool(&pool, dev) == cudaSuccess)
             cudaMemPoolTrimTo(pool, 0);
-        if ((pool = result_pool()))
-            cudaMemPoolTrimTo(pool, 0);
+        if (dev >= 0 && dev < 64)
+            trim_results(dev);
     }
     cudaGetLastError();
 }
@@ -131,7 +168,7 @@ rtree_status dmalloc(void **p, size_t bytes, cudaStream_t s, const char *what, B
     }
     size_t step = 1;
     cudaMemPool_t pool = nullptr;
-    if (kind != EXACT && bytes >= ((size_t)64 << 20)) {
+    if (kind != EXACT && bytes >= kLarge) {
         while (step <= bytes >> 5)
             step <<= 1;
         if (kind == RESULT)
@@ -314,6 +351,19 @@ extern "C" {
 const char *rtree_last_error(void) { return g_err.c_str(); }
 
 const char *rtree_version(void) { return "rtree-gb300 0.1 (sm_103a)"; }
+
+rtree_status rtree_trim(int device)
+{
+    clear_error();
+    int n = 0, dev = device;
+    RT_CUDA(cudaGetDeviceCount(&n));
+    if (dev < 0)
+        RT_CUDA(cudaGetDevice(&dev));
+    if (dev >= n || dev >= 64)
+        return fail(RTREE_EINVAL, "rtree_trim: no device %d", device);
+    RT_CUDA(trim_results(dev));
+    return RTREE_OK;
+}
 
 // Test hook: make the k-th following device allocation fail (k = -1 disables).
 void rtree_debug_fail_alloc_after(long long k) { g_alloc_countdown.store(k); }

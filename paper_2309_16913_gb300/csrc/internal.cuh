@@ -55,7 +55,7 @@ struct AllocScope {
 // counter can make the k-th allocation fail (fault injection for tests; no
 // GPU fault is involved).
 // Blocks of 64 MB and more that are not EXACT may be up to a sixteenth larger;
-// results come from a pool of their own.
+// such results come from a pool of their own (capi.cu).
 enum Block { EXACT, SCRATCH, RESULT };
 rtree_status dmalloc(void **p, size_t bytes, cudaStream_t s, const char *what, Block kind = EXACT);
 // Keeps freed blocks in the device's default pool between calls (once per device).

@@ -194,6 +194,7 @@ def _bind(lib):
         "rtree_result_free_async": (None, [vp, vp]),
         "rtree_result_wait": (C.c_int, [vp]),
         "rtree_last_error": (C.c_char_p, []),
+        "rtree_trim": (C.c_int, [C.c_int]),
         "rtree_version": (C.c_char_p, []),
         "rtree_debug_fail_alloc_after": (None, [C.c_longlong]),
         "rtree_debug_wq_wait": (None, [C.c_longlong, C.c_int]),
@@ -560,6 +561,13 @@ def rtree_result_wait(res: int) -> None:
 
 def rtree_last_error() -> str:
     return (load_library().rtree_last_error() or b"").decode()
+
+
+def rtree_trim(device: int = -1) -> None:
+    """Gives back to the device what the library's pool of large results keeps
+    (device < 0: of the current one)."""
+    lib = load_library()
+    _check(lib.rtree_trim(int(device)), lib)
 
 
 def rtree_version() -> str:
