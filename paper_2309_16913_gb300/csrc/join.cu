@@ -714,27 +714,33 @@ int top_bit(uint32_t all_or, uint32_t all_and)
     return b;
 }
 
-// Sorts (r, s) pairs lexicographically into `out` (may be `pairs`): stable
-// sort by s, then by r, each on the low bits in which its ids differ.
-rtree_status sort_pairs(const int2 *pairs, int2 *out, int64_t n, int r_bits, int s_bits, cudaStream_t s)
+// Sorts n (r, s) pairs lexicographically: stable sort by s, then by r, each on
+// the low bits in which its ids differ.  `pairs` may have room to spare and is
+// left with exactly n; it is given up in between, so that the sort holds 24
+// bytes a pair at most.
+rtree_status sort_pairs(DevBuf<int2> &pairs, int64_t n, int r_bits, int s_bits, cudaStream_t s)
 {
     if (n <= 0)
-        return RTREE_OK;
+        return pairs.alloc(0, "join pairs");
     DevBuf<uint32_t> k0(s), v0(s), k1(s), v1(s);
     RT_TRY(k0.alloc(n, "join sort"));
     RT_TRY(v0.alloc(n, "join sort"));
-    RT_TRY(k1.alloc(n, "join sort"));
-    RT_TRY(v1.alloc(n, "join sort"));
     {
         KernelTimer kt_("split_pairs", s);
-        k_split_pairs<<<blocks_for(n), 256, 0, s>>>(pairs, n, k0.p, v0.p);
+        k_split_pairs<<<blocks_for(n), 256, 0, s>>>(pairs.p, n, k0.p, v0.p);
         RT_LAUNCH();
     }
+    pairs.reset();
+    RT_TRY(k1.alloc(n, "join sort"));
+    RT_TRY(v1.alloc(n, "join sort"));
     RT_TRY(radix_sort_pairs(k0.p, v0.p, k1.p, v1.p, n, 0, s_bits, s));  // by s; v1 = r keys
     RT_TRY(radix_sort_pairs(v1.p, k1.p, v0.p, k0.p, n, 0, r_bits, s));  // by r; k0 = s keys
+    k1.reset();
+    v1.reset();
+    RT_TRY(pairs.alloc(n, "join pairs"));
     {
         KernelTimer kt_("merge_pairs", s);
-        k_merge_pairs<<<blocks_for(n), 256, 0, s>>>(v0.p, k0.p, n, out);
+        k_merge_pairs<<<blocks_for(n), 256, 0, s>>>(v0.p, k0.p, n, pairs.p);
         RT_LAUNCH();
     }
     return RTREE_OK;
@@ -842,7 +848,7 @@ rtree_status tree_join_queue(const rtree *R, const rtree *S, bool prune, cudaStr
         k_jq_check<<<1, 1, 0, s>>>(counter.p + 1, counter.p, flags.p);
         RT_LAUNCH();
     }
-    RT_TRY(sort_pairs(pairs.p, pairs.p, total, 32, 32, s));
+    RT_TRY(sort_pairs(pairs, total, 32, 32, s));
     // the scatter pass and the sort run on in the order of s; their flags
     // reach the result's status
     RT_TRY(post_result_status(flags.p, s, res));
@@ -851,19 +857,13 @@ rtree_status tree_join_queue(const rtree *R, const rtree *S, bool prune, cudaStr
     return RTREE_OK;
 }
 
-rtree_status tree_join(const rtree *R, const rtree *S, bool prune, cudaStream_t s,
-                       rtree_result *res, int64_t *stats)
+namespace {
+
+// The join by levels of two trees that are not empty.  lean: no buffer is larger
+// than what it is to hold (the levels are then run twice, first to count).
+rtree_status join_levels(const rtree *R, const rtree *S, bool prune, bool lean, cudaStream_t s,
+                         rtree_result *res, int64_t *stats)
 {
-    res->rows = 0;
-    res->total = 0;
-    res->offsets = nullptr;
-    if (R->nodes == 0 || S->nodes == 0) {
-        DevBuf<int32_t> ids(s);
-        RT_TRY(ids.alloc(2, "join pairs"));
-        RT_CUDA(cudaStreamSynchronize(s));
-        res->ids = ids.release();
-        return RTREE_OK;
-    }
     const TreeDev ta = R->view(), tb = S->view();
     // The modes of the levels are fixed by the heights alone.
     int mode[2 * RT_MAX_LEVELS], steps = 0;
@@ -882,8 +882,8 @@ rtree_status tree_join(const rtree *R, const rtree *S, bool prune, cudaStream_t 
     // a level that finds more says how many, and the traversal resumes at
     // that level with a buffer of that size.
     constexpr long long kMostPairs = 16ll << 20;
-    const long long front_cap = std::min<long long>(8ll * (R->nodes + S->nodes) + 65536, kMostPairs);
-    const long long out_cap = std::min<long long>(R->n + S->n + 65536, kMostPairs);
+    const long long front_cap = lean ? 1 : std::min<long long>(8ll * (R->nodes + S->nodes) + 65536, kMostPairs);
+    const long long out_cap = lean ? 1 : std::min<long long>(R->n + S->n + 65536, kMostPairs);
     DevBuf<int2> front[2] = {DevBuf<int2>(s), DevBuf<int2>(s)}, pairs(s);
     long long cap[3] = {front_cap, front_cap, out_cap};  // of front[0], front[1], pairs
     DevBuf<unsigned long long> n(s);
@@ -939,6 +939,8 @@ rtree_status tree_join(const rtree *R, const rtree *S, bool prune, cudaStream_t 
         if (to == 2 && h[full + 1] >= (uint64_t)INT32_MAX)
             break;  // too many results for the sort: reported below
         DevBuf<int2> &buf = to == 2 ? pairs : front[to];
+        if (to == 2)  // the last level needs its input only
+            front[(full + 1) & 1].reset();
         cap[to] = (long long)h[full + 1];
         RT_TRY(buf.alloc(cap[to], to == 2 ? "join pairs" : "join frontier"));
         RT_CUDA(cudaMemsetAsync(n.p + full + 1, 0, (steps - full) * sizeof(unsigned long long), s));
@@ -946,6 +948,7 @@ rtree_status tree_join(const rtree *R, const rtree *S, bool prune, cudaStream_t 
     }
     const int64_t total = (int64_t)h[steps];
     if (stats) {
+        std::fill_n(stats, 5, 0);
         for (int e = 0; e < steps; ++e)
             stats[mode[e]] += (int64_t)h[e];  // node pairs tested in this mode
         stats[4] = total;
@@ -955,13 +958,34 @@ rtree_status tree_join(const rtree *R, const rtree *S, bool prune, cudaStream_t 
                     (long long)total);
     front[0].reset();
     front[1].reset();
-    DevBuf<int2> sorted(s);
-    RT_TRY(sorted.alloc(total, "join pairs"));
-    RT_TRY(sort_pairs(pairs.p, sorted.p, total, top_bit(hbits[0], hbits[1]), top_bit(hbits[2], hbits[3]), s));
+    RT_TRY(sort_pairs(pairs, total, top_bit(hbits[0], hbits[1]), top_bit(hbits[2], hbits[3]), s));
     RT_CUDA(cudaStreamSynchronize(s));
     res->total = total;
-    res->ids = reinterpret_cast<int32_t *>(sorted.release());
+    res->ids = reinterpret_cast<int32_t *>(pairs.release());
     return RTREE_OK;
+}
+
+}  // namespace
+
+rtree_status tree_join(const rtree *R, const rtree *S, bool prune, cudaStream_t s,
+                       rtree_result *res, int64_t *stats)
+{
+    res->rows = 0;
+    res->total = 0;
+    res->offsets = nullptr;
+    if (R->nodes == 0 || S->nodes == 0) {
+        DevBuf<int32_t> ids(s);
+        RT_TRY(ids.alloc(2, "join pairs"));
+        RT_CUDA(cudaStreamSynchronize(s));
+        res->ids = ids.release();
+        return RTREE_OK;
+    }
+    rtree_status st = join_levels(R, S, prune, false, s, res, stats);
+    if (st == RTREE_ENOMEM) {  // once more without the room to spare
+        clear_error();
+        st = join_levels(R, S, prune, true, s, res, stats);
+    }
+    return st;
 }
 
 }  // namespace rt
