@@ -791,17 +791,19 @@ rtree_status str_order(const float4 *boxes, int64_t m, int64_t size, uint32_t *p
     if (m > kLevelMost || cluster_ctas() == 0)
         return str_order_large(boxes, m, (uint32_t)size, bits, pack, s);
     DevBuf<uint32_t> buf(s);
-    RT_TRY(buf.alloc(8 * (size_t)m, "level order"));
-    uint32_t *x = buf.p, *y = x + 4 * m;
+    RT_TRY(buf.alloc(7 * (size_t)m, "level order"));
+    uint32_t *x = buf.p, *y = x + 4 * m, *order_y = y + 2 * m;
     uint32_t *slab = x;  // the last x pass reads x + m and x + 3m
+    // each sort ends in the first of its buffers; pack is one of the y sort's
+    // on the way to order_y, or where it ends
     ClusterSort ax{nullptr, nullptr, boxes, nullptr, {x, x + m}, {x + 2 * m, x + 3 * m}, slab, (uint32_t)size,
                    0, (int)m, 0, 32, 4, 0};
-    ClusterSort ay{nullptr, nullptr, boxes, nullptr, {y, y + m}, {bits ? y + 2 * m : pack, y + 3 * m}, nullptr, 1,
+    ClusterSort ay{nullptr, nullptr, boxes, nullptr, {y, y + m}, {bits ? order_y : pack, bits ? pack : order_y}, nullptr, 1,
                    1, (int)m, 0, 32, 4, 0};
     if (bits == 0)  // one slab: the y order is the packing order
         return launch_cluster<SRC_BOXES>(ay, ay, 1, s);
     RT_TRY(launch_cluster<SRC_BOXES>(ax, ay, 2, s));
-    const ClusterSort as{nullptr, y + 2 * m, nullptr, slab, {y, y + m}, {pack, y + 3 * m}, nullptr, 1,
+    const ClusterSort as{nullptr, order_y, nullptr, slab, {y, y + m}, {pack, x + m}, nullptr, 1,
                          0, (int)m, 0, bits, (bits + 7) / 8, 0};
     return launch_cluster<SRC_TABLE>(as, as, 1, s);
 }
