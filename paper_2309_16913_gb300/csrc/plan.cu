@@ -83,17 +83,19 @@ void free_plan(rtree_plan *p)
     cudaGetLastError();
 }
 
-// Carves the plan's buffers out of one allocation (256-byte aligned pieces).
+// Carves the plan's buffers out of one allocation (256-byte aligned pieces);
+// those of the other mapping are left out.
 rtree_status allocate(rtree_plan *p)
 {
     const int64_t Q = p->max_q, C = p->ids_cap;
     // slots exceed hits: about 2x on large queries, up to F per hit on tiny ones
     const int64_t LC = 2 * C + 4 * (int64_t)p->tree->fanout * Q;
     p->leaf_cap = LC;
-    const long long wq_cap = Q + (Q > (1 << 20) ? Q : (1 << 20));
+    const bool wq = p->mapping == RTREE_MAP_WORK_QUEUE;
+    const long long wq_cap = wq ? Q + (Q > (1 << 20) ? Q : (1 << 20)) : 0;
     // large queries whose traversal is shared out; those past these limits are
     // walked by one warp each
-    const int64_t large_cap = Q < 16384 ? Q : 16384, task_cap = 1 << 18;
+    const int64_t large_cap = wq ? 0 : Q < 16384 ? Q : 16384, task_cap = wq ? 0 : 1 << 18;
     struct Piece {
         void **dst;
         size_t bytes;
@@ -110,11 +112,11 @@ rtree_status allocate(rtree_plan *p)
         {reinterpret_cast<void **>(&b.leaf), (size_t)LC * 4},
         {reinterpret_cast<void **>(&b.rng), (size_t)C * 8},
         {reinterpret_cast<void **>(&b.ids), (size_t)C * 4},
-        {reinterpret_cast<void **>(&b.cursors), (size_t)Q * 8},
+        {reinterpret_cast<void **>(&b.cursors), wq ? (size_t)Q * 8 : 0},
         {reinterpret_cast<void **>(&b.flags), 8},
         {reinterpret_cast<void **>(&b.ctr), 32},
         {reinterpret_cast<void **>(&b.large), (size_t)large_cap * 4},
-        {reinterpret_cast<void **>(&b.large_cur), (size_t)(2 * large_cap + 1) * 8},
+        {reinterpret_cast<void **>(&b.large_cur), wq ? 0 : (size_t)(2 * large_cap + 1) * 8},
         {reinterpret_cast<void **>(&b.tasks), (size_t)task_cap * 8},
         {reinterpret_cast<void **>(&b.wq_ctl), 24},
         {reinterpret_cast<void **>(&b.wq_items), (size_t)wq_cap * 8},
