@@ -422,6 +422,7 @@ struct SelectBuffers {
     unsigned long long *large_cur;  // [2 * large_cap + 1] their cursors, the number of tasks
     unsigned long long *tasks;   // [task_cap]
     int64_t large_cap, task_cap;
+    size_t clear_bytes;          // from flags on: the flags, counters and large queries' cursors
     unsigned long long *wq_ctl;  // 3 words, work-queue mapping
     unsigned long long *wq_items;
     long long wq_cap;

@@ -115,8 +115,8 @@ rtree_status allocate(rtree_plan *p)
         {reinterpret_cast<void **>(&b.cursors), wq ? (size_t)Q * 8 : 0},
         {reinterpret_cast<void **>(&b.flags), 8},
         {reinterpret_cast<void **>(&b.ctr), 32},
-        {reinterpret_cast<void **>(&b.large), (size_t)large_cap * 4},
         {reinterpret_cast<void **>(&b.large_cur), wq ? 0 : (size_t)(2 * large_cap + 1) * 8},
+        {reinterpret_cast<void **>(&b.large), (size_t)large_cap * 4},
         {reinterpret_cast<void **>(&b.tasks), (size_t)task_cap * 8},
         {reinterpret_cast<void **>(&b.wq_ctl), 24},
         {reinterpret_cast<void **>(&b.wq_items), (size_t)wq_cap * 8},
@@ -143,6 +143,7 @@ rtree_status allocate(rtree_plan *p)
         *pc.dst = at;
         at += (pc.bytes + 255) & ~(size_t)255;
     }
+    b.clear_bytes = reinterpret_cast<char *>(b.large) - reinterpret_cast<char *>(b.flags);
     b.rng_cap = b.ids_cap = C;
     b.leaf_cap = LC;
     b.large_cap = large_cap;

@@ -1169,7 +1169,7 @@ LargeKernel pick_large(int F, int layout)
 
 // The descriptors of the listed large queries (at most n_large of them and
 // n_tasks tasks).  io: as for DESC; lg: as filled by BOUND; cur: 2 * n_large +
-// 1 words for the cursors, which it sets in lg and zeroes here.
+// 1 words for the cursors, cleared, which it sets in lg.
 rtree_status launch_large(const rtree *t, const float4 *q, const SelIO &io, LargeIO &lg, int64_t n_large,
                           int64_t n_tasks, unsigned long long *tasks, unsigned long long *cur, int32_t *flags,
                           cudaStream_t s)
@@ -1195,7 +1195,6 @@ rtree_status launch_large(const rtree *t, const float4 *q, const SelIO &io, Larg
         const int64_t b = (items + kWarps - 1) / kWarps;
         return (unsigned)(b < 1 ? 1 : b < full ? b : full);
     };
-    RT_CUDA(cudaMemsetAsync(cur, 0, (2 * n_large + 1) * sizeof(unsigned long long), s));
     {
         KernelTimer kt_("select_large_expand", s);
         k_large_expand<<<grid(n_large), kThreads, smem, s>>>(t->view(), q, io, lg, flags, cap);
@@ -1321,6 +1320,7 @@ rtree_status range_select_bounded(const rtree *t, const float4 *queries, int64_t
     if (n_large > 0 && h[0] < lg.budget) {
         RT_TRY(tasks.alloc(n_tasks, "select tasks"));
         RT_TRY(large_cur.alloc(2 * n_large + 1, "select cursors"));
+        RT_CUDA(cudaMemsetAsync(large_cur.p, 0, (2 * n_large + 1) * sizeof(unsigned long long), s));
         RT_TRY(launch_large(t, queries, so, lg, n_large, n_tasks, tasks.p, large_cur.p, flags, s));
         pass = PASS_DESC_LARGE;
     }
@@ -1794,8 +1794,9 @@ rtree_status select_enqueue(const rtree *t, const float4 *queries, int64_t Q, in
     // (a graph cannot ask whether there are large queries, only prepare for them)
     const bool share_large = !wq && Q <= kSharedQueries;
     LargeIO lg{};
-    RT_CUDA(cudaMemsetAsync(b.flags, 0, 2 * sizeof(int32_t), s));
-    RT_CUDA(cudaMemsetAsync(b.ctr, 0, 4 * sizeof(unsigned long long), s));
+    // one node for all that starts at zero: the large queries' kernels, which a
+    // small batch runs for nothing, are two more in the chain
+    RT_CUDA(cudaMemsetAsync(b.flags, 0, b.clear_bytes, s));
     if (Q == 0 || t->nodes == 0) {
         RT_CUDA(cudaMemsetAsync(b.off, 0, (Q + 1) * sizeof(int64_t), s));
         RT_CUDA(cudaMemsetAsync(b.off_leaf, 0, (Q + 1) * sizeof(int64_t), s));
