@@ -146,7 +146,7 @@ __global__ void k_sort_children(const float4 *__restrict__ items, uint32_t *__re
 // path:
 //   (x centre key, item)  -> slab = rank / (S*F),
 //   (slab, y centre key, item) -> the packing order.
-constexpr int kSmallLevel = 1024;  // item indices fit 12 bits
+constexpr int kSmallLevel = 1024;  // (item indices fit the 12 low bits of the keys)
 
 struct SmallLevels {
     int count;                      // levels to build, bottom up

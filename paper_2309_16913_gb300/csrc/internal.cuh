@@ -451,7 +451,7 @@ struct SortSources {
 };
 
 // Writes segment i's ids, sorted ascending (signed), to
-// out[off[i] .. off[i+1]).  out may be the leaf array itself (in place).
+// out[off[i] .. off[i+1]).
 // Enqueues work only (no host synchronization); `total` must bound the sum
 // of the segments' lengths (it sizes the scratch), and segments ending past
 // out_cap (default: total) in `out` are skipped.  Offsets may be absolute
@@ -463,10 +463,6 @@ constexpr int kSortWhole = 32256;  // ids that one CTA sorts; longer segments ar
 rtree_status segmented_sort_gather(int32_t *out, const int64_t *off, int64_t nseg, int64_t total,
                                    const SortSources &src, cudaStream_t s, int32_t *flags,
                                    int64_t out_cap = -1, int64_t max_len = INT64_MAX, int64_t long_ids = -1);
-
-// Sorts every segment ids[offsets[i] .. offsets[i+1]) ascending, in place.
-rtree_status segmented_sort(int32_t *ids, const int64_t *offsets, int64_t nseg, int64_t total,
-                            cudaStream_t s);
 
 // Builds the tree from device rectangles (float4 rows) and device ids (or
 // NULL); sort_children orders every node's entries by ascending lx.

@@ -1695,16 +1695,4 @@ rtree_status segmented_sort_gather(int32_t *out, const int64_t *offsets, int64_t
     return launch_lsd(cr1, max_len, out, s);
 }
 
-rtree_status segmented_sort(int32_t *ids, const int64_t *offsets, int64_t nseg, int64_t total,
-                            cudaStream_t s)
-{
-    SortSources S{};
-    S.leaf = ids;
-    S.off_leaf = offsets;
-    DevBuf<int32_t> flags(s);
-    RT_TRY(flags.alloc(1, "sort flags"));
-    RT_CUDA(cudaMemsetAsync(flags.p, 0, sizeof(int32_t), s));
-    return segmented_sort_gather(ids, offsets, nseg, total, S, s, flags.p);
-}
-
 }  // namespace rt

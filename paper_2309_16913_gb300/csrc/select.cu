@@ -1380,6 +1380,7 @@ rtree_status range_select(const rtree *t, const float4 *queries, int64_t Q, bool
         return fail(RTREE_EINVAL, "unsupported fanout %d", t->fanout);
     if (sorted && !wq)
         return range_select_bounded(t, queries, Q, order, s, res, off);
+    // from here on: unsorted, or sorted by the work queue
 
     DevBuf<int32_t> cnt(s), cnt_leaf(s), cnt_rng(s), flags(s);
     DevBuf<unsigned long long> ctr(s);
@@ -1483,14 +1484,10 @@ rtree_status range_select(const rtree *t, const float4 *queries, int64_t Q, bool
         so.leaf_out = leaf.p;
         so.rng_out = rng.p;
         so.order = perm.p;
-        if (wq) {
-            so.offsets = off.p;
-            so.cur_leaf = cursors.p;
-            so.cur_rng = cursors.p + Q;
-            RT_TRY(launch_wq(PASS_DESC, t, queries, Q, so, flags.p, s));
-        } else {
-            RT_TRY(launch(PASS_DESC, t, queries, Q, so, ctr.p + 1, flags.p, s));
-        }
+        so.offsets = off.p;
+        so.cur_leaf = cursors.p;
+        so.cur_rng = cursors.p + Q;
+        RT_TRY(launch_wq(PASS_DESC, t, queries, Q, so, flags.p, s));
         SortSources src{};
         src.leaf = leaf.p;
         src.off_leaf = off_leaf.p;
