@@ -146,7 +146,7 @@ void trim_pools(cudaStream_t s)
 // Where no free block of a pool is large enough, the pool maps one together, at
 // a cost that grows with its size, and a caller that drops a result after the
 // next call makes large blocks of scratch and of results change places.  Three
-// batches of 1M queries on 11M rectangles in turn, 1.4G ids each, took 12.9 to
+// batches of 1M queries on 10M rectangles in turn, 1.4G ids each, took 12.9 to
 // 16.3 ms a call, one of them alone 11.0.  With sizes in steps and results apart
 // both take 11.0.
 rtree_status dmalloc(void **p, size_t bytes, cudaStream_t s, const char *what, Block kind)

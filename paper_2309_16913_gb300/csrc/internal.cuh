@@ -173,8 +173,9 @@ void timing_add_replay(const char *name, long long launches);
 struct Mailbox;
 
 // From this fanout on each whole subtree is a run of its own: a leaf has ids
-// enough for one copy, and what merging them adds to the descriptor pass made
-// it slower (172 -> 189 us at F=128, 100K queries of 0.01% on 2M).
+// enough for one copy, and what merging them adds to the descriptor pass makes
+// it slower (F = 128, 100K queries of 1e-6 to 1e-3 on 2M: 164 -> 181 us AoS, 171
+// -> 186 LOHI, 174 -> 191 SoA).
 constexpr int kRunSingly = 128;
 
 struct TreeDev {

@@ -143,7 +143,7 @@ __global__ void __launch_bounds__(kThreads) k_tile_scan(const __grid_constant__ 
 
 // Arrays of one tile, one after another by one CTA, and then the words of l:
 // a small call waits for the chain of its launches, and this is one for up to
-// four (one query on 2M rectangles: 165 -> 153 us).
+// four (one query on 1M rectangles: 165 -> 153 us).
 __global__ void __launch_bounds__(kThreads) k_scan_post(const __grid_constant__ ScanJobs j, int n,
                                                         const __grid_constant__ PostList l, uint32_t *__restrict__ dst)
 {

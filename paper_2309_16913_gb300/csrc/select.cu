@@ -58,14 +58,26 @@ constexpr int kThreads = kWarps * 32;
 enum { PASS_COUNT = 0, PASS_SCATTER = 1, PASS_DESC = 2, PASS_BOUND = 3, PASS_DESC_LARGE = 4 };
 enum { FLAG_STACK = 1, FLAG_COUNT_MISMATCH = 2, FLAG_TIMEOUT = 4 };
 // Leaves to visit from which a query is large, in batches that leave warps
-// without a query and in larger ones (see k_large_desc).
+// without a query and in larger ones (see k_large_desc).  Whole calls on 10M
+// rectangles (F = 64) in us, with lines of 8 / 32 / 64 / 160 / 400 leaves:
+//   48 windows                              330 /  329 /  326 /  448 /  594
+//   8,000 queries, 1% of them windows       417 /  425 /  423 /  526 /  701
+//   8,000 queries of 1e-5 to 1e-2          1344 / 1347 / 1365 / 1416 / 1541
+//   60,000 queries, 1% of them windows     1330 / 1335 / 1353 / 1433 / 1601
+//   100,000 queries of 1e-6 to 1e-3        1641 / 1481 / 1439 / 1464 / 1473
+//   the last at F = 16                     2242 / 1761 / 1694 / 1671 / 1767
+// A batch of few queries wants a low line.  With 100,000 a low one lists too
+// many; between 8,000 and 60,000 the higher line is early.
 constexpr int kLargeFew = 32, kLargeMany = 160;
 constexpr int64_t kFewQueries = 8192;
 constexpr int64_t kSharedQueries = 1 << 18;  // captured batches up to this size are prepared for large queries
 inline int large_leaves(int64_t Q) { return Q < kFewQueries ? kLargeFew : kLargeMany; }
 // A batch with more leaves to visit than this keeps every warp busy past the
-// walk of a large query: sharing those out would only cost (2% of a million
-// queries' select).
+// walk of a large query: sharing those out gains nothing any more.  Whole calls
+// on 10M rectangles (F = 64, queries of 1e-5 to 1e-2) in us, never / by this rule
+// / always shared out: 2,500 queries 831 / 628 / 629, 10,000 1829 / 1699 / 1695,
+// 20,000 (about here) 3030 / 2927 / 2942, 40,000 5600 / 5581 / 5507; a million of
+// 1e-6 to 1e-3 11326 / 11328 / 11390.
 inline int64_t large_budget(int F) { return (int64_t)F * kLargeMany * sm_count() * 48; }
 __device__ __forceinline__ bool treat_large(const LargeIO &lg)
 {
@@ -151,9 +163,9 @@ __device__ __forceinline__ int64_t reserve(int32_t *cursor, int n, int lane)
 // Whole subtrees are taken a run at a time: neighbouring children's subtrees
 // follow one another in the id array, so the run's first lane stands for it.
 // mc: the lanes with a whole subtree.  A window holds leaves side by side, so
-// runs are several times fewer than subtrees: 1M queries on 11M sort in
+// runs are several times fewer than subtrees: 1M queries on 10M sort in
 // 7.48 ms instead of 7.65 with fewer entries to read, and the unsorted copies of
-// 100K queries on 2M (F=16) take 561 us instead of 680, being longer.
+// 200K queries on 3M (F=32) take 561 us instead of 680, being longer.
 template <int F>
 __device__ __forceinline__ unsigned run_starts(const TreeDev &t, unsigned mc)
 {
@@ -463,11 +475,17 @@ __device__ __forceinline__ void flush_stats(unsigned long long *stats, const Wal
 
 // CTAs per SM the warp-per-query kernel is compiled for.  The descriptor
 // pass's walk is bound by the latency of dependent node loads, so it takes the
-// warps that the registers allow with at most a few spilled: left to the
-// compiler (51 registers, five CTAs) F=16 took 209 us instead of 188, F=32 in
-// the LOHI layout 220 instead of 188 (100K queries of 0.01% on 2M), F=64 2585
-// instead of 2530 (1M queries on 11M); at F=128 the five and six CTAs that
-// need fewer than 64 registers took 185 and 196 us instead of 172.
+// warps that the registers allow with at most a few spilled.  100K queries of
+// 1e-6 to 1e-3 on 2M, in us, compiled for 4 / 5 / 6 / 7 (SoA, AoS, LOHI):
+//   F = 4    232 / 221 / 213 / 228   259 / 252 / 250 / 264   232 / 236 / 231 / 241
+//   F = 8    213 / 203 / 196 / 208   208 / 197 / 192 / 206   186 / 189 / 184 / 195
+//   F = 16   216 / 205 / 199 / 208   226 / 216 / 208 / 218   196 / 200 / 192 / 200
+//   F = 32   207 / 214 / 213 / 209   201 / 208 / 202 / 199   204 / 204 / 195 / 197
+//   F = 64   167 / 168 / 182 / 184   170 / 170 / 180 / 178   181 / 182 / 191 / 190
+//   F = 128  174 / 188 / 195 / 284   164 / 177 / 186 / 229   171 / 183 / 193 / 255
+// F = 32 gains from seven on fewer, larger queries (20K of 1e-5 to 1e-2: 146 to
+// 157 us against 167 to 173 for four), F = 64 on a million queries on 10M (2530
+// us against 2585 for six).
 constexpr int select_min_blocks(int F, int pass)
 {
     return pass != PASS_DESC ? 1 : (F >= 128 ? 4 : (F >= 32 ? 7 : 6));
@@ -815,9 +833,8 @@ __global__ void k_wq_places(const SelIO io, int64_t Q, int32_t *__restrict__ fla
 // 48 windows of 1.6% of 10M rectangles each (F = 64): 484 us in the descriptor
 // pass before, 60 us in these kernels; a plan batch with 800 such windows
 // among 100K queries 2.25 -> 1.93 ms; 1000 queries of up to 30K ids 141 -> 92 us.
-// The lines: 32 leaves is where a walk of its own (a microsecond a leaf) takes
-// as long as two kernels more; batches that fill the warps several times over
-// gain from about 160 on.
+// The lines (kLargeFew, kLargeMany): a walk of 32 leaves of its own, at a
+// microsecond a leaf, takes as long as these two kernels' launches.
 // The runs [lo, lo + len) of the lanes of mc go to query `slot`.
 template <int F>
 __device__ __forceinline__ void large_runs(const TreeDev &t, const SelIO &io, const LargeIO &lg, const Seg &sg, int64_t slot, unsigned mc, int lo, int len,
