@@ -251,8 +251,9 @@ def algorithmic_bytes(stats, F, Q, seg_sizes):
     traversal counters and the per-query result sizes.
 
     Node visit: F entry MBRs (16 B each, unused slots included) + 16 B of node
-    metadata.  Whole subtree: 16 B metadata read + 8 B (lo, hi) written.  Leaf
-    hit: 4 B id read + 4 B written.  Sorting an id: 4 B gathered + 4 B written
+    metadata.  Whole subtree: 16 B metadata read, and an 8 B entry written at
+    F >= 128 (below, neighbouring subtrees share one; theirs, a few per query,
+    are left out).  Leaf hit: 4 B id read + 4 B written.  Sorting an id: 4 B gathered + 4 B written
     (segments over 32256 ids are first gathered and scattered into buckets,
     which adds two reads and two writes).
     The bound pass visits the internal nodes only; the descriptor pass after
@@ -271,7 +272,7 @@ def algorithmic_bytes(stats, F, Q, seg_sizes):
     return {
         "select_count": float(traverse + Q * (16 + 3 * 4)),
         "select_bound": float(internal + Q * (16 + 3 * 4)),
-        "select_desc": float(traverse + Q * (16 + 32 + 8) + leaf_hits * 8 + whole * 8),
+        "select_desc": float(traverse + Q * (16 + 32 + 8) + leaf_hits * 8 + (whole * 8 if F >= 128 else 0)),
         "select_scatter": float(traverse + Q * (16 + 16) + hits * 8),
         "sort_warp": float(warp_ids * 8),
         "sort_cta": float(cta_ids * 8),
@@ -311,7 +312,7 @@ def join_roofline(st, Fr, Fs, kern, hbm, peak_kind, clk):
            "frac": round(achieved / hbm, 4), "peak_kind": peak_kind, "ms_per_step": round(ms, 4),
            "algorithmic_bytes_per_step": int(algo), "node_pairs": int(visited),
            "predicate_tests_per_s": round(tests / (ms / 1e3), 1)}
-    issue = issue_fraction([n for n in names], visited, ms, clk, fanout=Fr)
+    issue = issue_fraction([n for n in names if n != "join_init"], visited, ms, clk, fanout=Fr)
     if issue:
         out["issue"] = issue
     return out
@@ -541,7 +542,8 @@ def run_ours(args):
         roofline["note"] = ("sort_all = the whole segmented sort (warp, CTA and long-segment classes on side "
                             "streams), wall time of its span; 8 B per id (gathered + written), 16 B more per id of "
                             "segments over 32256; bound by shared-memory work and per-segment latency, not by HBM "
-                            "(ncu: 45-53% issue active, a few % of DRAM peak)")
+                            "(ncu on the profile case: 44-63% of the issue slots, 42-51% of the shared-memory "
+                            "wavefronts, 13% of the DRAM peak)")
     # the node-test kernels, each against HBM (ncu DRAM bytes) and issue slots
     roofline_node_test = node_test_roofline(kern, algo, stats, args.steps, hbm, peak_kind, clk, F, layout)
 
