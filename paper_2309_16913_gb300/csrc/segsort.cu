@@ -569,9 +569,10 @@ __device__ __forceinline__ void zero_counters(CtaSmem<THREADS, ITEMS> &sm, int n
 // where a larger one lies (win) the write-out counts inversions instead: an
 // id at p belongs at p + (later ids smaller than it) - (earlier ids larger).
 //
-// Bound by shared memory and by instruction issue together (22 wavefronts and
-// 95-115 warp instructions per 32 ids, half of the peak of either; the random
-// atomics, loads and stores of the count and the scatter are ten of the 22).
+// Bound by shared memory and by instruction issue together, in phases that
+// barriers separate (22 to 24 wavefronts and 94 to 118 warp instructions per 32
+// ids, 27 and 130 in the smallest class: about half of the peak of either; the
+// random atomics, loads and stores of the count and the scatter are ten of the 22).
 // All classes on 1.43G ids (10M rectangles, 1M queries): 7.65 ms, against
 // 10.4 ms with buckets of three to five ids sorted by per-thread bitonic
 // networks, a third of whose instructions were the networks' padding.
